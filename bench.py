@@ -81,18 +81,14 @@ SERVE = {"workload": "serve2d_poisson_arrivals", "seed": 4, "n_ops": 6, "depths"
          "kinds": ["dtn", "iti"], "rebuild_frac": 0.2, "requests": 60, "rates": [0.5, 0.9, 1.5],
          "pool": 3, "max_batch": 8, "n_streams": 4, "op_budget_gb": 150}
 
-# bf16 digit products per FP64 multiply-add in the tensor-core products
-# (ten 6-bit digits per operand, the pairs of digit indices summing to <= 11)
-TC_DIGIT_PRODUCTS = 55
+# fp16 digit products per FP64 multiply-add in the tensor-core products (eight
+# 8-bit digits per operand, the pairs of digit indices summing to <= 9); fp16
+# runs at the bf16 rate
+TC_DIGIT_PRODUCTS = 36
 # DRAM bytes (read + write) per launch of a kernel class, averaged over every
 # launch of one build, from an ncu capture of the same workload (summaries
 # under profiles/); None where no capture of the current kernels exists
-NCU_TRAFFIC = {
-    ("helmholtz2d_iti_c128_depth6_p16", "gemm_tc"): {
-        "bytes_per_launch": 182930000,
-        "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over the 581 k_gemm_tc launches of one "
-                  "build (106.3 GB), profiles/k_gemm_tc_traffic_helmholtz2d_depth6.md"},
-}
+NCU_TRAFFIC = {}
 
 COMMON = {"seed_solve_source": 11, "root_map": False, "step": "hps_build + hps_solve(new f) + hps_free",
           "l2": "no flush: the step's factor working set is far above the 129 MB L2"}
@@ -397,9 +393,9 @@ def run_ours(args, rank, world):
     ach = classes[dom]["flops"] / sec / 1e12 if sec > 0 else 0.0
     ach_exec = classes[dom]["exec_flops"] / sec / 1e12 if sec > 0 else 0.0
     if dom == "gemm_tc":
-        # digit-slice products on the bf16 tensor cores: algorithmic FP64
+        # digit-slice products on the 16-bit tensor cores: algorithmic FP64
         # flops against the scheme's ceiling, the measured sustained cuBLAS
-        # bf16 rate (the kernel runs inside a long build) over the 55 bf16
+        # bf16 rate (the kernel runs inside a long build) over the 36 fp16
         # digit products each FP64 multiply-add takes; the executed bf16
         # rate (padded tiles) beside it
         bf16, src = tensor_peak()
@@ -410,7 +406,7 @@ def run_ours(args, rank, world):
                     "unit": "TFLOP/s", "frac": round(ach / ceil, 4),
                     "traffic": traffic["bytes_per_launch"] if traffic else None,
                     "flops_counted": "algorithmic FP64 flops of the products (real multiply-add 2, complex 8)",
-                    "peak_source": f"{src}, divided by {TC_DIGIT_PRODUCTS} bf16 digit products per FP64 "
+                    "peak_source": f"{src}, divided by {TC_DIGIT_PRODUCTS} fp16 digit products per FP64 "
                                    "multiply-add (the digit-slice scheme's ceiling)",
                     "traffic_source": traffic["source"] if traffic else None,
                     "executed_bf16_tflops": round(ach_exec, 4), "executed_bf16_frac": round(ach_exec / bf16, 4),

@@ -144,10 +144,10 @@ typedef struct {
                            problem is far from resonance: max c <= min a * pi^2 /
                            (2 h^2) and max |b| h <= min a, h the leaf side. */
   int fp64_gemm;        /* 0: hps_build runs its large real and complex products
-                           on the tensor cores as exact bf16 digit-slice
-                           products (FP64 accuracy: operands cut into ten 6-bit
-                           digits, the 55 digit products of weight above 2^-66
-                           accumulated exactly and recombined in 64-bit
+                           on the tensor cores as exact fp16 digit-slice
+                           products (FP64 accuracy: operands cut into eight 8-bit
+                           digits, the 36 digit products of weight 2^-68 and
+                           above accumulated exactly and recombined in 64-bit
                            integers; it needs a transient device
                            workspace of up to about 1 GB, and a product whose
                            workspace cannot be allocated runs on the FP64
@@ -181,7 +181,7 @@ enum {
   HPS_KCLASS_DOWN = 6,        /* downward-pass and leaf-output products              */
   HPS_KCLASS_OTHER = 7,       /* fills and copies                                    */
   HPS_KCLASS_GEMM_TC = 8,     /* FP64 / complex GEMM on the tensor cores (digit slices) */
-  HPS_KCLASS_SPLIT = 9,       /* cutting GEMM operands into bf16 digit slices        */
+  HPS_KCLASS_SPLIT = 9,       /* cutting GEMM operands into fp16 digit slices        */
   HPS_KCLASS_COUNT = 10
 };
 
@@ -192,9 +192,9 @@ typedef struct {
   double exec_flops; /* flops the executing pipe performs: the FP64 pipe's equal
                         flops except for the complex GEMM, which takes 3 real
                         products per complex multiply-add (Gauss / 3M form: 6
-                        flops instead of 8); for HPS_KCLASS_GEMM_TC the bf16
+                        flops instead of 8); for HPS_KCLASS_GEMM_TC the fp16
                         tensor-core flops of the digit products over the padded
-                        128 x 48 x 16 tiles (55 products per real product)    */
+                        128 x 64 (or 32) x 16 tiles (36 per real product)     */
 } hps_kernel_stat;
 
 typedef struct hps_handle hps_handle;
@@ -312,9 +312,9 @@ void hps_free(hps_handle* h);
  * B + b*strideB (k x n, ldb), C item b at C + b*strideC (m x n, ldc); strides
  * and leading dimensions in elements.  dtype HPS_F64 (double) or HPS_C128
  * (interleaved complex; alpha and beta are real).  mode 0: the tensor-core
- * digit-slice product that hps_build uses (operands cut into ten 6-bit bf16
- * digits per row of A / column of B, the 55 digit products whose digit
- * indices sum to at most 11 accumulated exactly in fp32, recombined in
+ * digit-slice product that hps_build uses (operands cut into eight 8-bit fp16
+ * digits per row of A / column of B, the 36 digit products whose digit
+ * indices sum to at most 9 accumulated exactly in fp32, recombined in
  * 64-bit integers; for complex data the real and imaginary parts of a row /
  * column share one scale and each component of C is one accumulation of two
  * real products; a transient device workspace of up to about 1 GB); mode 1:

@@ -1,42 +1,47 @@
 // FP64 and complex128 GEMMs on the tcgen05 tensor cores by exact digit
-// slicing (an Ozaki-type splitting of each operand into bf16 digit matrices).
+// slicing (an Ozaki-type splitting of each operand into fp16 digit matrices).
 //
-// Why: the FP64 FMA pipe of this GPU does 4 flop/clk/SM, while the bf16
+// Why: the FP64 FMA pipe of this GPU does 4 flop/clk/SM, while the 16-bit
 // tensor cores do ~7000.  A real product C = A B is computed as
 //
-//   A(i, k) ~ 2^{e_i} sum_p a_p(i, k) 2^{-6p},   B(k, j) ~ 2^{f_j} sum_q b_q(k, j) 2^{-6q},
+//   A(i, k) ~ 2^{e_i} sum_p a_p(i, k) 2^{2-8p},   B(k, j) ~ 2^{f_j} sum_q b_q(k, j) 2^{2-8q},
 //
-// p, q = 1..10, where 2^{e_i} (2^{f_j}) is the power of two above the
-// largest |A(i, :)| (|B(:, j)|) and the digits are the balanced base-64
-// digits of the scaled value rounded to 60 fraction bits: the leading digit
-// in [-64, 64], the others in [-32, 31].  Integers of that size are exact in
-// bf16, their products are exact in the fp32 accumulators of tcgen05.mma, and
-// so are sums of up to 2^22 / 12288 of the products that share one
-// anti-diagonal d = p + q (weight 2^{-6d}).  The product keeps the pairs with
-// p + q <= 11 and accumulates each diagonal exactly in its own TMEM
-// accumulator over K chunks of up to 256.  The epilogue converts the ten
-// diagonal sums to integers, adds them in a 64-bit fixed-point integer (the
-// low diagonals first at full precision, then rounded once) and scales by
-// 2^{e_i + f_j} into FP64.  Errors: operand rounding 2^{-61} 2^{e_i} per
-// entry (unbiased), dropped pairs about 2^{-59} K 2^{e_i + f_j}, half a unit
-// of the fixed point (2^{-lsb}, lsb = 62 - ceil(log2 K)) per chunk, and the
+// p, q = 1..8, where 2^{e_i} (2^{f_j}) is the power of two above the
+// largest |A(i, :)| (|B(:, j)|) and the digits are the balanced base-256
+// digits of the scaled value rounded to 62 fraction bits: the leading digit
+// in [-64, 64], the others in [-128, 127].  Integers of that size are exact in
+// fp16, their products are exact in the fp32 accumulators of tcgen05.mma, and
+// so are sums below 2^24 of the products that share one anti-diagonal
+// D = p + q (weight 2^{4-8D}).  The product keeps the 36 pairs with p + q <= 9
+// and accumulates each diagonal exactly in its own TMEM accumulator over K
+// chunks of up to 128.  The epilogue reduces the eight diagonal sums to one
+// 64-bit fixed-point integer (exact down to 2^-57 or 2^-56, what lies below
+// rounded once) and scales it by 2^{e_i + f_j} into FP64.  Errors: operand
+// rounding 2^{-63} 2^{e_i} per entry (unbiased), dropped pairs at most
+// 2^{-59} K 2^{e_i + f_j}, half a unit of the fixed point per chunk, and the
 // final rounding to FP64: at or below FP64's own rounding error for a dot
 // product of length K when rows and columns are not far from their largest
 // entries.
 //
+// Why 8-bit digits: ten 6-bit digits (the earlier form) take 55 tensor-core
+// products and ten accumulators per output, allow chunks of 256, and write 20
+// digit bytes per entry; eight 8-bit digits take 36 products, eight
+// accumulators and 16 bytes.  Wider digits would need chunks below 36.
+//
 // Layout: the slicing kernel writes each operand's digits, K-major, in the
 // tensor core's canonical no-swizzle layout (8-row x 16-byte core matrices;
 // a 16-deep k step of a 128-row A tile is one 4 KB block per digit, of a
-// 48-column B tile one 1.5 KB block), so that one k step of all digits is one
-// contiguous bulk copy (cp.async.bulk) per operand.  The GEMM kernel computes
-// 128 x 48 output tiles, one CTA per SM walking the launch's tiles: a
-// producer warp streams the digit blocks through a 3-stage shared-memory
-// ring, one thread issues the products as 15 MMAs per k step (digits of B
-// stacked along N, up to 5 per MMA, land in adjacent diagonal accumulators),
-// ten TMEM accumulators take 480 of the 512 columns, and eight epilogue
-// warps (two per TMEM lane quarter, one per half of the columns) read them
-// back while the next tile's copies and products proceed.  A product with
-// few rows may run transposed (C^T = B^T A^T, C's rows on the 48-wide side).
+// TN-column B tile one block of 32 TN bytes), so that one k step of all
+// digits is one contiguous bulk copy (cp.async.bulk) per operand.  The GEMM
+// kernel computes 128 x TN output tiles (TN = 64 or 32), one CTA per SM
+// walking the launch's tiles: a producer warp streams the digit blocks through
+// a shared-memory ring, one thread issues the products (digits of B stacked
+// along N, up to 256 rows per MMA, land in adjacent diagonal accumulators),
+// the eight TMEM accumulators take 512 columns (TN = 64) or 256 (TN = 32, two
+// sets, so that the next chunk's products overlap the read-back), and sixteen
+// epilogue warps (four per TMEM lane quarter, one per quarter of the columns)
+// read them back while the next tile's copies and products proceed.  A product
+// with few rows may run transposed (C^T = B^T A^T, C's rows on the TN side).
 //
 // Complex products are two launches, one per component of C, each
 // accumulating two real products in the same TMEM accumulators
@@ -48,46 +53,52 @@
 #include "devmem.h"
 #include "linalg.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
-#include <mutex>
+#include <cmath>
 #include <type_traits>
 
 namespace hps {
 namespace tc {
 
-constexpr int DIG = 10;             // digits per operand
-constexpr int BITS = 6;             // bits per digit
-constexpr int FRAC = DIG * BITS;    // fraction bits of the scaled operands
-constexpr int DSUM = 11;            // keep digit pairs with p + q <= DSUM (1-based)
-constexpr int NDIAG = DSUM - 1;     // accumulators: d = 2 .. DSUM
-constexpr int TM = 128, TN = 48, TK = 16;
-constexpr int KC = 256;             // k per exact fp32 accumulation chunk
-constexpr int KCT = KC / TK;        // k steps per chunk
+constexpr int DIG = 8;              // digits per operand
+constexpr int BITS = 8;             // bits per digit
+constexpr int FRAC = 62;            // fraction bits of the scaled operands (leading digit in [-64, 64])
+constexpr int DSUM = 9;             // keep digit pairs with p + q <= DSUM (1-based)
+constexpr int NDIAG = DSUM - 1;     // accumulators: D = 2 .. DSUM
+constexpr int TM = 128, TK = 16;
+constexpr int KC1 = 64;             // summed products a single-chunk tile may hold (KC = 64)
+constexpr int KC2 = 128;            // k per exact fp32 accumulation chunk (KC = 128)
 constexpr int ABLK = TM * TK * 2;   // bytes of one digit of an A tile k step
-constexpr int BBLK = TN * TK * 2;
 constexpr int ASTG = DIG * ABLK;
-constexpr int BSTG = DIG * BBLK;
-constexpr int STAGE = ASTG + BSTG;
-constexpr int QGRP = 5;             // B digits stacked into one MMA (N = 5 * 48 = 240 <= 256)
-constexpr int NST = 3;
-constexpr int TMP = TM + 1;          // C staging row stride (odd: transposed reads spread over banks)
-constexpr int CSTG = TN * TMP * 8;    // the C tile staged for the epilogue (column-major)
-constexpr int SMEM = NST * STAGE + CSTG;
-constexpr int TMEM_COLS = 512;
-constexpr int EPI_WARPS = 8;        // two per TMEM lane quarter, each half of the tile's columns
-constexpr int ECOLS = TN / 2;       // columns per epilogue thread
+constexpr int bblk(int tn) { return tn * TK * 2; }   // of a B tile
+constexpr int bstg(int tn) { return DIG * bblk(tn); }
+constexpr int EPI_WARPS = 16;       // four per TMEM lane quarter, each a quarter of the tile's columns
 constexpr int THREADS = 32 * EPI_WARPS + 64;   // + producer warp + MMA-issue warp
 constexpr long SPIN = 1L << 22;     // polls before a wait gives up
+constexpr int LSB1 = 57, LSB2 = 56; // fixed-point fraction bits of a KC = 64 tile, of a KC = 128 chunk
 
-static_assert(NDIAG * TN <= TMEM_COLS, "accumulators exceed TMEM");
-static_assert(ECOLS % 4 == 0, "epilogue column groups of 4");
-static_assert(NDIAG == 10 && DSUM == 11 && BITS == 6, "the epilogue pairs diagonals 2..11 into H (2..7) and L (8..11)");
-// largest |sum of the digit products on one diagonal| per k: the two pairs
-// with a leading digit (64 * 32 each) and the others (32 * 32), or 64 * 64
-// (below 2^22 the epilogue converts them to integers with one fp32 add)
-static_assert((long)KC * (2 * 64 * 32 + (DIG - 2) * 32 * 32) < (1L << 22), "diagonal sums must stay exact in fp32");
-static_assert((long)KC * 64 * 64 < (1L << 22), "diagonal sums must stay exact in fp32");
-static_assert(SMEM <= 227 * 1024, "shared memory ring too large");
+// Shared memory: the copy ring; transposed tiles' staging (one block of
+// 32 x TN / 4 results per epilogue warp, odd stride); at TN = 32 two tiles of
+// old C values, copied a tile ahead.
+constexpr int stages(int tn, bool trans) { return trans ? 3 : 4; }
+constexpr int stage_bytes(int tn) { return ASTG + bstg(tn); }
+constexpr int trans_bytes(int tn, bool trans) { return trans ? EPI_WARPS * 32 * (tn / 4 + 1) * 8 : 0; }
+constexpr int old_bytes(int tn) { return tn == 32 ? 2 * TM * 32 * 8 : 0; }
+constexpr int smem_bytes(int tn, bool trans) { return stages(tn, trans) * stage_bytes(tn) + trans_bytes(tn, trans) + old_bytes(tn); }
+constexpr int accum_sets(int tn) { return 512 / (NDIAG * tn); }
+
+// largest |sum of the digit products on diagonal D| per summed product: two
+// pairs with a leading digit (64 * 128 each) and D - 3 others (128 * 128)
+constexpr long diag_max(int D, long kc) { return (D == 2 ? 64L * 64 : (D - 2) * 128L * 128) * kc; }
+static_assert(diag_max(9, KC2) < (1L << 24), "diagonal sums must stay exact in fp32");
+// a float integer of magnitude up to 2^22 plus 1.5 * 2^23 holds it in its low mantissa bits
+static_assert(diag_max(6, KC1) <= (1L << 22) && diag_max(7, KC1) / 2 < (1L << 22), "KC = 64 conversion");
+static_assert(diag_max(4, KC2) <= (1L << 22) && diag_max(5, KC2) / 2 < (1L << 22) &&
+              (diag_max(6, KC2) + 256) / 4 < (1L << 22) && (diag_max(7, KC2) + 512) / 4 < (1L << 22), "KC = 128 conversion");
+static_assert(smem_bytes(64, true) <= 226 * 1024 && smem_bytes(64, false) <= 226 * 1024 &&
+              smem_bytes(32, true) <= 226 * 1024 && smem_bytes(32, false) <= 226 * 1024, "shared memory too large");
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -134,7 +145,7 @@ struct Src {
 __device__ __forceinline__ int row_exp(int evm) { return evm ? evm - 1022 : 0; }
 
 // The operands of one product call (A and B) as rows x K, cut into digit
-// blocks with row tiles of TR rows.  A complex operand yields the digits of
+// blocks.  A complex operand yields the digits of
 // its real part in out and of its imaginary part in out2, both scaled by one
 // power of two per row (above the row's largest |re| or |im|), so that the
 // products of both parts can share accumulators.
@@ -142,131 +153,151 @@ constexpr int MAXOPS = 4;
 template <typename T>
 struct SplitSet {
   Src<T> s[MAXOPS];
-  int R[MAXOPS], TR[MAXOPS], RT[MAXOPS];
+  int R[MAXOPS], ltr[MAXOPS], RT[MAXOPS];   // rows, log2 of the tile rows, row tiles
   uint8_t* out[MAXOPS];
   uint8_t* out2[MAXOPS];  // imaginary part's digits (complex operands)
   int* ex[MAXOPS];    // biased exponent of each row's largest |entry| (0: zero row)
   int items[MAXOPS];  // batch items to cut: 1 for an operand shared by every item
 };
 
-__device__ __forceinline__ unsigned long long mag_bits(double v) {
-  return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
-}
-__device__ __forceinline__ unsigned long long mag_bits(const cplx& v) {
-  return max(mag_bits(v.re), mag_bits(v.im));
-}
+// upper word of the magnitude (the larger part's of a complex entry)
+__device__ __forceinline__ uint32_t mag_hi(double v) { return (uint32_t)__double2hiint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint32_t mag_hi(const cplx& v) { return max(mag_hi(v.re), mag_hi(v.im)); }
 
-// Balanced base-64 digits of v 2^{FRAC - e} rounded to an integer, as bf16
-// values, for the 8 consecutive k of one 16-byte row segment of a block:
-// blk points at digit 0's segment; digit p lies BLK bytes further.
-__device__ __forceinline__ void put_digits(const double (&v)[8], int e, uint8_t* blk, int BLK) {
-  int dg[8][DIG];
+// Digits of v 2^{FRAC - e} rounded to an integer x (|x| < 2^62), as fp16
+// values, for the 8 consecutive k of one 16-byte row segment of a block: blk
+// points at digit 0's segment; digit p lies BLK bytes further.  With 128 added
+// at every byte position, x's balanced base-256 digits are the bytes of the
+// sum minus 128 each; a byte b becomes the fp16 value b - 128 as the difference
+// of 1024 + b (bits 0x6400 | b) and 1152, two digits per instruction.
+__device__ __forceinline__ void put_digits(const double (&v)[8], int evm, uint8_t* blk, int BLK) {
+  uint32_t x[8][2];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v[c]);
-    const int ev = (int)((u >> 52) & 0x7FF);
-    // |v| 2^{FRAC - e} rounded to an integer (<= 2^FRAC), then signed
-    const long long m = (long long)((u & 0xFFFFFFFFFFFFFull) | (1ull << 52));
-    const int sh = ev - (1075 - FRAC) - e;
-    long long x = 0;
-    if (ev != 0) {
-      if (sh >= 0) x = m << sh;
-      else if (sh > -62) x = ((m >> (-sh - 1)) + 1) >> 1;
-    }
-    if (u >> 63) x = -x;
-    // balanced base-64 digits, least significant first, in 32-bit halves:
-    // x = hi 2^30 + lo with 0 <= lo < 2^30.  A digit is d = (t & 63) - 32
-    // with t = v + 32, and the rest is (v - d) / 64 = t >> 6.  Five digits
-    // of lo leave a carry of 0 or 1 into hi; four of hi leave the leading
-    // digit (|.| <= 64).
-    int lo = (int)(x & 0x3FFFFFFFll), hi = (int)(x >> 30);
-#pragma unroll
-    for (int p = DIG - 1; p >= DIG - 5; --p) {
-      const int t = lo + 32;
-      dg[c][p] = (t & 63) - 32;
-      lo = t >> BITS;
-    }
-    hi += lo;
-#pragma unroll
-    for (int p = DIG - 6; p > 0; --p) {
-      const int t = hi + 32;
-      dg[c][p] = (t & 63) - 32;
-      hi = t >> BITS;
-    }
-    dg[c][0] = hi;
+    const uint32_t uh = (uint32_t)__double2hiint(v[c]), ul = (uint32_t)__double2loint(v[c]);
+    const int ev = (int)((uh >> 20) & 0x7FF);
+    // |v| 2^{FRAC - e + 1} is the mantissa << 10 shifted right by the
+    // distance of v's exponent to the row's largest
+    const unsigned long long full = ((unsigned long long)((uh & 0xFFFFFu) | 0x100000u) << 32 | ul) << 10;
+    unsigned long long m = full >> min(evm - ev, 63);
+    m = ev == 0 ? 0ull : (m + 1) >> 1;
+    const unsigned long long t = (int)uh < 0 ? 0x8080808080808080ull - m : 0x8080808080808080ull + m;
+    x[c][1] = (uint32_t)t;
+    x[c][0] = (uint32_t)(t >> 32);
   }
 #pragma unroll
   for (int p = 0; p < DIG; ++p) {
+    const uint32_t byte = 3 - (p & 3);
     uint32_t w[4];
 #pragma unroll
     for (int c = 0; c < 8; c += 2) {
-      // d (|d| <= 64) as an exact float: 1.5 * 2^23 + d has d in its low
-      // mantissa bits; subtracting 1.5 * 2^23 leaves d, whose upper 16
-      // bits are its bf16 encoding (d has at most 7 significant bits)
-      const float f0 = __int_as_float(0x4B400000 + dg[c][p]) - 12582912.0f;
-      const float f1 = __int_as_float(0x4B400000 + dg[c + 1][p]) - 12582912.0f;
-      w[c >> 1] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+      const uint32_t b2 =
+          (__byte_perm(x[c][p >> 2], x[c + 1][p >> 2], byte | (byte + 4) << 8) & 0x00FF00FFu) | 0x64006400u;
+      asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w[c >> 1]) : "r"(b2), "r"(0xE480E480u));
     }
     *reinterpret_cast<uint4*>(blk + (int64_t)p * BLK) = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
-// One launch for all operands: CTA = 32 rows x 8 warps; warp w takes the
-// 8-deep k groups w, w+8, ...  Pass 1 finds each row's largest magnitude
-// (compared as bit patterns, which order like the values; over both parts
-// of a complex row), pass 2 writes the balanced base-64 digits of the row
-// scaled by 2^{FRAC - e}, rounded to an integer (both parts of a complex
-// row from one read).
+// One launch for all operands.  A warp takes units of 32 rows x UK k (16 for
+// real data: a whole k step; 8 for complex); of a CTA's 8 warps, KW share 32
+// rows and split the units of their inner dimension, and 8 / KW such row
+// groups share the CTA, so that short inner dimensions keep every warp busy.
+// Long ones spread over the CS CTAs of a cluster as well (few rows and many k
+// would leave most SMs idle).  Pass 1 finds each row's largest magnitude (by
+// its upper word: only the exponent counts; over both parts of a complex
+// row), pass 2 writes the digits; when no warp has more than one unit, each
+// entry is read once and stays in registers.  An operand whose k runs along
+// its columns (ks = 1: B, or B^T in the A slot) is read in segments of UK
+// entries per row and turned around in shared memory: one row per lane would
+// touch 32 cache lines per load.  Rows beyond R are not written: their
+// products land in outputs that nobody stores.
 template <typename T>
-__global__ void __launch_bounds__(256) k_split(SplitSet<T> ss, int K, int KT, int b0, int nb) {
-  const int op = blockIdx.z / nb, bl = blockIdx.z % nb, b = b0 + bl;
-  const int R = ss.R[op], TR = ss.TR[op], Rpad = ss.RT[op] * TR;
-  if (blockIdx.x * 32 >= Rpad || bl >= ss.items[op]) return;  // uniform over the CTA
+__global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT, int b0, int KW, int CS) {
+  constexpr int UK = std::is_same<T, cplx>::value ? 8 : 16;   // k per unit
+  constexpr int RL = 32 / UK;                                 // rows per load of a turned unit
+  const int op = blockIdx.y, bl = blockIdx.z, b = b0 + bl;
+  const int R = ss.R[op], lt = ss.ltr[op], Rpad = ss.RT[op] << lt;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cr = (int)blockIdx.x % CS;                        // CTA of the cluster (clusters run along x)
+  const int rg = (int)blockIdx.x / CS;
+  if (rg * (8 / KW) * 32 >= R || bl >= ss.items[op]) return;  // uniform over the cluster
   const Src<T>& s = ss.s[op];
-  const int lr = threadIdx.x & 31, kw = threadIdx.x >> 5;
-  const int r = blockIdx.x * 32 + lr;
+  const int kw = warp & (KW - 1);
+  const int rbase = (rg * (8 / KW) + warp / KW) * 32;
+  const int r = rbase + lane;
   const T* X = s.X.item(b);
   const bool live = r < R;
   const int64_t roff = live ? (int64_t)s.rmap.at(b, r) * s.rs : 0;
-  const int ngrp = KT * 2;
-  __shared__ unsigned long long smax[8][32];
-  unsigned long long mx = 0;
-  if (live)
-    for (int gi = kw; gi < ngrp; gi += 8)
-      for (int c = 0; c < 8; ++c) {
-        const int k = gi * 8 + c;
-        if (k >= K) break;
-        mx = max(mx, mag_bits(X[roff + (int64_t)s.kmap.at(b, k) * s.ks]));
+  const int* kidx = s.kmap.idx ? s.kmap.idx + (b % s.kmap.period) * s.kmap.len : nullptr;
+  const int64_t rs = s.rs, ks = s.ks;
+  const bool turn = ks == 1 && !s.rmap.idx;
+  const int nu = KT * (TK / UK), step = KW * CS, u0 = cr * KW + kw;
+  __shared__ uint32_t smax[8][32];
+  __shared__ uint32_t cmax[8][8][32];   // [CTA of the cluster][row group][row]
+  __shared__ T tile[8][32 * (UK + 1)];
+  T xv[UK];
+  auto load = [&](int u) {
+    if (turn) {
+      const int k = u * UK + (lane & (UK - 1));
+      const int64_t ko = k < K ? (kidx ? (int64_t)kidx[k] : (int64_t)k) : -1;
+#pragma unroll
+      for (int q = 0; q < UK; ++q) {
+        const int row = rbase + q * RL + lane / UK;
+        xv[q] = (ko >= 0 && row < R) ? X[(int64_t)row * rs + ko] : T(0.0);
       }
-  smax[kw][lr] = mx;
-  __syncthreads();
+      __syncwarp();
 #pragma unroll
-  for (int w = 0; w < 8; ++w) mx = max(mx, smax[w][lr]);
-  const int evm = (int)(mx >> 52);
-  if (kw == 0 && r < Rpad) ss.ex[op][(int64_t)bl * Rpad + r] = evm;
-  if (r >= Rpad) return;
-  const bool zero = evm == 0;
-  const int e = row_exp(evm);
-  const int BLK = TR * TK * 2;
-  const int tile = r / TR, rr = r % TR;
-  const int64_t rowoff = ((int64_t)bl * ss.RT[op] + tile) * KT * (int64_t)(DIG * BLK) + (rr >> 3) * 256 + (rr & 7) * 16;
-  for (int gi = kw; gi < ngrp; gi += 8) {
-    const int k0 = gi * 8;
-    T xv[8];
+      for (int q = 0; q < UK; ++q) tile[warp][(q * RL + lane / UK) * (UK + 1) + (lane & (UK - 1))] = xv[q];
+      __syncwarp();
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int k = k0 + c;
-      xv[c] = (live && !zero && k < K) ? X[roff + (int64_t)s.kmap.at(b, k) * s.ks] : T(0.0);
+      for (int c = 0; c < UK; ++c) xv[c] = tile[warp][lane * (UK + 1) + c];
+    } else {
+#pragma unroll
+      for (int c = 0; c < UK; ++c) {
+        const int k = u * UK + c;
+        xv[c] = (live && k < K) ? X[roff + (int64_t)(kidx ? kidx[k] : k) * ks] : T(0.0);
+      }
     }
-    const int64_t boff = rowoff + (int64_t)(k0 >> 4) * (DIG * BLK) + ((k0 >> 3) & 1) * 128;
-    double v[8];
+  };
+  uint32_t mx = 0;
+  for (int u = u0; u < nu; u += step) {
+    load(u);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = part_of(xv[c], 0);
-    put_digits(v, e, ss.out[op] + boff, BLK);
-    if constexpr (std::is_same<T, cplx>::value) {
+    for (int c = 0; c < UK; ++c) mx = max(mx, mag_hi(xv[c]));
+  }
+  smax[warp][lane] = mx;
+  __syncthreads();
+  for (int w = 0; w < KW; ++w) mx = max(mx, smax[warp - kw + w][lane]);
+  if (CS > 1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    if (kw == 0)
+      for (int d = 0; d < CS; ++d) cl.map_shared_rank(&cmax[0][0][0], d)[(cr * 8 + warp) * 32 + lane] = mx;
+    cl.sync();
+    for (int d = 0; d < CS; ++d) mx = max(mx, cmax[d][warp - kw][lane]);
+  }
+  const int evm = (int)(mx >> 20);
+  if (kw == 0 && cr == 0 && live) ss.ex[op][(int64_t)bl * Rpad + r] = evm;
+  const int BLK = TK * 2 << lt;
+  const int tl = r >> lt, rr = r & ((1 << lt) - 1);
+  const int64_t rowoff = ((int64_t)bl * ss.RT[op] + tl) * KT * (int64_t)(DIG * BLK) + (rr >> 3) * 256 + (rr & 7) * 16;
+  for (int u = u0; u < nu; u += step) {
+    if (nu > step) load(u);
+    if (!live) continue;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) v[c] = part_of(xv[c], 1);
-      put_digits(v, e, ss.out2[op] + boff, BLK);
+    for (int half = 0; half < UK / 8; ++half) {
+      const int k8 = u * (UK / 8) + half;   // 8-deep k group
+      const int64_t boff = rowoff + (int64_t)(k8 >> 1) * (DIG * BLK) + (k8 & 1) * 128;
+      double v[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = part_of(xv[half * 8 + c], 0);
+      put_digits(v, evm, ss.out[op] + boff, BLK);
+      if constexpr (std::is_same<T, cplx>::value) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = part_of(xv[half * 8 + c], 1);
+        put_digits(v, evm, ss.out2[op] + boff, BLK);
+      }
     }
   }
 }
@@ -291,7 +322,69 @@ __device__ __forceinline__ double fixed_to_double(long long R, int es) {
   return __longlong_as_double((long long)(sgn | (((unsigned long long)(e2 + 1022) << 52) + m)));
 }
 
-template <typename T>
+__device__ __noinline__ double fixed_slow(long long R, int es) { return fixed_to_double(R, es); }
+
+// R 2^(E - 1086) as a double when |R| >= 2^32 and the result is normal (the
+// caller has checked both): as fixed_to_double with one count of leading
+// zeros, no range checks, and ties (one value in 1024) rounded away from zero.
+__device__ __forceinline__ double fixed_fast(long long R, int E, uint32_t flip) {
+  const uint32_t hi = (uint32_t)((unsigned long long)R >> 32);
+  const uint32_t s = (uint32_t)((int)hi >> 31);
+  const unsigned long long a0 = ((unsigned long long)R ^ ((unsigned long long)s << 32 | s)) + (s & 1u);
+  const uint32_t ah = (uint32_t)(a0 >> 32), al = (uint32_t)a0;
+  const int sh = __clz((int)ah) - 1;           // 0 .. 30; the leading one goes to bit 62
+  const unsigned long long a = ((unsigned long long)__funnelshift_l(al, ah, sh) << 32 | (al << sh)) + 512ull;
+  const uint32_t nh = (uint32_t)(a >> 32), nl = (uint32_t)a;
+  // 53 bits; the hidden bit adds one to the exponent field
+  const uint32_t oh = (nh >> 10) + ((uint32_t)(E - 2 - sh) << 20);
+  return __hiloint2double((int)(oh | ((hi ^ flip) & 0x80000000u)), (int)__funnelshift_r(nl, nh, 10));
+}
+
+// The eight diagonal sums x_D (exact floats) of one output as a fixed-point
+// integer, rounded once: units of 2^-57 (KC = 64) or 2^{-56 + sh} (KC = 128,
+// sh = 0 .. 6).  A sum below 2^22 becomes an integer with one addition (its
+// bits after adding 1.5 * 2^23); a larger one is halved or quartered with
+// rounding and its small remainder handed to the next diagonal, where it is
+// 256 times as much and the sum stays below 2^24.  The two lowest diagonals
+// and the last remainder are rounded to the unit, unbiased.
+template <int KC>
+__device__ __forceinline__ long long diag_fixed(const float (&x)[NDIAG], int sh, float unit) {
+  constexpr float MG = 12582912.0f;            // 1.5 * 2^23
+  constexpr uint32_t MB = 0x4B400000u;         // its bits
+  if constexpr (KC == KC1) {
+    const uint32_t a2 = __float_as_uint(x[0] + MG), a3 = __float_as_uint(x[1] + MG);
+    const uint32_t a4 = __float_as_uint(x[2] + MG), a5 = __float_as_uint(x[3] + MG);
+    const uint32_t a6 = __float_as_uint(x[4] + MG);
+    const float h7 = fmaf(x[5], 0.5f, MG), r7 = fmaf(h7 - MG, -2.0f, x[5]);
+    const float z = fmaf(r7, 256.0f, fmaf(x[7], 1.0f / 256.0f, x[6]));
+    const uint32_t c = __float_as_uint(fmaf(z, 1.0f / 8.0f, MG));              // units 2^-57
+    // x6 2^13 + (x7 / 2) 2^6 + c; the offset of c's bits goes into the sum's
+    const int P = (int)(a6 * 128u + __float_as_uint(h7) - (129u * MB + (MB >> 6)));
+    const int Q = (int)(a4 * 256u + a5 - 257u * MB);                            // units 2^-36: 2^21
+    const int S = (int)(a2 * 256u + a3 - 257u * MB);                            // units 2^-20: 2^37
+    long long w = (long long)P * 64 + (long long)(unsigned long long)c;
+    w += (long long)Q * (1ll << 21);
+    return w + ((long long)S << 37);
+  } else {
+    const uint32_t a2 = __float_as_uint(x[0] + MG), a3 = __float_as_uint(x[1] + MG);
+    const uint32_t a4 = __float_as_uint(x[2] + MG);
+    const float h5 = fmaf(x[3], 0.5f, MG), r5 = fmaf(h5 - MG, -2.0f, x[3]);
+    const float y6 = fmaf(r5, 256.0f, x[4]);
+    const float h6 = fmaf(y6, 0.25f, MG), r6 = fmaf(h6 - MG, -4.0f, y6);
+    const float y7 = fmaf(r6, 256.0f, x[5]);
+    const float h7 = fmaf(y7, 0.25f, MG), r7 = fmaf(h7 - MG, -4.0f, y7);
+    const float z = fmaf(r7, 256.0f, fmaf(x[7], 1.0f / 256.0f, x[6]));
+    const uint32_t c = __float_as_uint(fmaf(z, unit, MG));                      // z / 16, units of 2^-56, at sh = 0
+    // in units of 2^-56: (x6 / 4) 2^14 + (x7 / 4) 2^6 + c
+    const int P = (int)(__float_as_uint(h6) * 256u + __float_as_uint(h7) - (257u * MB + (MB >> (6 - sh))));
+    const int Q = (int)(a4 * 128u + __float_as_uint(h5) - 129u * MB);           // x4 2^28 + (x5 / 2) 2^21
+    const int S = (int)(a2 * 256u + a3 - 257u * MB);                            // 2^36
+    long long w = (long long)P * (64 >> sh) + (long long)(unsigned long long)c;
+    w += (long long)Q * (int)((1u << 21) >> sh);
+    return w + ((long long)S << (36 - sh));
+  }
+}
+
 struct GemmP {
   const uint8_t* As;
   const uint8_t* Bs;
@@ -306,36 +399,50 @@ struct GemmP {
   int MT, NT, KT, M, N;
   int lsb;             // fraction bits of the fixed-point result
   double alpha, beta;
-  int amode;                 // 1: alpha = +-1 (applied as a sign flip)
-  long long asign;           // sign bit to flip when amode = 1
-  BOp<T> C;
+  long long asign;     // alpha = +-1: sign bit to flip
+  // C as doubles: strides and offsets in doubles, W doubles per entry (2 for
+  // complex C, whose component is part of the offset)
+  BOp<double> C;
+  int W;
   IMap crow;
-  int cpart;           // complex C: component written (0 re, 1 im)
   int b0;              // first batch item of this launch
   int a_bl, b_bl;      // 1, or 0 for an operand whose digits serve every item
   int nitems;          // batch items of this launch (tiles: MT NT nitems)
   unsigned* err;
 };
 
-template <typename T, bool BETA0, bool TRANS>
-__global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
+// Epilogue forms: C <- +-P, C <- C +- P, or alpha P + beta C.  Kept apart:
+// FP64 instructions of a form not taken still cost the FP64 pipe its cycles
+// when the compiler predicates them.
+enum { TC_SET = 0, TC_ADD = 1, TC_GENERAL = 2 };
+
+// What bounds it: at long K the tensor pipe (36 products of 128 x TN x 16 per
+// k step), at short K the epilogue: one FP64 addition per output (2 per
+// clock and SM) and ~60 other instructions.  Sixteen epilogue warps of at
+// most 112 registers keep four warps on each scheduler (eight warps of 167
+// registers issued in 27 % of the cycles).
+template <int EPI, bool TRANS, int TN, int KC>
+__global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP g) {
   // Persistent: CTA c takes the tiles c, c + gridDim.x, ... of the launch
   // (tile t = item t / (MT NT), then row tile, then column tile), so that the
   // next tile's copies and products overlap this tile's epilogue and the
   // TMEM allocation and barrier set-up happen once per CTA.  The stage ring,
   // the accumulator hand-over (acc_full / acc_empty) and their phases run on
   // across tiles.
+  constexpr int NST = stages(TN, TRANS), STAGE = stage_bytes(TN), BBLK = bblk(TN), BSTG = bstg(TN);
+  constexpr int NSET = accum_sets(TN);      // accumulator sets taken in turn
+  constexpr int QGRP = 256 / TN;            // B digits stacked into one MMA (N <= 256)
+  constexpr int ECOLS = TN / 4;             // columns per epilogue warp
+  constexpr int KCT = KC2 / TK;             // k steps per chunk (a KC = 64 tile has one chunk)
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t full[NST], empty[NST], acc_full, acc_empty;
-  __shared__ int s_eb[TN];
+  __shared__ __align__(8) uint64_t full[NST], empty[NST], acc_full[NSET], acc_empty[NSET];
   __shared__ uint32_t tslot;
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_item = g.MT * g.NT;
   const int ntiles = tiles_item * g.nitems;
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)),
-                 "r"(TMEM_COLS));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "n"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (threadIdx.x == 32) {
@@ -343,8 +450,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&full[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&empty[i])));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&acc_full)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acc_empty)), "r"(32 * EPI_WARPS));
+    for (int i = 0; i < NSET; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&acc_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acc_empty[i])), "n"(EPI_WARPS));
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     abort_flag = 0;
   }
@@ -354,7 +463,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
   const uint32_t tmem = tslot;
   volatile int* abrt = &abort_flag;
   const int KTV = g.pair ? 2 * g.KT : g.KT;   // k steps of a tile (both products of a pair)
-  const int nchunk = (KTV + KCT - 1) / KCT;
+  const int nchunk = KC == KC1 ? 1 : (KTV + KCT - 1) / KCT;
   const uint32_t sbase = su32(smem);
 
   if (warp == EPI_WARPS) {
@@ -392,22 +501,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
       }
     }
   } else if (warp == EPI_WARPS + 1) {
-    // MMA issue: 55 digit-pair products per k step into the 10 diagonal accumulators
+    // MMA issue: 36 digit-pair products per k step into the 8 diagonal accumulators
     if (lane == 0) {
       // B's digit blocks lie one after another with the same row-group stride,
-      // so digits q0 .. q0+n-1 form one operand of n * 48 rows, and A_p times
+      // so digits q0 .. q0+n-1 form one operand of n * TN rows, and A_p times
       // it lands in the accumulators of diagonals p+q0 .. p+q0+n-1, which are
-      // adjacent in TMEM: one MMA (N <= 240) per (p, group of <= 5 digits).
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
+      // adjacent in TMEM: one MMA (N <= 256) per (p, group of <= QGRP digits).
+      // Instruction descriptor: fp32 accumulator, A and B fp16, K-major.
+      const uint32_t idesc0 = (1u << 4) | ((uint32_t)(TM >> 4) << 24);
       long it = 0, cc = 0;   // k steps and accumulator chunks issued so far
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int kk = 0;
         for (int c = 0; c < nchunk && ok; ++c, ++cc) {
-          // the epilogue has read the previous chunk's accumulators
-          if (cc > 0 && !mbar_wait(su32(&acc_empty), (int)((cc - 1) & 1), abrt)) { ok = false; break; }
+          const int set = (int)(cc % NSET);
+          const uint32_t tset = tmem + (uint32_t)(set * NDIAG * TN);
+          // the epilogue has read this set's previous chunk
+          if (cc >= NSET && !mbar_wait(su32(&acc_empty[set]), (int)((cc / NSET) & 1) ^ 1, abrt)) { ok = false; break; }
           fence_after();
-          const int kend = min(KTV, (c + 1) * KCT);
+          const int kend = KC == KC1 ? KTV : min(KTV, (c + 1) * KCT);
           const int kbeg = kk;
           for (; kk < kend; ++kk, ++it) {
             const int s = (int)(it % NST);
@@ -420,7 +532,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
 #pragma unroll
             for (int p = 0; p < DIG; ++p) {
               const uint64_t ad = sdesc(a0 + p * ABLK, 128, 256);
-              const int nq_all = (DSUM - 1 - p) < DIG ? (DSUM - 1 - p) : DIG;   // q = 0 .. nq_all-1
+              const int nq_all = DSUM - 1 - p;   // q = 0 .. nq_all-1
 #pragma unroll
               for (int q0 = 0; q0 < nq_all; q0 += QGRP) {
                 const int nq = (nq_all - q0) < QGRP ? (nq_all - q0) : QGRP;
@@ -430,7 +542,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
                 const uint32_t idesc = idesc0 | ineg | ((uint32_t)((nq * TN) >> 3) << 17);
                 asm volatile(
                     "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)((p + q0) * TN)),
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tset + (uint32_t)((p + q0) * TN)),
                     "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
               }
             }
@@ -440,7 +552,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
           }
           if (!ok) break;
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           su32(&acc_full))
+                           su32(&acc_full[set]))
                        : "memory");
         }
       }
@@ -450,153 +562,205 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP<T> g) {
       }
     }
   } else {
-    // epilogue: warp w reads TMEM lane quarter w % 4 (its rows) and column
-    // half w / 4; thread = row, 24 fixed-point sums.  While the MMAs run, the
-    // C tile (beta != 0) and the columns' exponents are staged in shared
-    // memory with asynchronous copies.  A transposed tile (rows of C^T are
-    // C's columns) is staged and stored by all epilogue threads with the tile
-    // column fastest, so that its global accesses stay coalesced, and each
-    // thread's results pass through shared memory.  Every epilogue thread
-    // runs the same tiles and the same named barriers; after a wait gives up
-    // it skips the remaining waits and stores but still takes the barriers.
+    // epilogue: warp w reads TMEM lane quarter w % 4 (its rows) and columns
+    // (w / 4) ECOLS ..; thread = row.  A normal tile's rows are C's rows, so
+    // its accesses are coalesced as they are; a transposed tile's rows are C's
+    // columns: the warp's results pass through its own block of shared memory
+    // and leave with the tile column (C's row) fastest.  No barrier between
+    // the epilogue warps; a warp none of whose rows or columns exist only
+    // waits and arrives.  After a wait gives up (agreed over the warp) it
+    // skips the remaining waits and stores.
     const int quarter = warp & 3, c0 = (warp >> 2) * ECOLS;
-    const int row = quarter * 32 + lane;
-    double* s_c = reinterpret_cast<double*>(smem + NST * STAGE);
-    constexpr int SLD = TRANS ? TMP : TM;   // staging stride
-    constexpr int W = (int)(sizeof(T) / sizeof(double));
-    const int etid = threadIdx.x;   // 0 .. 32 * EPI_WARPS - 1
-    // diagonal d = di + 2 has weight 2^{-6d}; R counts units of 2^{-lsb}.
-    // Adjacent diagonals pair up exactly in 32 bits (y = x_d * 64 + x_{d+1},
-    // |y| < 2^29), the pairs of d = 2..7 form H (units 2^{-42}) and those of
-    // d = 8..11 form L (units 2^{-66}) in 64 bits; H enters R exactly and L
-    // rounded once.  lsb is at least 42 (K <= 2^20).
-    const int shH = g.lsb - 42, shL = 66 - g.lsb;
-    const long long halfL = 1ll << (shL - 1);
-    const bool amode1 = g.amode == 1, beta1 = g.beta == 1.0;
-    bool ok = true;
-    long cc = 0;   // accumulator chunks consumed so far
-    bool first = true;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    double* s_c = reinterpret_cast<double*>(smem + NST * STAGE) + warp * 32 * (ECOLS + 1);
+    // TN = 32: the old C values of the next tile are copied into this thread's
+    // slots of shared memory while this tile is converted
+    double* s_old = reinterpret_cast<double*>(smem + NST * STAGE + trans_bytes(TN, TRANS)) + (warp * 32 + lane) * 1;
+    constexpr bool STAGED = TN == 32 && EPI != TC_SET;
+    constexpr int OSET = EPI_WARPS * 32 * ECOLS;   // doubles per staged tile
+    constexpr int RSTEP = 32 / ECOLS;         // transposed: C columns per store
+    const uint32_t flip = (uint32_t)((unsigned long long)g.asign >> 32);
+    const int sh = min(LSB2 - g.lsb, 6), sh2 = LSB2 - g.lsb - sh;   // KC = 128: unit of a chunk, rest beyond 6 bits
+    const float unit = 1.0f / (float)(16 << sh);
+    struct Tile {
+      double* Cp;          // this thread's first C entry (normal: its tile row; transposed: its tile column's row)
+      int ebase, eb;       // exponent of its row (with the fixed point's), of column `lane`
+      int nrow, ncol;      // rows and columns of this warp that exist (<= 0: none)
+      bool safe;           // every exponent is far from the ends of the range
+    };
+    const int64_t cstep = (int64_t)g.C.ld * g.W * (TRANS ? RSTEP : 1);
+    // entry jj of this thread exists
+    auto live = [&](const Tile& q, int jj) {
+      return TRANS ? (lane % ECOLS < q.ncol && jj * RSTEP + lane / ECOLS < q.nrow) : (lane < q.nrow && jj < q.ncol);
+    };
+    auto setup = [&](int t, int buf) {
+      Tile q;
       const int bl = t / tiles_item, rem = t % tiles_item;
       const int mt = rem % g.MT, nt = rem / g.MT;
-      const int i = mt * TM + row;
-      const int b = g.b0 + bl;
-      double* Cb = reinterpret_cast<double*>(g.C.item(b));
-      const int64_t ci = (!TRANS && i < g.M) ? (int64_t)g.crow.at(b, i) : 0;
-      // the previous tile's conversion has finished with s_eb and s_c
-      if (!first) asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS) : "memory");
-      first = false;
-      if (threadIdx.x < TN)
-        s_eb[threadIdx.x] = nt * TN + threadIdx.x < g.N ? row_exp(g.eb[(int64_t)(bl * g.b_bl) * g.NT * TN + nt * TN + threadIdx.x]) : 0;
-      // the old C values of a normal tile go straight to registers (issued
-      // now, they arrive while the products finish); a transposed tile's are
-      // staged in shared memory, tile column fastest
-      double cold[ECOLS];
-      if constexpr (!TRANS) {
-        if (!BETA0 && ok && i < g.M) {
+      const int i0 = mt * TM + quarter * 32, j0 = nt * TN + c0;
+      q.nrow = min(32, g.M - i0);
+      q.ncol = min(ECOLS, g.N - j0);
+      q.Cp = nullptr;
+      q.ebase = q.eb = 0;
+      q.safe = true;
+      if (q.nrow > 0 && q.ncol > 0) {
+        const int b = g.b0 + bl;
+        const int crw = TRANS ? j0 + lane % ECOLS : i0 + lane;
+        const int ccl = TRANS ? i0 + lane / ECOLS : j0;
+        const bool in = crw < (TRANS ? g.N : g.M);
+        int er = 0;
+        if (lane < q.nrow) er = row_exp(g.ea[(int64_t)(bl * g.a_bl) * g.MT * TM + i0 + lane]);
+        if (lane < q.ncol) q.eb = row_exp(g.eb[(int64_t)(bl * g.b_bl) * g.NT * TN + j0 + lane]);
+        q.Cp = g.C.item(b) + ((int64_t)(in ? g.crow.at(b, crw) : 0) + (int64_t)ccl * g.C.ld) * g.W;
+        if constexpr (STAGED) {
 #pragma unroll
-          for (int jj = 0; jj < ECOLS; ++jj) {
-            const int col = nt * TN + c0 + jj;
-            cold[jj] = col < g.N ? Cb[(ci + (int64_t)col * g.C.ld) * W + g.cpart] : 0.0;
-          }
+          for (int jj = 0; jj < ECOLS; ++jj)
+            if (live(q, jj))
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(su32(s_old + buf * OSET + jj * (EPI_WARPS * 32))),
+                           "l"(q.Cp + cstep * jj) : "memory");
+        } else if constexpr (EPI != TC_SET && KC != KC1) {
+#pragma unroll
+          for (int jj = 0; jj < ECOLS; ++jj)
+            if (live(q, jj)) asm volatile("prefetch.global.L2 [%0];" ::"l"(q.Cp + cstep * jj));
         }
+        q.safe = __all_sync(0xffffffffu, abs(er) <= 400 && abs(q.eb) <= 400);
+        q.ebase = er - g.lsb + 1086;
       }
-      if (!BETA0 && ok) {
-        if constexpr (TRANS) {
-          for (int e2 = etid; e2 < TM * TN; e2 += 32 * EPI_WARPS) {
-            const int j = e2 % TN, r = e2 / TN;
-            const int crw = nt * TN + j, ccol = mt * TM + r;
-            if (crw < g.N && ccol < g.M)
-              asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(su32(s_c + j * TMP + r)),
-                           "l"(Cb + ((int64_t)g.crow.at(b, crw) + (int64_t)ccol * g.C.ld) * W + g.cpart)
-                           : "memory");
-          }
+      if constexpr (STAGED) asm volatile("cp.async.commit_group;" ::: "memory");
+      return q;
+    };
+    bool ok = true;
+    long cc = 0;   // accumulator chunks consumed so far
+    int buf = 0;
+    constexpr bool AHEAD = TN == 32;   // the next tile's addresses, exponents and copies a tile ahead
+    Tile nx;
+    if (AHEAD && (int)blockIdx.x < ntiles) nx = setup(blockIdx.x, 0);
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
+      const Tile q = AHEAD ? nx : setup(t, 0);
+      const bool any = q.nrow > 0 && q.ncol > 0;   // this warp has outputs
+      const bool more = t + (int)gridDim.x < ntiles;
+      if (AHEAD && more) nx = setup(t + gridDim.x, buf ^ 1);
+      double cold[STAGED || EPI == TC_SET ? 1 : ECOLS];
+      auto load_old = [&]() {
+        if constexpr (!STAGED && EPI != TC_SET) {
+#pragma unroll
+          for (int jj = 0; jj < ECOLS; ++jj) cold[jj] = live(q, jj) ? q.Cp[cstep * jj] : 0.0;
         }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      long long R[ECOLS];
+      };
+      auto old_c = [&](int jj) { return STAGED ? s_old[buf * OSET + jj * (EPI_WARPS * 32)] : cold[STAGED ? 0 : jj]; };
+      auto finish = [&](double val, int jj) {
+        if constexpr (EPI == TC_SET) return val;
+        else if constexpr (EPI == TC_ADD) return old_c(jj) + val;
+        else return fma(g.alpha, val, g.beta == 0.0 ? 0.0 : g.beta * old_c(jj));
+      };
+      // four adjacent results.  |R| below 2^32 (zeros among them) and extreme
+      // exponents take the general form, all lanes together
+      auto convert4 = [&](const long long (&R)[4], int jb) {
+        bool fast = q.safe;
 #pragma unroll
-      for (int j = 0; j < ECOLS; ++j) R[j] = 0;
-      for (int c = 0; c < nchunk; ++c, ++cc) {
-        if (!ok) continue;
-        if (!mbar_wait(su32(&acc_full), (int)(cc & 1), abrt)) { ok = false; continue; }
-        fence_after();
+        for (int j = 0; j < 4; ++j) fast = fast && (uint32_t)((unsigned long long)R[j] >> 32) + 1u > 1u;
+        fast = __all_sync(0xffffffffu, fast || lane >= q.nrow);
+        double val[4];
+        if (fast) {
 #pragma unroll
-        for (int cg = 0; cg < ECOLS / 4; ++cg) {
-          uint32_t v[NDIAG][4];
-#pragma unroll
-          for (int di = 0; di < NDIAG; ++di) {
-            const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(di * TN + c0 + cg * 4);
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                         : "=r"(v[di][0]), "=r"(v[di][1]), "=r"(v[di][2]), "=r"(v[di][3])
-                         : "r"(ta));
-          }
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          for (int j = 0; j < 4; ++j)
+            val[j] = fixed_fast(R[j], q.ebase + __shfl_sync(0xffffffffu, q.eb, jb + j), EPI == TC_GENERAL ? 0u : flip);
+        } else {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            // an fp32 holding an integer below 2^22, plus 1.5 * 2^23, has the
-            // integer in its low mantissa bits: x = bits - 0x4B400000
-            int y[NDIAG / 2];
+            val[j] = fixed_slow(R[j], q.ebase - 1086 + __shfl_sync(0xffffffffu, q.eb, jb + j));
+            if (EPI != TC_GENERAL) val[j] = __longlong_as_double(__double_as_longlong(val[j]) ^ g.asign);
+          }
+        }
+        if constexpr (TRANS) {
 #pragma unroll
-            for (int k = 0; k < NDIAG / 2; ++k) {
-              const uint32_t a = __float_as_uint(__uint_as_float(v[2 * k][j]) + 12582912.0f);
-              const uint32_t c2 = __float_as_uint(__uint_as_float(v[2 * k + 1][j]) + 12582912.0f);
-              y[k] = (int)(a * 64u + c2 - 65u * 0x4B400000u);
+          for (int j = 0; j < 4; ++j) s_c[lane * (ECOLS + 1) + jb + j] = val[j];
+        } else if (lane < q.nrow) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (jb + j < q.ncol) q.Cp[cstep * (jb + j)] = finish(val[j], jb + j);
+        }
+      };
+      auto old_ready = [&]() {
+        if constexpr (STAGED) {   // this tile's copies: all but the group of the next tile
+          if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+          else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+      };
+      if (KC == KC1 && any && ok) load_old();   // arrive while the products finish
+      long long R[ECOLS / 4][4];
+      for (int c = 0; c < nchunk; ++c, ++cc) {
+        if (!ok) continue;
+        const int set = (int)(cc % NSET);
+        ok = __all_sync(0xffffffffu, mbar_wait(su32(&acc_full[set]), (int)((cc / NSET) & 1), abrt));
+        if (!ok) continue;
+        fence_after();
+        if (any) {
+          if (KC == KC1 && !TRANS) old_ready();
+          const uint32_t ta0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(set * NDIAG * TN + c0);
+#pragma unroll
+          for (int cg = 0; cg < ECOLS / 4; ++cg) {
+            uint32_t v[NDIAG][4];
+#pragma unroll
+            for (int di = 0; di < NDIAG; ++di)
+              asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                           : "=r"(v[di][0]), "=r"(v[di][1]), "=r"(v[di][2]), "=r"(v[di][3])
+                           : "r"(ta0 + (uint32_t)(di * TN + cg * 4)));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (cg == ECOLS / 4 - 1) {
+              fence_before();
+              __syncwarp();
+              if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acc_empty[set])) : "memory");
             }
-            const long long H = ((long long)y[0] << 24) + ((long long)y[1] << 12) + (long long)y[2];
-            const long long L = ((long long)y[3] << 12) + (long long)y[4];
-            R[cg * 4 + j] += (H << shH) + ((L + halfL) >> shL);
-          }
-        }
-        fence_before();
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acc_empty)) : "memory");
-      }
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS) : "memory");   // s_eb and s_c from other epilogue threads
-      if (ok && i < g.M) {
-        const int er = row_exp(g.ea[(int64_t)(bl * g.a_bl) * g.MT * TM + i]);
+            long long w4[4];
 #pragma unroll
-        for (int jj = 0; jj < ECOLS; ++jj) {
-          const int j = c0 + jj;
-          const int col = nt * TN + j;
-          if (col >= g.N) break;
-          double val = fixed_to_double(R[jj], er + s_eb[j] - g.lsb);
-          double* sp = s_c + j * SLD + row;
-          double c_old = 0.0;
-          if constexpr (!BETA0) c_old = TRANS ? *sp : cold[jj];
-          double out;
-          if (amode1) {                // alpha = +-1: a sign flip
-            val = __longlong_as_double(__double_as_longlong(val) ^ g.asign);
-            if (BETA0) out = val;
-            else if (beta1) out = c_old + val;
-            else out = fma(g.beta, c_old, val);
-          } else {
-            if (BETA0) out = g.alpha * val;
-            else out = fma(g.alpha, val, g.beta * c_old);
+            for (int j = 0; j < 4; ++j) {
+              float x[NDIAG];
+#pragma unroll
+              for (int di = 0; di < NDIAG; ++di) x[di] = __uint_as_float(v[di][j]);
+              w4[j] = diag_fixed<KC>(x, sh, unit);
+            }
+            if constexpr (KC == KC1) {
+              convert4(w4, cg * 4);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                long long w = w4[j];
+                if (sh2 > 0) w = (w + (1ll << (sh2 - 1)) - ((~w >> sh2) & 1)) >> sh2;   // ties to even
+                R[cg][j] = c == 0 ? w : R[cg][j] + w;
+              }
+            }
           }
-          if constexpr (!TRANS) Cb[(ci + (int64_t)col * g.C.ld) * W + g.cpart] = out;
-          else *sp = out;
+        } else {
+          fence_before();
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acc_empty[set])) : "memory");
         }
+      }
+      if (!any || !ok) continue;
+      if constexpr (KC != KC1) {
+        load_old();
+        if (!TRANS) old_ready();
+#pragma unroll
+        for (int cg = 0; cg < ECOLS / 4; ++cg) convert4(R[cg], cg * 4);
       }
       if constexpr (TRANS) {
-        asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS) : "memory");
-        if (ok)
-          for (int e2 = etid; e2 < TM * TN; e2 += 32 * EPI_WARPS) {
-            const int j = e2 % TN, r = e2 / TN;
-            const int crw = nt * TN + j, ccol = mt * TM + r;
-            if (crw < g.N && ccol < g.M)
-              Cb[((int64_t)g.crow.at(b, crw) + (int64_t)ccol * g.C.ld) * W + g.cpart] = s_c[j * TMP + r];
-          }
+        old_ready();
+        __syncwarp();
+#pragma unroll
+        for (int jj = 0; jj < ECOLS; ++jj)
+          if (live(q, jj)) q.Cp[cstep * jj] = finish(s_c[(jj * RSTEP + lane / ECOLS) * (ECOLS + 1) + lane % ECOLS], jj);
+        __syncwarp();   // read before the next tile's results overwrite it
       }
     }
-    if (!ok) {
+    if constexpr (STAGED) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok && lane == 0) {
       *abrt = 1;
       atomicOr(g.err, DEV_ERR_TIMEOUT);
     }
   }
   fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512));
 }
 
 // digit pairs (p, q), 1 <= p, q <= DIG, with p + q <= DSUM
@@ -606,9 +770,8 @@ constexpr int npairs() {
     for (int q = 1; q <= DIG; ++q) n += (p + q <= DSUM) ? 1 : 0;
   return n;
 }
-static_assert(npairs() == 55, "digit pair count");
-static_assert(DIG == 10 && BITS == 6 && FRAC == 60, "the slicing splits 60 bits into 30 + 30");
-static_assert(QGRP * TN <= 256 && (QGRP * TN) % 16 == 0, "MMA N for M = 128");
+static_assert(npairs() == 36, "digit pair count");
+static_assert(DIG == 8 && BITS == 8 && FRAC == 62, "the slicing takes the bytes of a 64-bit integer");
 
 int ceil_log2(int64_t x) {
   int c = 0;
@@ -616,12 +779,27 @@ int ceil_log2(int64_t x) {
   return c;
 }
 
-template <typename T, bool BETA0, bool TRANS>
-void set_smem_attr() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_gemm_tc<T, BETA0, TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-  });
+template <int EPI, bool TRANS, int TN, int KC>
+cudaError_t launch(const GemmP& p, int grid, cudaStream_t st) {
+  constexpr int SM = smem_bytes(TN, TRANS);
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_gemm_tc<EPI, TRANS, TN, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+  if (attr != cudaSuccess) return attr;
+  k_gemm_tc<EPI, TRANS, TN, KC><<<grid, THREADS, SM, st>>>(p);
+  return cudaGetLastError();
+}
+
+template <int EPI, bool TRANS, int TN>
+cudaError_t launch_kc(const GemmP& p, int kc, int grid, cudaStream_t st) {
+  return kc == KC1 ? launch<EPI, TRANS, TN, KC1>(p, grid, st) : launch<EPI, TRANS, TN, KC2>(p, grid, st);
+}
+
+template <int EPI, bool TRANS>
+cudaError_t launch_tn(const GemmP& p, int tn, int kc, int grid, cudaStream_t st) {
+  // the general alpha / beta form is not on the build's path: one tile shape
+  // and chunk serve it
+  if constexpr (EPI == TC_GENERAL) return launch<EPI, TRANS, 64, KC2>(p, grid, st);
+  else return tn == 64 ? launch_kc<EPI, TRANS, 64>(p, kc, grid, st) : launch_kc<EPI, TRANS, 32>(p, kc, grid, st);
 }
 
 struct Sizes {
@@ -629,15 +807,15 @@ struct Sizes {
   size_t a_item, b_item, ea_item, eb_item;
 };
 
-Sizes sizes(int M, int N, int K) {
+Sizes sizes(int M, int N, int K, int tn) {
   Sizes z;
   z.MT = (M + TM - 1) / TM;
-  z.NT = (N + TN - 1) / TN;
+  z.NT = (N + tn - 1) / tn;
   z.KT = (K + TK - 1) / TK;
   z.a_item = (size_t)z.MT * z.KT * ASTG;
-  z.b_item = (size_t)z.NT * z.KT * BSTG;
+  z.b_item = (size_t)z.NT * z.KT * bstg(tn);
   z.ea_item = (size_t)z.MT * TM * sizeof(int);
-  z.eb_item = (size_t)z.NT * TN * sizeof(int);
+  z.eb_item = (size_t)z.NT * tn * sizeof(int);
   return z;
 }
 
@@ -657,14 +835,12 @@ void tc_release(TcWorkspace* w) {
   if (w) { w->p = nullptr; w->bytes = 0; }
 }
 
-// Fraction of the 128 x 48 output tiles that holds the product, in the
-// better of the two orientations.
+// Fraction of the output tiles that holds the product, in the better of the
+// two orientations and tile widths.
 static double tile_fill(int M, int N) {
   using namespace tc;
-  const double mn = (double)M * N;
-  const double normal = (double)((M + TM - 1) / TM) * TM * ((N + TN - 1) / TN) * TN;
-  const double trans = (double)((N + TM - 1) / TM) * TM * ((M + TN - 1) / TN) * TN;
-  return mn / std::min(normal, trans);
+  auto padded = [](int n, int t) { return (double)((n + t - 1) / t) * t; };
+  return (double)M * N / std::min(padded(M, TM) * padded(N, 32), padded(N, TM) * padded(M, 32));
 }
 
 // At most 8 rows against many columns and a long inner dimension.
@@ -709,6 +885,49 @@ bool tc_applicable<cplx>(const GemmArgs<cplx>& g) {
 
 namespace {
 
+// Orientation and width of the output tiles: C = A B in 128 x TN tiles of C
+// (TN columns), or C^T = B^T A^T in 128 x TN tiles of C^T (TN of C's rows).
+struct Tiling {
+  bool trans;
+  int tn;
+};
+
+// The choice with the least estimated time: waves of tiles over the SMs (one
+// CTA each) times a tile's cycles, the largest of its digit products (measured
+// 1840 per k step at TN = 64 and 1300 at 32, where L2 delivers about 30 bytes
+// per clock to each SM; with one accumulator set, TN = 64, a third of the
+// epilogue per chunk comes on top), its epilogue (by its average number of
+// outputs) and its traffic (digits, and C at about 12 bytes per clock and SM
+// when all SMs stream: 164 x 164 x 32, 4096 items, 773 us at TN = 64 and
+// 1135 us at 32), so that few-row products (the 32-row updates of the
+// recursive LU and triangular solves) fill their tiles and small grids spread
+// over more SMs.
+Tiling choose_tiling(int M, int N, int K, int batch, bool pair) {
+  using namespace tc;
+  const int64_t sms = device_sms();
+  const double kt = (double)((K + TK - 1) / TK) * (pair ? 2 : 1);
+  Tiling best{false, 64};
+  double bt = -1.0;
+  for (int trans = 0; trans < 2; ++trans)
+    for (int tn = 64; tn >= 32; tn -= 32) {
+      const int64_t r = trans ? N : M, c = trans ? M : N;
+      const int64_t rt = (r + TM - 1) / TM, ct = (c + tn - 1) / tn;
+      const double waves = (double)((rt * ct * batch + sms - 1) / sms);
+      const double outs = (double)r * c / ((double)rt * ct);
+      const double epi = (600.0 + 0.55 * outs) * (trans ? 1.15 : 1.0);
+      const double chunks = kt * TK <= KC1 ? 1.0 : std::ceil(kt * TK / KC2);
+      const double prod = tn == 64 ? 1840.0 * kt + 0.33 * epi * chunks : 1300.0 * kt;
+      const double traffic = kt * (ASTG + bstg(tn)) / 30.0 + 16.0 * outs / 12.0;
+      const double tile = std::max(std::max(prod, epi), traffic);
+      const double t = waves * tile + prod + epi;
+      if (bt < 0.0 || t < 0.98 * bt) {
+        bt = t;
+        best = Tiling{trans != 0, tn};
+      }
+    }
+  return best;
+}
+
 cudaError_t ensure_ws(TcWorkspace* w, size_t bytes, cudaStream_t st) {
   if (w->bytes >= bytes) {
     if (w->st != st && w->p) {
@@ -735,19 +954,42 @@ cudaError_t ensure_ws(TcWorkspace* w, size_t bytes, cudaStream_t st) {
 }
 
 template <typename T>
-void launch_split(const tc::SplitSet<T>& ss, int nops, int K, int KT, int b0, int nb, cudaStream_t st, Prof* pf) {
+cudaError_t launch_split(const tc::SplitSet<T>& ss, int nops, int K, int KT, int b0, int nb, cudaStream_t st, Prof* pf) {
   int rmax = 0;
-  for (int o = 0; o < nops; ++o) rmax = std::max(rmax, ss.RT[o] * ss.TR[o]);
+  for (int o = 0; o < nops; ++o) rmax = std::max(rmax, ss.R[o]);
   if (pf) {
     pf->begin(st);
     pf->note(rmax, nops, K, nb);
   }
-  tc::k_split<T><<<dim3((rmax + 31) / 32, 1, nops * nb), 256, 0, st>>>(ss, K, KT, b0, nb);
+  // warps along k: a power of two, at most 8 and no more than units of k;
+  // CTAs of a cluster along k while the warps have several units each and
+  // the grid leaves SMs idle
+  const int nu = KT * (std::is_same<T, cplx>::value ? 2 : 1);
+  int kw = 1;
+  while (kw < 8 && kw < nu) kw *= 2;
+  const int rows = 32 * (8 / kw);
+  const int64_t ctas = (int64_t)((rmax + rows - 1) / rows) * nops * nb;
+  int cs = 1;
+  while (cs < 8 && nu > kw * cs && ctas * cs < 4 * device_sms()) cs *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((rmax + rows - 1) / rows * cs, nops, nb);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cs > 1 ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, tc::k_split<T>, ss, K, KT, b0, kw, cs);
   if (pf) pf->end(K_SPLIT, 0.0, st);
+  return e;
 }
 
-template <typename T>
-void launch_mma(const tc::GemmP<T>& p, bool trans, int nb, int M, int N, int K, cudaStream_t st, Prof* pf) {
+cudaError_t launch_mma(const tc::GemmP& p, const Tiling& tl, int kc, int nb, int M, int N, int K, cudaStream_t st,
+                       Prof* pf) {
+  using namespace tc;
   if (pf) {
     pf->begin(st);
     pf->note(M, N, K, nb);
@@ -757,22 +999,19 @@ void launch_mma(const tc::GemmP<T>& p, bool trans, int nb, int M, int N, int K, 
   // one CTA per tile
   const int64_t ntiles = (int64_t)p.MT * p.NT * nb;
   const bool persist = K >= lu_tune(TUNE_TC_PERSIST_MIN_K);
-  dim3 grid((unsigned)(persist ? std::min<int64_t>(ntiles, device_sms()) : ntiles));
-  auto go = [&](auto beta0, auto trans) {
-    constexpr bool B0 = decltype(beta0)::value, TR = decltype(trans)::value;
-    tc::set_smem_attr<T, B0, TR>();
-    tc::k_gemm_tc<T, B0, TR><<<grid, tc::THREADS, tc::SMEM, st>>>(p);
-  };
-  using t_ = std::true_type;
-  using f_ = std::false_type;
-  if (p.beta == 0.0) { if (trans) go(t_(), t_()); else go(t_(), f_()); }
-  else { if (trans) go(f_(), t_()); else go(f_(), f_()); }
-  // executed: bf16 tensor-core flops of the digit products over the padded
+  const int grid = (int)(persist ? std::min<int64_t>(ntiles, device_sms()) : ntiles);
+  const bool unit = p.alpha == 1.0 || p.alpha == -1.0;
+  const int epi = unit && p.beta == 0.0 ? TC_SET : unit && p.beta == 1.0 ? TC_ADD : TC_GENERAL;
+  cudaError_t e;
+  if (epi == TC_SET) e = tl.trans ? launch_tn<TC_SET, true>(p, tl.tn, kc, grid, st) : launch_tn<TC_SET, false>(p, tl.tn, kc, grid, st);
+  else if (epi == TC_ADD) e = tl.trans ? launch_tn<TC_ADD, true>(p, tl.tn, kc, grid, st) : launch_tn<TC_ADD, false>(p, tl.tn, kc, grid, st);
+  else e = tl.trans ? launch_tn<TC_GENERAL, true>(p, 64, KC2, grid, st) : launch_tn<TC_GENERAL, false>(p, 64, KC2, grid, st);
+  // executed: fp16 tensor-core flops of the digit products over the padded
   // tiles; algorithmic: 2 M N K per real product (a pair holds two)
-  const double npairs = tc::npairs();
   const double nprod = p.pair ? 2.0 : 1.0;
-  const double exec = 2.0 * npairs * nprod * (double)p.MT * tc::TM * (double)p.NT * tc::TN * (double)p.KT * tc::TK * nb;
+  const double exec = 2.0 * npairs() * nprod * (double)p.MT * TM * (double)p.NT * tl.tn * (double)p.KT * TK * nb;
   if (pf) pf->end(K_GEMM_TC, 2.0 * nprod * M * (double)N * K * nb, st, exec);
+  return e;
 }
 
 }  // namespace
@@ -786,32 +1025,21 @@ bool shared_operand(const BOp<T>& X, const IMap& r, const IMap& k) {
          (!k.idx || k.period == 1);
 }
 
-// Orientation of the output tiles: C = A B in 128 x 48 tiles of C, or
-// C^T = B^T A^T in 128 x 48 tiles of C^T (48-row tiles of C), the latter
-// when it takes a quarter fewer waves of tiles over the SMs -- a product with few rows (the
-// 32-row updates of the recursive LU and triangular solves, M = 32..64)
-// wastes most of a 128-row tile but fits a 48-column one; a grid that fits
-// in one wave either way stays in the normal form.
-static bool tc_transposed(int M, int N, int batch) {
-  using namespace tc;
-  const int64_t sms = device_sms();
-  const int64_t normal = (int64_t)((M + TM - 1) / TM) * ((N + TN - 1) / TN) * batch;
-  const int64_t trans = (int64_t)((N + TM - 1) / TM) * ((M + TN - 1) / TN) * batch;
-  // one CTA per SM: the time goes with the number of waves of tiles; the
-  // transposed epilogue (staged through shared memory) costs more per tile,
-  // so it has to save at least a quarter of the waves
-  return 4 * ((trans + sms - 1) / sms) <= 3 * ((normal + sms - 1) / sms);
-}
-
 template <typename T>
 cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
   using namespace tc;
   constexpr int NP = std::is_same<T, cplx>::value ? 2 : 1;
   TcWorkspace* w = tc_workspace();
-  const bool tr = tc_transposed(g.M, g.N, g.batch);
-  // rows of the A slot (the 128-row tiles) and of the B slot (48-row tiles)
+  double alpha, beta;
+  if constexpr (NP == 2) { alpha = g.alpha.re; beta = g.beta.re; }
+  else { alpha = g.alpha; beta = g.beta; }
+  Tiling tl = choose_tiling(g.M, g.N, g.K, g.batch, NP == 2);
+  const bool general = (alpha != 1.0 && alpha != -1.0) || (beta != 0.0 && beta != 1.0);
+  if (general) tl.tn = 64;   // the general form's tiles
+  const bool tr = tl.trans;
+  // rows of the A slot (the 128-row tiles) and of the B slot (TN-row tiles)
   const int Ma = tr ? g.N : g.M, Nb = tr ? g.M : g.N;
-  const Sizes z = sizes(Ma, Nb, g.K);
+  const Sizes z = sizes(Ma, Nb, g.K, tl.tn);
   const bool shA = g.batch > 1 && shared_operand(g.A, g.arow, g.acol);
   const bool shB = g.batch > 1 && shared_operand(g.B, g.brow, IMap());
   const bool shSa = tr ? shB : shA, shSb = tr ? shA : shB;   // per slot
@@ -842,11 +1070,12 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     ea = reinterpret_cast<int*>(q); q += z.ea_item * na;
     eb = reinterpret_cast<int*>(q); q += z.eb_item * nbb;
   }
-  // fixed-point fraction bits: a complex component sums 2K products
-  const int lsb = 62 - ceil_log2(std::max(NP * g.K, 1));
-  double alpha, beta;
-  if constexpr (NP == 2) { alpha = g.alpha.re; beta = g.beta.re; }
-  else { alpha = g.alpha; beta = g.beta; }
+  // chunk and fixed-point fraction bits, by the products summed per output (a
+  // complex component sums 2K): scaled entries stay below 1 - 2^-54, so the
+  // sum below 2^63 units with room for the chunks' roundings up to 2^17 terms
+  const int ksum = NP * z.KT * TK;
+  const int kc = ksum <= KC1 && !general ? KC1 : KC2;
+  const int lsb = kc == KC1 ? LSB1 : ksum <= KC2 ? LSB2 : (ksum <= 1 << 17 ? 63 : 62) - ceil_log2(ksum);
   for (int b0 = 0; b0 < g.batch; b0 += nb_max) {
     const int nb = std::min(nb_max, g.batch - b0);
     SplitSet<T> ss;
@@ -855,29 +1084,32 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     sa.X = g.A; sa.rmap = g.arow; sa.kmap = g.acol; sa.rs = 1; sa.ks = g.A.ld;
     Src<T> sb;
     sb.X = g.B; sb.kmap = g.brow; sb.rs = g.B.ld; sb.ks = 1;
-    ss.s[0] = tr ? sb : sa; ss.R[0] = Ma; ss.TR[0] = TM; ss.RT[0] = z.MT;
+    ss.s[0] = tr ? sb : sa; ss.R[0] = Ma; ss.ltr[0] = 7; ss.RT[0] = z.MT;
     ss.out[0] = As[0]; ss.out2[0] = As[1]; ss.ex[0] = ea;
     ss.items[0] = (shSa && b0 > 0) ? 0 : (shSa ? 1 : nb);  // a shared operand is cut once per call
-    ss.s[1] = tr ? sa : sb; ss.R[1] = Nb; ss.TR[1] = TN; ss.RT[1] = z.NT;
+    ss.s[1] = tr ? sa : sb; ss.R[1] = Nb; ss.ltr[1] = tl.tn == 64 ? 6 : 5; ss.RT[1] = z.NT;
     ss.out[1] = Bs[0]; ss.out2[1] = Bs[1]; ss.ex[1] = eb;
     ss.items[1] = (shSb && b0 > 0) ? 0 : (shSb ? 1 : nb);
-    launch_split<T>(ss, 2, g.K, z.KT, b0, nb, st, pf);
-    GemmP<T> p;
+    if ((e = launch_split<T>(ss, 2, g.K, z.KT, b0, nb, st, pf)) != cudaSuccess) return e;
+    GemmP p;
     p.MT = z.MT; p.NT = z.NT; p.KT = z.KT; p.M = Ma; p.N = Nb; p.lsb = lsb;
-    p.C = g.C; p.crow = g.crow; p.b0 = b0; p.err = *w->err_slot;
+    p.crow = g.crow; p.b0 = b0; p.err = *w->err_slot;
+    p.W = NP;
+    p.C.ptrs = reinterpret_cast<double* const*>(g.C.ptrs);
+    p.C.base = reinterpret_cast<double*>(g.C.base);
+    p.C.stride = NP * g.C.stride; p.C.sub = NP * g.C.sub; p.C.off = NP * g.C.off;
+    p.C.ld = g.C.ld; p.C.div = g.C.div;
     p.a_bl = shSa ? 0 : 1;
     p.b_bl = shSb ? 0 : 1;
     p.nitems = nb;
     p.ea = ea; p.eb = eb;
     p.alpha = alpha;
     p.beta = beta;
-    p.amode = (alpha == 1.0 || alpha == -1.0) ? 1 : 0;
     p.asign = alpha == -1.0 ? (long long)(1ull << 63) : 0ll;
     if constexpr (NP == 1) {
       p.As = As[0]; p.Bs = Bs[0];
       p.As2 = nullptr; p.Bs2 = nullptr; p.pair = 0; p.neg2 = 0;
-      p.cpart = 0;
-      launch_mma<T>(p, tr, nb, g.M, g.N, g.K, st, pf);
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
     } else {
       // complex (real alpha, beta), each component one launch of two
       // products into the same accumulators:
@@ -893,13 +1125,12 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
       slots(0, 0, p.As, p.Bs);
       slots(1, 1, p.As2, p.Bs2);
       p.neg2 = 1;
-      p.cpart = 0;
-      launch_mma<T>(p, tr, nb, g.M, g.N, g.K, st, pf);
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
       slots(0, 1, p.As, p.Bs);
       slots(1, 0, p.As2, p.Bs2);
       p.neg2 = 0;
-      p.cpart = 1;
-      launch_mma<T>(p, tr, nb, g.M, g.N, g.K, st, pf);
+      p.C.off += 1;   // the imaginary component
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
     }
   }
   return cudaGetLastError();

@@ -1012,6 +1012,381 @@ int panel_cluster_size(int rows, int nb, int batch) {
   return cs <= mx ? cs : 0;
 }
 
+// Panel LU with the panel's rows in registers.
+//
+// The rows [k0, n) are split into CS contiguous chunks of at most 512, one per
+// CTA of the matrix's cluster (CS = 1: a plain CTA).  A row belongs to CT
+// threads of different warps, thread q holding its columns q, q + CT, ... :
+// one thread per row when the chunk has a warp of rows for each of the SM's
+// four schedulers, two or four when it has fewer.  Every step works on the
+// registers' front column: the owners' update writes one register down, so
+// that one loop body serves a whole segment of steps (the width shrinks by a
+// segment at a time: at most 10 % of the multiply-adds are spent on columns
+// already left behind).  Rows never move during the panel: a chosen row only
+// leaves the search, the interchanges are recorded in LAPACK's form (ipiv) by
+// a replay of the swap sequence on the panel's top positions (every warp keeps
+// its own copy in registers, lane t for position k0 + t), the finished entries
+// of L and U collect in shared memory, and at the end every row is written to
+// its final position.
+//
+// Per column: each warp of the column's owners finds its candidate (largest
+// magnitude, and on ties the lowest current position -- the row order after
+// the interchanges so far, which is LAPACK's choice) with warp-wide integer
+// maxima of the magnitude's two words; after one block barrier every warp
+// knows the CTA's candidate; the warps that hold it push its key and values
+// into the shared memory of every CTA of the cluster, and its reciprocal as
+// soon as it is formed, with stores that count their bytes on the receiver's
+// mbarriers (bounded waits); every warp then picks the same pivot from its own
+// shared memory.  Candidates are double-buffered by column parity: a CTA
+// pushes into a slot again only two columns later, after receiving the
+// candidates that every CTA sends once it has finished with the slot.
+//
+// What bounds it: the chain from one pivot to the next.  The FP64 pipe takes
+// 64 cycles per warp instruction and scheduler; a division is ~440 cycles, the
+// exchange ~700, the searches ~400, the update of 432 rows on 16 CTAs ~460.
+// Measured, 32 columns of one matrix: 432 rows 100 -> 46 us, 1728 rows 110 ->
+// 64 us, 6720 rows 176 -> 113 us (FP64 update ~3900 of 6700 cycles a column);
+// 16 complex columns of 1696 rows 75 -> 53 us.  The earlier form kept the rows
+// in shared memory, where each multiply-add waited for the store before it,
+// and took two cluster-wide barriers' time per column.
+template <typename T> struct LuNB;
+template <> struct LuNB<double> { enum { NB = 32 }; };
+template <> struct LuNB<cplx> { enum { NB = 16 }; };
+
+// Largest key (hi, lo) over the warp's lanes, lowest position on ties; hi = 0
+// means no candidate.  Returns the lane that holds it.
+__device__ __forceinline__ int warp_pivot(uint32_t& hi, uint32_t& lo, uint32_t& pos) {
+  const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
+  const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  const bool in = hi == mh && lo == ml;
+  const uint32_t mp = __reduce_min_sync(0xffffffffu, in ? pos : 0xffffffffu);
+  const int src = __ffs((int)__ballot_sync(0xffffffffu, in && pos == mp)) - 1;
+  hi = mh;
+  lo = ml;
+  pos = mp;
+  return src;
+}
+
+// Store to another CTA's shared memory (cluster addresses) that adds its bytes
+// to that CTA's mbarrier when it lands.
+__device__ __forceinline__ void st_async(uint32_t dst, double v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+               "l"(__double_as_longlong(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async(uint32_t dst, cplx v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+               "l"(__double_as_longlong(v.re)), "l"(__double_as_longlong(v.im)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async(uint32_t dst, uint4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst),
+               "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t peer_addr(uint32_t local, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+// bounded wait for a phase whose bytes come from the cluster's CTAs
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, int parity) {
+  for (int it = 0; it < (1 << 22); ++it) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+    if (ok) return true;
+    if (it > 1024) __nanosleep(64);
+  }
+  return false;
+}
+
+template <typename T, bool CL, int CT>
+struct PanelReg {
+  enum { NB = LuNB<T>::NB, SEG = 4, NQ = NB / CT };
+  T* Ps;          // finished entries, column-major, ld rows
+  T* cv;          // [2 slots][CS][NB] candidate rows (lay)
+  T* cinv;        // [2][CS] reciprocals of their pivot entries
+  uint4* crec;    // [2][CS] their keys: magnitude hi + 1, lo, position, row
+  uint64_t* bar;  // [2] keys and rows of a slot have arrived, [2] reciprocals
+  uint4* wrec;    // [RW] this CTA's warps' candidates
+  T* srow;        // [NB + 1] the CTA candidate's row and reciprocal (3 more are read past a row's end)
+  unsigned* err;
+  int CS, g, k0, nb, r0, ld, RW;
+  int lane, rw, q;   // row warp, column group
+  int row;        // row of the chunk
+  int phys, pos;  // row now at position k0 + lane; position of row k0 + lane
+  int chosen;     // step at which this thread's row became the pivot, or -1
+  bool done;      // row absent or chosen
+  T a[NQ];        // columns q, q + CT, ... of the row; a[0] is the first not finished (beyond the panel, and of a done row: unused)
+
+  // place of column jj + r in a candidate row of step jj: each group's columns together
+  static __device__ __forceinline__ int lay(int r) { return CT == 1 ? r : (r & (CT - 1)) * NQ + r / CT; }
+
+  // step jj on registers of WIDTH / CT columns each (jj .. of the segment)
+  template <int WIDTH>
+  __device__ __forceinline__ void step(int jj, int* ip, int* info_b) {
+    constexpr int WQ = WIDTH / CT;
+    const int slot = jj & 1;
+    const int pr = r0 + row;
+    const bool own = CT == 1 || q == (jj & (CT - 1));   // this group holds column jj
+    const int o = CT == 1 ? 0 : (q - jj) & (CT - 1), f = jj + o;   // panel column of a[0]
+    const int ptop = __shfl_sync(0xffffffffu, pos, (pr - k0) & 31);
+    if (CL && threadIdx.x == 0) {
+      mbar_expect(bar + slot, (uint32_t)(CS * ((NB - jj) * (int)sizeof(T) + 16)));
+      mbar_expect(bar + 2 + slot, (uint32_t)(CS * (int)sizeof(T)));
+    }
+    if (own) {
+      const unsigned long long mb = (unsigned long long)__double_as_longlong(mag1(a[0]));
+      uint32_t hi = done ? 0u : (uint32_t)(mb >> 32) + 1u, lo = done ? 0u : (uint32_t)mb;
+      uint32_t ps = (uint32_t)(pr - k0 < nb ? ptop : pr);
+      const int src = warp_pivot(hi, lo, ps);
+      if (lane == src) wrec[rw] = make_uint4(hi, lo, ps, (uint32_t)pr);
+    }
+    __syncthreads();
+    uint4 rec = wrec[RW > 1 && lane < RW ? lane : 0];
+    int w = 0;
+    if (RW > 1) {
+      if (lane >= RW) rec = make_uint4(0u, 0u, 0xffffffffu, 0u);
+      w = warp_pivot(rec.x, rec.y, rec.z);
+      rec.w = __shfl_sync(0xffffffffu, rec.w, w);
+    }
+    if (rw == w) {   // the warps that hold the CTA's candidate row
+      if (pr == (int)rec.w) {
+#pragma unroll
+        for (int i = 0; i < WQ; ++i) srow[o * NQ + i] = a[i];
+      }
+      if constexpr (CL) {
+        __syncwarp();
+        const int i = lane & (NQ - 1);
+        if (f + i * CT < NB) {
+          const T v = srow[o * NQ + i];
+          const uint32_t dv = smem_addr(cv + (slot * CS + g) * NB + o * NQ + i), db = smem_addr(bar + slot);
+          for (int d = lane / NQ; d < CS; d += 32 / NQ) st_async(peer_addr(dv, d), v, peer_addr(db, d));
+        }
+        if (own && lane < CS)
+          st_async(peer_addr(smem_addr(crec + slot * CS + g), lane), rec, peer_addr(smem_addr(bar + slot), lane));
+      }
+      if (own) {
+        if (pr == (int)rec.w) srow[NB] = (rec.x <= 1u && rec.y == 0u) ? T(0.0) : recip(a[0]);
+        if constexpr (CL) {
+          __syncwarp();
+          if (lane < CS)
+            st_async(peer_addr(smem_addr(cinv + slot * CS + g), lane), srow[NB],
+                     peer_addr(smem_addr(bar + 2 + slot), lane));
+        }
+      }
+    }
+    T inv;
+    const T* Wv;
+    int prow, pq;
+    bool zero;
+    if constexpr (CL) {
+      const int par = (jj >> 1) & 1;
+      bool ok = mbar_wait_cluster(bar + slot, par);
+      uint4 c = lane < CS ? crec[slot * CS + lane] : make_uint4(0u, 0u, 0xffffffffu, 0u);
+      const int pw = warp_pivot(c.x, c.y, c.z);
+      prow = (int)__shfl_sync(0xffffffffu, c.w, pw);
+      pq = (int)c.z;
+      zero = c.x <= 1u && c.y == 0u;
+      Wv = cv + (slot * CS + pw) * NB;
+      ok = mbar_wait_cluster(bar + 2 + slot, par) && ok;
+      if (!ok) atomicOr(err, DEV_ERR_TIMEOUT);
+      inv = cinv[slot * CS + pw];
+    } else {
+      prow = (int)rec.w;
+      pq = (int)rec.z;
+      zero = rec.x <= 1u && rec.y == 0u;
+      __syncthreads();
+      Wv = srow;
+      inv = srow[NB];
+    }
+    if (pr == prow) {
+      done = true;
+      chosen = jj;
+    }
+    T l = T(0.0);
+    if (own) {
+      l = a[0] * inv;
+      if (!done) Ps[jj * ld + row] = l;
+    }
+    if constexpr (CT > 1) {
+      __syncthreads();
+      if (!own) l = Ps[jj * ld + row];
+    }
+    // the remaining columns; the owners' move one register down.  The pivot
+    // row is read eight values ahead: a load right before its multiply-add
+    // would show its latency (113 instead of 64 cycles each)
+    {
+      const T* Wq = Wv + o * NQ;
+      constexpr int BW = 8;
+#pragma unroll
+      for (int i0 = 0; i0 < WQ; i0 += BW) {
+        T w[BW];
+#pragma unroll
+        for (int i = 0; i < BW && i0 + i < WQ; ++i) w[i] = Wq[i0 + i];
+        if (own) {
+#pragma unroll
+          for (int i = (i0 == 0 ? 1 : 0); i < BW && i0 + i < WQ; ++i) a[i0 + i - 1] = fmsc(a[i0 + i], l, w[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < BW && i0 + i < WQ; ++i) a[i0 + i] = fmsc(a[i0 + i], l, w[i]);
+        }
+      }
+      if (own) a[WQ - 1] = T(0.0);
+    }
+    // the pivot row's entries of U
+    if (q == 0 && (unsigned)(prow - r0 - rw * 32) < 32u)
+      for (int r = lane; jj + r < nb; r += 32) Ps[(jj + r) * ld + prow - r0] = Wv[lay(r)];
+    // LAPACK interchange: position j <-> the winner's current position
+    const int j = k0 + jj;
+    {
+      const int rj = __shfl_sync(0xffffffffu, phys, jj);
+      if (lane == rj - k0) pos = pq;
+      if (pq - k0 < nb && lane == pq - k0) phys = rj;
+      if (lane == jj) phys = prow;
+      if (prow - k0 < nb && lane == prow - k0) pos = j;
+    }
+    if (g == 0 && threadIdx.x == 0) {
+      ip[j] = pq;
+      if (zero && *info_b == 0) *info_b = j + 1;
+    }
+  }
+
+  template <int WIDTH>
+  __device__ __forceinline__ void run(int jj, int* ip, int* info_b) {
+    for (int e = min(jj + (int)SEG, nb); jj < e; ++jj) step<WIDTH>(jj, ip, info_b);
+    if constexpr (WIDTH > SEG) {
+      if (jj < nb) run<WIDTH - SEG>(jj, ip, info_b);
+    }
+  }
+};
+
+template <typename T, bool CL, int CT>
+__global__ void __launch_bounds__(512) k_lu_panel_reg(BOp<T> A, int n, int k0, int nb, int CS, int* ipiv, int* info,
+                                                      unsigned* err) {
+  namespace cg = cooperative_groups;
+  constexpr int NB = LuNB<T>::NB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint4 wrec[16];
+  __shared__ uint4 crec[2 * 16];
+  __shared__ __align__(8) uint64_t bars[4];
+  PanelReg<T, CL, CT> p;
+  p.CS = CL ? CS : 1;
+  p.g = CL ? (int)cg::this_cluster().block_rank() : 0;
+  const int b = blockIdx.x / p.CS;
+  const int rows = n - k0, ch = (rows + p.CS - 1) / p.CS;
+  p.k0 = k0;
+  p.nb = nb;
+  p.r0 = k0 + p.g * ch;
+  const int rc = max(0, min(ch, n - p.r0));
+  p.RW = blockDim.x / (32 * CT);
+  p.ld = p.RW * 32;
+  p.Ps = reinterpret_cast<T*>(smem_raw);
+  p.cv = p.Ps + (size_t)NB * p.ld;
+  p.cinv = p.cv + 2 * p.CS * NB;
+  p.srow = p.cinv + 2 * p.CS;
+  p.wrec = wrec;
+  p.crec = crec;
+  p.bar = bars;
+  p.err = err;
+  p.lane = threadIdx.x & 31;
+  p.rw = CT == 1 ? threadIdx.x >> 5 : (threadIdx.x >> 5) % p.RW;
+  p.q = CT == 1 ? 0 : (threadIdx.x >> 5) / p.RW;
+  p.row = p.rw * 32 + p.lane;
+  p.phys = p.pos = k0 + p.lane;
+  p.chosen = -1;
+  p.done = p.row >= rc;
+  T* Ab = A.item(b);
+  const int64_t lda = A.ld;
+  const T* src = Ab + (p.r0 + p.row) + (int64_t)k0 * lda;
+#pragma unroll
+  for (int i = 0; i < NB / CT; ++i)
+    p.a[i] = (!p.done && p.q + i * CT < nb) ? src[(p.q + i * CT) * lda] : T(0.0);
+  if constexpr (CL) {
+    if (threadIdx.x == 0) {
+      for (int i = 0; i < 4; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bars + i)));
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cg::this_cluster().sync();   // every CTA has started before any writes into its shared memory
+  }
+  p.template run<NB>(0, ipiv + (int64_t)b * n, info + b);
+  if constexpr (CL) cg::this_cluster().sync();   // every CTA has read its rows and its candidates
+  else __syncthreads();
+  // rows to their final positions
+  const int pr = p.r0 + p.row;
+  const int ptop = __shfl_sync(0xffffffffu, p.pos, (pr - k0) & 31);
+  if (p.row >= rc) return;
+  const int dst = p.chosen >= 0 ? k0 + p.chosen : pr - k0 < nb ? ptop : pr;
+  T* out = Ab + dst + (int64_t)k0 * lda;
+  for (int c = p.q; c < nb; c += CT) out[c * lda] = p.Ps[c * p.ld + p.row];
+}
+
+// CTAs per matrix for a panel of `rows` rows of `batch` matrices: a power of
+// two, enough for at most 512 rows each, then more while a CTA would hold more
+// than 32 and the clusters of all matrices still fit on the SMs at once (the
+// update shrinks with the rows; measured 32 / 64 / 128 rows a CTA: adaptive
+// build 17.5 / 19.0 / 19.8 ms of panels); 0 when even the largest cluster is
+// too small.
+template <typename T>
+size_t panel_reg_smem(int ld, int cs) {
+  return ((size_t)LuNB<T>::NB * ld + 2 * (size_t)cs * (LuNB<T>::NB + 1) + LuNB<T>::NB + 4) * sizeof(T);
+}
+
+template <typename T, int CT>
+bool panel_reg_attr(size_t sm) {
+  return cudaFuncSetAttribute(k_lu_panel_reg<T, false, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
+         cudaFuncSetAttribute(k_lu_panel_reg<T, true, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
+         cudaFuncSetAttribute(k_lu_panel_reg<T, true, CT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+}
+
+template <typename T>
+int panel_reg_max() {
+  static const int mx = [] {
+    const size_t sm = panel_reg_smem<T>(512, 16);
+    if (!panel_reg_attr<T, 1>(sm) || !panel_reg_attr<T, 2>(sm) || !panel_reg_attr<T, 4>(sm)) {
+      cudaGetLastError();
+      return 0;
+    }
+    for (int cs = 16; cs >= 2; cs /= 2) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(cs);
+      cfg.blockDim = dim3(512);
+      cfg.dynamicSmemBytes = sm;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = cs;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int ncl = 0;
+      if (cudaOccupancyMaxActiveClusters(&ncl, (void*)k_lu_panel_reg<T, true, 1>, &cfg) == cudaSuccess && ncl > 0) return cs;
+      cudaGetLastError();
+    }
+    return 1;
+  }();
+  return mx;
+}
+
+template <typename T>
+int panel_reg_size(int rows, int batch) {
+  const int mx = panel_reg_max<T>();
+  if (mx < 1) return 0;
+  int cs = 1;
+  while (cs <= mx && (rows + cs - 1) / cs > 512) cs *= 2;
+  if (cs > mx) return 0;
+  while (cs < mx && (rows + cs - 1) / cs > 32 && (int64_t)batch * cs * 2 <= device_sms()) cs *= 2;
+  return cs;
+}
+
+template <typename T, int CT>
+cudaError_t launch_panel_reg(const cudaLaunchConfig_t& cfg, int cs, BOp<T> A, int n, int k0, int nb, int* ipiv, int* info, unsigned* err) {
+  return cs > 1 ? cudaLaunchKernelEx(&cfg, k_lu_panel_reg<T, true, CT>, A, n, k0, nb, cs, ipiv, info, err)
+                : cudaLaunchKernelEx(&cfg, k_lu_panel_reg<T, false, CT>, A, n, k0, nb, cs, ipiv, info, err);
+}
+
 // Apply the panel's interchanges to every column outside the panel and
 // solve U12 = L11^{-1} A12 for the columns in [k0 + nb, trsm_end).
 //
@@ -1141,10 +1516,6 @@ int& lu_tune(int param) {
   return v[param];
 }
 
-template <typename T> struct LuNB;
-template <> struct LuNB<double> { enum { NB = 32 }; };
-template <> struct LuNB<cplx> { enum { NB = 16 }; };
-
 template <typename T>
 int lu_group_size(int n, int batch, int num_sms) {
   const int nb = LuNB<T>::NB;
@@ -1211,12 +1582,34 @@ static cudaError_t lu_leaf(BOp<T> A, int n, int k0, int nb, int trsm_end, int ba
     pfl += below * (nb - jj - 1) + below;
   }
   pfl *= F * batch;
-  const int CS = (Gk > 1 && lu_tune(TUNE_LU_CLUSTER_PANEL)) ? panel_cluster_size<T>(rows, nb, batch) : 0;
+  // one row per thread (CR CTAs a matrix) up to 512 rows a CTA; taller panels
+  // in a cluster's shared memory (CS) or a cooperative group
+  const int CR = lu_tune(TUNE_LU_CLUSTER_PANEL) ? panel_reg_size<T>(rows, batch) : 0;
+  const int CS = (CR == 0 && Gk > 1 && lu_tune(TUNE_LU_CLUSTER_PANEL)) ? panel_cluster_size<T>(rows, nb, batch) : 0;
   if (pf) {
     pf->begin(st);
-    pf->note(rows, nb, CS > 1 ? CS : Gk, batch);  // k: CTAs per matrix
+    pf->note(rows, nb, CR > 0 ? CR : CS > 1 ? CS : Gk, batch);  // k: CTAs per matrix
   }
-  if (CS > 1) {
+  if (CR > 0) {
+    const int rw = ((rows + CR - 1) / CR + 31) / 32;   // row warps
+    const int ct = rw == 1 ? 4 : rw == 2 ? 2 : 1;      // column groups: a warp for every scheduler
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(batch * CR);
+    cfg.blockDim = dim3(32 * rw * ct);
+    cfg.dynamicSmemBytes = panel_reg_smem<T>(32 * rw, CR);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CR;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CR > 1 ? 1 : 0;
+    e = ct == 4 ? launch_panel_reg<T, 4>(cfg, CR, A, n, k0, nb, ipiv, info, dev_err)
+        : ct == 2 ? launch_panel_reg<T, 2>(cfg, CR, A, n, k0, nb, ipiv, info, dev_err)
+                  : launch_panel_reg<T, 1>(cfg, CR, A, n, k0, nb, ipiv, info, dev_err);
+    if (e != cudaSuccess) return e;
+  } else if (CS > 1) {
     // the panel in the distributed shared memory of a cluster per matrix
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch * CS);

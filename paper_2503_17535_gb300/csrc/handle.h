@@ -35,6 +35,7 @@ struct LevelDev {
   void* X = nullptr;    // [nmerge][n_int x (n_ext+1)]  D^{-1} [C | h_int]
   int G = 1;
   LuWork luw;
+  TrsvInv inv;          // diagonal-block inverses of D's (W's) factors, when few matrices
   bool lazy = false;    // root only: X holds [C | h_int]; D^{-1} is applied per solve
   // adjoint B^H products of DtN levels, in two passes over the children of
   // even / odd popcount (children sharing an interface differ in one bit, so
@@ -70,6 +71,7 @@ struct ItiElim {
   cplx* S = nullptr;                       // [leaf] no x no (LU)
   int *ipivS = nullptr, *permS = nullptr;
   LuWork luw, luwS;
+  TrsvInv inv, invS;
   int G = 1, GS = 1;
   int cap = 0;                             // columns the workspace holds
   double *z = nullptr, *z2 = nullptr, *t = nullptr;
@@ -82,6 +84,7 @@ struct AGroup {
   int level = 0, n_int = 0, n_ext = 0, G = 1;
   std::vector<int> members;      // indices into hps_handle::am
   LuWork luw;
+  TrsvInv inv;
   int *ipiv = nullptr, *perm = nullptr, *info = nullptr;  // [members][n_int], [members]
   double **dD = nullptr, **dX = nullptr, **dR = nullptr;  // build operands
   double **dTP = nullptr;                                 // parents' [T | h]
@@ -158,6 +161,7 @@ struct hps_handle {
   void* leafX = nullptr;  // DtN: X = L_ii^{-1}[L_ie P | -f_i]; ItI: [Y | v]
   void* leafTH = nullptr; // [T | h]
   LuWork leaf_luw;
+  hps::TrsvInv leaf_inv;
   int leaf_G = 1;
   std::vector<LevelDev> lev;
   unsigned* dev_err = nullptr;
@@ -299,6 +303,16 @@ inline bool is_device_ptr(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Storage for the diagonal-block inverses of `batch` factors of order n when
+// their solves want them; false: out of memory.
+template <typename T>
+bool alloc_inv(hps_handle* h, int n, int64_t batch, TrsvInv* inv) {
+  if (!trsv_cluster_wanted(n, batch)) return true;
+  inv->p = dalloc(h, (size_t)trsv_inv_elems(n, batch) * sizeof(T));
+  inv->ready = false;
+  return inv->p != nullptr;
 }
 
 template <typename T> struct Kind;

@@ -215,6 +215,7 @@ hps_status adaptive_build(hps_handle* h, const hps_tree* tree, const hps_coeffs*
     HPS_CUDA(cudaMemsetAsync(h->leaf_luw.bars, 0, sizeof(unsigned) * 2 * nl, st));
   }
   BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)ni * ni, ni);
+  if (!alloc_inv<T>(h, ni, nl, &h->leaf_inv)) return HPS_ERR_OOM;
   HPS_CUDA(getrf<T>(LA, ni, (int)nl, h->leaf_ipiv, h->leaf_perm, h->leaf_info, h->dev_err, h->leaf_G, h->leaf_luw,
                     st, pf));
   BOp<T> LX = bop<T>((T*)h->leafX, (int64_t)ni * (nb + 1), ni);
@@ -407,28 +408,34 @@ hps_status adaptive_build(hps_handle* h, const hps_tree* tree, const hps_coeffs*
         if (!A.luw.bars || !A.luw.pub) return HPS_ERR_OOM;
         HPS_CUDA(cudaMemsetAsync(A.luw.bars, 0, sizeof(unsigned) * 2 * nbat, st));
       }
+      const bool lazy = nbat == 1 && h->am[(size_t)A.members[0]].node == 0 && h->opts.lazy_root && !h->opts.want_root_map;
+      const bool by_flags = lazy && trsv_flags_preferred(nI);
+      if (!by_flags && !alloc_inv<T>(h, nI, nbat, &A.inv)) return HPS_ERR_OOM;
       BOp<T> DD = bopp<T>(A.dD, nI);
       BOp<T> XX = bopp<T>(A.dX, nI);
       HPS_CUDA(getrf<T>(DD, nI, nbat, A.ipiv, A.perm, A.info, h->dev_err, A.G, A.luw, st, pf));
       AMergeDev& M0 = h->am[(size_t)A.members[0]];
-      if (nbat == 1 && M0.node == 0 && h->opts.lazy_root && !h->opts.want_root_map) {
+      if (lazy) {
         // lazy root: keep [C | h_int] (in X's storage) and D's factors
         M0.lazy = true;
         HPS_CUDA(cudaMemcpyAsync(M0.X, Rof[(size_t)A.members[0]], (size_t)nI * (ne + 1) * sizeof(T),
                                  cudaMemcpyDeviceToDevice, st));
-        const int nf = (nI + 31) / 32;
-        h->trsv.flags = (unsigned*)dalloc(h, (size_t)nf * sizeof(unsigned));
-        h->trsv.dinv = dalloc(h, (size_t)2 * nf * 1024 * sizeof(T));
-        h->trsv.dinv_ready = false;
-        if (!h->trsv.flags || !h->trsv.dinv) return HPS_ERR_OOM;
-        HPS_CUDA(cudaMemsetAsync(h->trsv.flags, 0, (size_t)nf * sizeof(unsigned), st));
-        h->trsv.nflags = nf;
-        HPS_CUDA(cudaHostAlloc((void**)&h->trsv_err_host, sizeof(int), cudaHostAllocMapped));
-        *h->trsv_err_host = 0;
-        int* dp = nullptr;
-        HPS_CUDA(cudaHostGetDevicePointer((void**)&dp, h->trsv_err_host, 0));
-        h->trsv.host_err = h->trsv_err_host;
-        h->trsv.dev_err = dp;
+        if (by_flags) {
+          // a large root: flags and a host-mapped error word for the flag-ordered solves
+          const int nf = (nI + 31) / 32;
+          h->trsv.flags = (unsigned*)dalloc(h, (size_t)nf * sizeof(unsigned));
+          h->trsv.dinv = dalloc(h, (size_t)2 * nf * 1024 * sizeof(T));
+          h->trsv.dinv_ready = false;
+          if (!h->trsv.flags || !h->trsv.dinv) return HPS_ERR_OOM;
+          HPS_CUDA(cudaMemsetAsync(h->trsv.flags, 0, (size_t)nf * sizeof(unsigned), st));
+          h->trsv.nflags = nf;
+          HPS_CUDA(cudaHostAlloc((void**)&h->trsv_err_host, sizeof(int), cudaHostAllocMapped));
+          *h->trsv_err_host = 0;
+          int* dp = nullptr;
+          HPS_CUDA(cudaHostGetDevicePointer((void**)&dp, h->trsv_err_host, 0));
+          h->trsv.host_err = h->trsv_err_host;
+          h->trsv.dev_err = dp;
+        }
       } else {
         HPS_CUDA(permute_rows<T>(bopp<T>(A.dR, nI), XX, A.perm, nI, ne + 1, nbat, st, pf));
         HPS_CUDA(getrs_inplace<T>(DD, nI, XX, ne + 1, nbat, st, pf));
@@ -665,7 +672,7 @@ hps_status adaptive_solve(hps_handle* h, int nrhs, const void* g_in, const void*
     BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)ni * ni, ni);
     BOp<T> XF = bop<T>(xf, (int64_t)ni * nrhs, ni);
     HPS_CUDA(permute_rows<T>(bop<T>(tmp, (int64_t)ni * nrhs, ni), XF, h->leaf_perm, ni, nrhs, (int)nl, st, pf));
-    HPS_CUDA(getrs_inplace<T>(LA, ni, XF, nrhs, (int)nl, st, pf));
+    HPS_CUDA(getrs_inplace<T>(LA, ni, XF, nrhs, (int)nl, st, pf, &h->leaf_inv));
     GemmArgs<T> gl;
     gl.M = nb; gl.N = nrhs; gl.K = ni; gl.batch = (int)nl;
     gl.A = bop<T>(h->dQi, 0, nb);
@@ -686,12 +693,12 @@ hps_status adaptive_solve(hps_handle* h, int nrhs, const void* g_in, const void*
       HPS_CUDA(proj_rows_group<T>(L.pr, L.npr, L.tpr, h->dF2C, st, pf));
       HPS_CUDA(gather_h_group<T>(L.gh, L.ngh, L.tgh, st, pf));
       for (size_t gi = g0; gi < g1; ++gi) {
-        const AGroup& G = h->ag[gi];
+        AGroup& G = h->ag[gi];
         const int nbat = (int)G.members.size();
         if (h->am[(size_t)G.members[0]].lazy) continue;  // the root's D^{-1} runs in the downward pass
         BOp<T> XB = bopp<T>(G.dx, G.n_int);
         HPS_CUDA(permute_rows<T>(bopp<T>(G.dr, G.n_int), XB, G.perm, G.n_int, nrhs, nbat, st, pf));
-        HPS_CUDA(getrs_inplace<T>(bopp<T>(G.dD, G.n_int), G.n_int, XB, nrhs, nbat, st, pf));
+        HPS_CUDA(getrs_inplace<T>(bopp<T>(G.dD, G.n_int), G.n_int, XB, nrhs, nbat, st, pf, &G.inv));
       }
       for (size_t gi = g0; gi < g1; ++gi) {
         const AGroup& G = h->ag[gi];
@@ -720,7 +727,7 @@ hps_status adaptive_solve(hps_handle* h, int nrhs, const void* g_in, const void*
       if (trsv_flags_applicable<T>(M.n_int, nrhs, 1, h->trsv))
         HPS_CUDA(getrs_flags<T>((const T*)M.D, M.n_int, M.n_int, (T*)M.gint, M.n_int, nrhs, h->trsv, st, pf));
       else
-        HPS_CUDA(getrs_inplace<T>(bop<T>((T*)M.D, 0, M.n_int), M.n_int, GI, nrhs, 1, st, pf));
+        HPS_CUDA(getrs_inplace<T>(bop<T>((T*)M.D, 0, M.n_int), M.n_int, GI, nrhs, 1, st, pf, &h->ag.back().inv));
     }
     // the level's other merges, their children's data and its unprojection
     HPS_CUDA(gint_group<T>(L.gi, L.ngi, L.tgi, newf ? 1 : 0, st, pf));

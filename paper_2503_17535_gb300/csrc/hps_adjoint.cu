@@ -215,7 +215,7 @@ hps_status apply_Dinv_h(hps_handle* h, int m, T* y, T* b, int nrhs, cudaStream_t
   BOp<T> YB = bop<T>(y, (int64_t)ni * nrhs, ni);
   BOp<T> BB = bop<T>(b, (int64_t)ni * nrhs, ni);
   if (!Kind<T>::iti) {
-    HPS_CUDA(getrs_h<T>(bop<T>((T*)Lv.D, (int64_t)ni * ni, ni), ni, YB, nrhs, nm, st, pf));
+    HPS_CUDA(getrs_h<T>(bop<T>((T*)Lv.D, (int64_t)ni * ni, ni), ni, YB, nrhs, nm, st, pf, &Lv.inv));
     HPS_CUDA(permute_rows_inv<T>(YB, BB, Lv.perm, ni, nrhs, nm, st));
     return HPS_OK;
   }
@@ -226,7 +226,7 @@ hps_status apply_Dinv_h(hps_handle* h, int m, T* y, T* b, int nrhs, cudaStream_t
   // b2bar = y2bar
   HPS_CUDA(copy_block<T>(y + hn, (int64_t)ni * nrhs, ni, b + hn, (int64_t)ni * nrhs, ni, hn, nrhs, nm, st, pf));
   // b1'bar = W^{-H} y1bar
-  HPS_CUDA(getrs_h<T>(bop<T>((T*)Lv.W, (int64_t)hn * hn, hn), hn, YB, nrhs, nm, st, pf));
+  HPS_CUDA(getrs_h<T>(bop<T>((T*)Lv.W, (int64_t)hn * hn, hn), hn, YB, nrhs, nm, st, pf, &Lv.inv));
   HPS_CUDA(permute_rows_inv<T>(YB, BB, Lv.perm, hn, nrhs, nm, st));
   // b2bar += -D12^H b1'bar  (forward D12 product: C = b rows odd_eq, B = b rows odd_var)
   HPS_CUDA(child_block_h<T>(h, m, true, grouped(BB, 2), grouped(BB, 2), nrhs, st, pf));
@@ -395,7 +395,7 @@ hps_status adjoint_impl(hps_handle* h, int nrhs, const void* ub_in, void* gbar_o
   } else {
     BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)nlu * nlu, nlu);
     BOp<T> XF = bop<T>(xf, (int64_t)xr * nrhs, xr);
-    HPS_CUDA(getrs_h<T>(LA, nlu, XF, nrhs, (int)nl, st, pf));
+    HPS_CUDA(getrs_h<T>(LA, nlu, XF, nrhs, (int)nl, st, pf, &h->leaf_inv));
     HPS_CUDA(permute_rows_inv<T>(XF, bop<T>(tmp, (int64_t)xr * nrhs, xr), h->leaf_perm, nlu, nrhs, (int)nl, st));
   }
   HPS_CUDA(cudaMemsetAsync(fbar, 0, ubytes, st));

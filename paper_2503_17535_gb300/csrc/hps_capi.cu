@@ -49,6 +49,10 @@ size_t plan_bytes(const hps_handle* h, bool with_solve_ws) {
   b += (size_t)nl * h->xrows_leaf * (h->nb + 1) * es;        // leaf X
   b += (size_t)nl * h->nb * (h->nb + 1) * es;                // leaf T|h
   b += (size_t)nl * h->nlu_leaf * 3 * sizeof(int);
+  auto inv = [&](int n, int64_t batch) {
+    return trsv_cluster_wanted(n, batch) ? (size_t)trsv_inv_elems(n, batch) * es : 0;
+  };
+  b += inv(h->nlu_leaf, nl);
   size_t scratch = (size_t)nl * h->xrows_leaf * (h->nb + 1) * es;
   int n = h->n0 > 0 ? h->n0 : (h->dim == 2 ? h->q : h->q * h->q);
   int64_t nm = nl;
@@ -61,6 +65,7 @@ size_t plan_bytes(const hps_handle* h, bool with_solve_ws) {
     b += (size_t)nm * n_ext * (n_ext + 1) * es;   // TP
     b += (size_t)nm * n_int * n_int * es;         // D
     if (h->iti) b += (size_t)nm * (n_int / 2) * (n_int / 2) * es;
+    b += inv(h->iti ? n_int / 2 : n_int, nm);
     b += (size_t)nm * n_int * (n_ext + 1) * es;   // X
     scratch = std::max(scratch, (size_t)nm * n_int * (n_ext + 1) * es);
     if (with_solve_ws) b += (size_t)nm * (3 * n_int + 2 * n_ext) * es * 2;
@@ -230,6 +235,7 @@ hps_status build_impl(hps_handle* h, const hps_coeffs* cf, const void* f_in, cud
       HPS_CUDA(cudaMemsetAsync(h->leaf_luw.bars, 0, sizeof(unsigned) * 2 * nl, st));
     }
     BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)nlu * nlu, nlu);
+    if (!alloc_inv<T>(h, nlu, nl, &h->leaf_inv)) return HPS_ERR_OOM;
     HPS_CUDA(getrf<T>(LA, nlu, (int)nl, h->leaf_ipiv, h->leaf_perm, h->leaf_info, h->dev_err, h->leaf_G,
                       h->leaf_luw, st, pf));
     HPS_CUDA(permute_rows<T>(bop<T>(RHS, (int64_t)xr * (nb + 1), xr), LX, h->leaf_perm, nlu, nb + 1, (int)nl, st, pf));
@@ -304,8 +310,10 @@ hps_status build_impl(hps_handle* h, const hps_coeffs* cf, const void* f_in, cud
       return HPS_ERR_OOM;
     HPS_CUDA(cudaMemsetAsync(Lv.info, 0, (size_t)nm * sizeof(int), st));
     Lv.lazy = Lv.top() && h->opts.lazy_root && !h->opts.want_root_map;
-    if (Lv.lazy && nm == 1) {
-      // flags and a host-mapped error word for the flag-ordered solves
+    const bool by_flags = Lv.lazy && nm == 1 && trsv_flags_preferred(nlu_m);
+    if (!by_flags && !alloc_inv<T>(h, nlu_m, nm, &Lv.inv)) return HPS_ERR_OOM;
+    if (by_flags) {
+      // a large root: flags and a host-mapped error word for the flag-ordered solves
       const int nf = (ni + 31) / 32;
       h->trsv.flags = (unsigned*)dalloc(h, (size_t)nf * sizeof(unsigned));
       h->trsv.dinv = dalloc(h, (size_t)2 * nf * 1024 * sizeof(T));
@@ -493,7 +501,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
     if (!h->capturing && trsv_flags_applicable<T>(ni, nrhs, nm, h->trsv))
       HPS_CUDA(getrs_flags<T>((const T*)Lv.D, ni, ni, y, ni, nrhs, h->trsv, st, pf));
     else
-      HPS_CUDA(getrs_inplace<T>(DD, ni, YB, nrhs, nm, st, pf));
+      HPS_CUDA(getrs_inplace<T>(DD, ni, YB, nrhs, nm, st, pf, &Lv.inv, h->capturing));
     return HPS_OK;
   }
   const int hn = ni / 2, nb = h->nb;
@@ -524,7 +532,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
   if (!h->capturing && trsv_flags_applicable<T>(hn, nrhs, nm, h->trsv))
     HPS_CUDA(getrs_flags<T>((const T*)Lv.W, hn, hn, y, ni, nrhs, h->trsv, st, pf));
   else
-    HPS_CUDA(getrs_inplace<T>(WW, hn, YB, nrhs, nm, st, pf));
+    HPS_CUDA(getrs_inplace<T>(WW, hn, YB, nrhs, nm, st, pf, &Lv.inv, h->capturing));
   HPS_CUDA(copy_block<T>(b + hn, (int64_t)ni * nrhs, ni, y + hn, (int64_t)ni * nrhs, ni, hn, nrhs, nm, st, pf));
   // y2 <- b2 - D21 y1 (even children's interior blocks)
   HPS_CUDA(child_block(false, grouped(YB, 2), grouped(YB, 2)));
@@ -572,7 +580,7 @@ hps_status solve_impl(hps_handle* h, int nrhs, const void* g_in, const void* f_i
     } else {
       BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)nlu * nlu, nlu);
       HPS_CUDA(permute_rows<T>(bop<T>(tmp, (int64_t)xr * nrhs, xr), XF, h->leaf_perm, nlu, nrhs, (int)nl, st, pf));
-      HPS_CUDA(getrs_inplace<T>(LA, nlu, XF, nrhs, (int)nl, st, pf));
+      HPS_CUDA(getrs_inplace<T>(LA, nlu, XF, nrhs, (int)nl, st, pf, &h->leaf_inv, h->capturing));
     }
     GemmArgs<T> gl;
     gl.M = nb; gl.N = nrhs; gl.K = ITI ? (int)h->npts : xr; gl.batch = (int)nl;

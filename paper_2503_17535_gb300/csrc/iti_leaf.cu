@@ -167,6 +167,7 @@ hps_status iti_elim_setup(hps_handle* h, const Coeffs& co, cudaStream_t st, Prof
   E.ipivS = (int*)dalloc(h, (size_t)nl * no * sizeof(int));
   E.permS = (int*)dalloc(h, (size_t)nl * no * sizeof(int));
   if (!E.Goe || !E.Goi || !E.LU || !E.W || !E.S || !E.ipiv || !E.perm || !E.ipivS || !E.permS) return HPS_ERR_OOM;
+  if (!alloc_inv<double>(h, ni, nl, &E.inv) || !alloc_inv<cplx>(h, no, nl, &E.invS)) return HPS_ERR_OOM;
   HPS_TRY(ensure_cap(h, h->nb + 1));
   // the build's scratch holds the temporaries (it is sized for nl x p^2 x (nb + 1) complex)
   double* tmp = (double*)h->scratch;
@@ -227,7 +228,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   BOp<double> LUo = bop<double>(E.LU, (int64_t)ni * ni, ni);
   BOp<double> Z2 = bop<double>(E.z2, (int64_t)ni * 2 * m, ni);
   HPS_CUDA(permute_rows<double>(bop<double>(E.z, (int64_t)ni * 2 * m, ni), Z2, E.perm, ni, 2 * m, (int)nl, st, pf));
-  HPS_CUDA(getrs_inplace<double>(LUo, ni, Z2, 2 * m, (int)nl, st, pf));
+  HPS_CUDA(getrs_inplace<double>(LUo, ni, Z2, 2 * m, (int)nl, st, pf, &E.inv, h->capturing));
   // q = r_o - G_oi z
   {
     GemmArgs<double> g;
@@ -245,7 +246,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   BOp<cplx> SB = bop<cplx>(E.S, (int64_t)no * no, no);
   BOp<cplx> Q2 = bop<cplx>(E.q2, (int64_t)no * m, no);
   HPS_CUDA(permute_rows<cplx>(bop<cplx>(E.q, (int64_t)no * m, no), Q2, E.permS, no, m, (int)nl, st, pf));
-  HPS_CUDA(getrs_inplace<cplx>(SB, no, Q2, m, (int)nl, st, pf));
+  HPS_CUDA(getrs_inplace<cplx>(SB, no, Q2, m, (int)nl, st, pf, &E.invS, h->capturing));
   // y_i = z - W y_e
   k_split<<<gridn(nl * no * 2 * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
                                                   (int64_t)no * 2 * m);
@@ -300,7 +301,7 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
   // x_o = S^{-H} q
   BOp<cplx> QB = bop<cplx>(E.q, (int64_t)no * m, no);
   BOp<cplx> Q2 = bop<cplx>(E.q2, (int64_t)no * m, no);
-  HPS_CUDA(getrs_h<cplx>(bop<cplx>(E.S, (int64_t)no * no, no), no, QB, m, (int)nl, st, pf));
+  HPS_CUDA(getrs_h<cplx>(bop<cplx>(E.S, (int64_t)no * no, no), no, QB, m, (int)nl, st, pf, &E.invS));
   HPS_CUDA(permute_rows_inv<cplx>(QB, Q2, E.permS, no, m, (int)nl, st));
   // z_i -= G_oi^T x_o
   k_split<<<gridn(nl * no * 2 * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
@@ -319,7 +320,7 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
   }
   // x_i = L_ii^{-T} z_i
   BOp<double> Z2 = bop<double>(E.z2, (int64_t)ni * 2 * m, ni);
-  HPS_CUDA(getrs_h<double>(bop<double>(E.LU, (int64_t)ni * ni, ni), ni, ZB, 2 * m, (int)nl, st, pf));
+  HPS_CUDA(getrs_h<double>(bop<double>(E.LU, (int64_t)ni * ni, ni), ni, ZB, 2 * m, (int)nl, st, pf, &E.inv));
   HPS_CUDA(permute_rows_inv<double>(ZB, Z2, E.perm, ni, 2 * m, (int)nl, st));
   // Rbar rows: [x_o; x_i]
   k_copy_rows<<<gridn(nl * no * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, no, m, nl, Rb, xs, xr, nullptr, 0,

@@ -360,13 +360,24 @@ __global__ void __launch_bounds__(256) k_gemm_skinny_kg(GemmArgs<T> g) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[c] = T(0.0);
     if (act) {
-#pragma unroll 4
-      for (int l = w; l < g.K; l += 8) {
-        const T a = A[ar + (int64_t)g.acol.at(b, l) * g.A.ld];
-        const int64_t br = g.brow.at(b, l);
+      // eight entries (and their gathered indices) in flight
+      const int* ac = g.acol.idx ? g.acol.idx + (b % g.acol.period) * g.acol.len : nullptr;
+      const int* bi = g.brow.idx ? g.brow.idx + (b % g.brow.period) * g.brow.len : nullptr;
+      for (int l0 = w; l0 < g.K; l0 += 64) {
+        T a[8], x[8][NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
-          if (c < g.N) acc[c] = fmac(acc[c], a, B[br + (int64_t)c * g.B.ld]);
+        for (int k = 0; k < 8; ++k) {
+          const int l = l0 + 8 * k;
+          const bool in = l < g.K;
+          a[k] = in ? A[ar + (int64_t)(ac ? ac[l] : l) * g.A.ld] : T(0.0);
+          const int64_t br = in ? (bi ? bi[l] : l) : 0;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) x[k][c] = in && c < g.N ? B[br + (int64_t)c * g.B.ld] : T(0.0);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], a[k], x[k][c]);
       }
     }
 #pragma unroll
@@ -479,7 +490,7 @@ cudaError_t gemm(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
   if (g.ta) {
     dim3 grid((g.M + 31) / 32, (g.N + 31) / 32, std::min(g.batch, 65535));
     k_gemm_ta<T><<<grid, 256, 0, st>>>(g);
-  } else if (g.N <= 8 && g.K >= 128 && (int64_t)((g.M + 127) / 128) * g.batch < 304) {
+  } else if (g.N <= 8 && g.K >= 32 && (int64_t)((g.M + 127) / 128) * g.batch < 304) {
     dim3 grid((g.M + 31) / 32, 1, std::min(g.batch, 65535));
     if (g.N == 1) k_gemm_skinny_kg<T, 1><<<grid, 256, 0, st>>>(g);
     else if (g.N == 2) k_gemm_skinny_kg<T, 2><<<grid, 256, 0, st>>>(g);
@@ -2084,8 +2095,10 @@ static cudaError_t rtrsm_upper(BOp<T> LU, BOp<T> X, int p0, int n1, int nrhs, in
 
 template <typename T>
 cudaError_t getrs_inplace(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st,
-                          Prof* pf) {
+                          Prof* pf, TrsvInv* inv, bool capturing) {
   if (n <= 0 || nrhs <= 0 || batch <= 0) return cudaSuccess;
+  if (trsv_few_applicable<T>(n, nrhs, batch, inv))
+    return trsv_few<T>(LU, n, X, nrhs, batch, false, inv, capturing, st, pf);
   cudaError_t e;
   // forward: unit lower; backward: non-unit upper
   if ((e = rtrsm_lower<T>(LU, X, 0, n, nrhs, batch, st, pf)) != cudaSuccess) return e;
@@ -2356,7 +2369,11 @@ cudaError_t permute_rows_inv(BOp<T> src, BOp<T> dst, const int* perm, int n, int
 // X <- (U^H)^{-1} then (L^H)^{-1}: the conjugate transpose of getrs_inplace
 // (without the row permutation, which the caller applies after).
 template <typename T>
-cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf) {
+cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf, TrsvInv* inv,
+                    bool capturing) {
+  if (n <= 0 || nrhs <= 0 || batch <= 0) return cudaSuccess;
+  if (trsv_few_applicable<T>(n, nrhs, batch, inv))
+    return trsv_few<T>(LU, n, X, nrhs, batch, true, inv, capturing, st, pf);
   const int pb0 = 32;
   const int by = std::min(batch, 65535);
   const int bx = std::min((nrhs + 127) / 128, 1024);
@@ -2407,11 +2424,11 @@ cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_
                                 const LuWork&, cudaStream_t, Prof*);                             \
   template cudaError_t permute_rows<T>(BOp<T>, BOp<T>, const int*, int, int, int, cudaStream_t,  \
                                        Prof*);                                                   \
-  template cudaError_t getrs_inplace<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*);                   \
+  template cudaError_t getrs_inplace<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*, bool);   \
   template bool trsv_flags_applicable<T>(int, int, int, const TrsvWork&);                        \
   template cudaError_t getrs_flags<T>(const T*, int, int, T*, int, int, TrsvWork&, cudaStream_t, Prof*); \
   template cudaError_t permute_rows_inv<T>(BOp<T>, BOp<T>, const int*, int, int, int, cudaStream_t);    \
-  template cudaError_t getrs_h<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*);
+  template cudaError_t getrs_h<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*, bool);
 
 HPS_INST(double)
 HPS_INST(cplx)

@@ -187,9 +187,30 @@ template <typename T>
 cudaError_t permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch,
                          cudaStream_t st, Prof* pf);
 
+// Inverses of the diagonal blocks of a batch of factors (trsv.cu): storage of
+// trsv_inv_elems elements that lives as long as the factors, filled by the
+// first solve with few right-hand sides.
+struct TrsvInv {
+  void* p = nullptr;
+  bool ready = false;
+};
+inline int64_t trsv_inv_elems(int n, int64_t batch) { return batch * 2 * ((n + 31) / 32) * 1024; }
+// Whether solves of this batch take a cluster per matrix (and want a TrsvInv).
+bool trsv_cluster_wanted(int n, int64_t batch);
+// Whether a lazy root of order n takes the flag-ordered solve instead.
+bool trsv_flags_preferred(int n);
+template <typename T>
+bool trsv_few_applicable(int n, int nrhs, int batch, const TrsvInv* inv);
+// Both triangles in one launch, X already row-permuted: X <- U^{-1} L^{-1} X,
+// or with herm X <- L^{-H} U^{-H} X (before the inverse permutation).
+// capturing: the stream is being captured into a graph.
+template <typename T>
+cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm, TrsvInv* inv, bool capturing,
+                     cudaStream_t st, Prof* pf);
+
 template <typename T>
 cudaError_t getrs_inplace(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st,
-                          Prof* pf);
+                          Prof* pf, TrsvInv* inv = nullptr, bool capturing = false);
 
 // One n x n LU factor against nrhs <= 8 columns (X <- U^{-1} L^{-1} X, X
 // already row-permuted), each triangle in a single cooperative launch:
@@ -222,7 +243,8 @@ template <typename T>
 cudaError_t permute_rows_inv(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch,
                              cudaStream_t st);
 template <typename T>
-cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf);
+cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf,
+                    TrsvInv* inv = nullptr, bool capturing = false);
 
 // C = alpha * C + beta (identity added on the diagonal when diag != 0) helpers
 template <typename T>

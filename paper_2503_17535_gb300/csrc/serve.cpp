@@ -500,8 +500,11 @@ void sched_main(hps_server* s) {
       return nullptr;
     };
     std::vector<int> apply_only;  // idle slots whose head is a solve with the build-time source
+    // rr moves on with each dispatch; one pass visits every slot once, from
+    // where it stood (a slot met twice would enter a group twice)
+    const size_t first = rr;
     for (size_t k = 0; k < ns; ++k) {
-      const int si = (int)((rr + k) % ns);
+      const int si = (int)((first + k) % ns);
       Slot& sl = s->slots[si];
       if (sl.busy || sl.q.empty()) continue;
       Req* head = sl.q.front();

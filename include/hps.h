@@ -46,9 +46,10 @@
  * not be used from two host threads at the same time.
  *
  * Device memory of handles and their workspaces comes from a stream-ordered
- * pool per device (cudaMallocFromPoolAsync / cudaFreeAsync, release
- * threshold 0): building, growing a workspace or freeing a handle never
- * waits for other streams.
+ * pool per device (cudaMallocFromPoolAsync / cudaFreeAsync): building,
+ * growing a workspace or freeing a handle never waits for other streams.
+ * The pool keeps up to a sixteenth of the device's memory after frees for the
+ * next builds; hps_trim gives it back.
  *
  * Errors: every call returns an hps_status; nothing is thrown across the ABI.
  * On failure *out handles are set to NULL and no memory is leaked.
@@ -304,6 +305,12 @@ hps_status hps_coeff_gradient(hps_handle* h, int nrhs, const void* u, const void
  * to the library's stream-ordered pool, so a free never stalls unrelated
  * streams. */
 void hps_free(hps_handle* h);
+
+/* Give the freed device memory that the library's pool keeps on the current
+ * device (at most a sixteenth of the device's memory) back to the device, for
+ * a program that needs it for something else.  Memory of live handles and of
+ * work in flight stays.  HPS_ERR_CUDA when a CUDA call fails. */
+hps_status hps_trim(void);
 
 /* Batched dense product C = alpha A B + beta C (no counterpart in the paper:
  * the GEMM every merge and leaf stage of hps_build is made of, exposed so

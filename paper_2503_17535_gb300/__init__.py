@@ -21,7 +21,7 @@ from . import _capi
 from ._capi import (HPS_C128, HPS_DTN, HPS_F64, HPS_ITI, HPS_OK, hps_coeffs,  # noqa: F401
                     hps_options, hps_tree)
 
-__all__ = ["hps_nodes", "hps_sizes", "hps_build", "hps_solve", "hps_solve_batched", "hps_free",
+__all__ = ["hps_nodes", "hps_sizes", "hps_build", "hps_solve", "hps_solve_batched", "hps_free", "hps_trim",
            "hps_error_string", "hps_last_error_detail", "hps_device_bytes",
            "hps_last_launch_count", "hps_kernel_stats", "hps_set_profiling", "hps_solve_noalloc",
            "hps_solve_multi",
@@ -296,6 +296,11 @@ def hps_free(h: Handle):
     if h is not None and h.ptr:
         _capi.lib().hps_free(h.ptr)
         h.ptr = None
+
+
+def hps_trim() -> None:
+    """Give the freed device memory the library keeps for later builds back to the device."""
+    _check(_capi.lib().hps_trim(), "hps_trim")
 
 
 def hps_error_string(status: int) -> str:

@@ -19,7 +19,7 @@ HPS_DTN, HPS_ITI = 0, 1
 HPS_F64, HPS_C128 = 0, 1
 
 EXPORTED = [
-    "hps_nodes", "hps_sizes", "hps_build", "hps_solve", "hps_solve_batched", "hps_solve_multi", "hps_free",
+    "hps_nodes", "hps_sizes", "hps_build", "hps_solve", "hps_solve_batched", "hps_solve_multi", "hps_free", "hps_trim",
     "hps_error_string", "hps_last_error_detail", "hps_device_bytes", "hps_last_launch_count",
     "hps_kernel_stats", "hps_set_profiling", "hps_solve_noalloc", "hps_refine", "hps_trace_count",
     "hps_trace_get", "hps_plan_bytes", "hps_solve_adjoint", "hps_coeff_gradient", "hps_gemm", "hps_getrf",
@@ -108,6 +108,8 @@ def lib() -> ctypes.CDLL:
     L.hps_solve_multi.restype = c_int
     L.hps_free.argtypes = [c_void_p]
     L.hps_free.restype = None
+    L.hps_trim.argtypes = []
+    L.hps_trim.restype = c_int
     L.hps_error_string.argtypes = [c_int]
     L.hps_error_string.restype = c_char_p
     L.hps_last_error_detail.argtypes = [c_void_p, POINTER(c_int64)]

@@ -8,6 +8,7 @@ namespace hps {
 namespace {
 
 constexpr int kMaxDevices = 64;
+constexpr size_t kKeepShare = 16;   // freed memory a pool may keep: this fraction of the device's
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
 cudaStream_t g_idle_stream[kMaxDevices] = {};
@@ -27,8 +28,10 @@ cudaError_t pool_of_current(cudaMemPool_t* out) {
     cudaMemPool_t pool = nullptr;
     e = cudaMemPoolCreate(&pool, &props);
     if (e != cudaSuccess) return e;
-    uint64_t thr = 0;
-    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    size_t fr = 0, tot = 0;
+    e = cudaMemGetInfo(&fr, &tot);
+    uint64_t thr = tot / kKeepShare;
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     if (e != cudaSuccess) {
       cudaMemPoolDestroy(pool);
       return e;
@@ -66,6 +69,22 @@ void dev_free_idle(void* p) {
     st = g_idle_stream[dev];
   }
   if (cudaFreeAsync(p, st) != cudaSuccess) cudaGetLastError();
+}
+
+cudaError_t dev_pool_trim() {
+  int dev = 0;
+  cudaStream_t idle = nullptr;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = pool_of_current(&pool);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    idle = g_idle_stream[dev];
+  }
+  // frees of released handles are queued on the idle stream only
+  if (idle && (e = cudaStreamSynchronize(idle)) != cudaSuccess) return e;
+  return cudaMemPoolTrimTo(pool, 0);
 }
 
 size_t dev_pool_idle_bytes() {

@@ -1509,6 +1509,12 @@ hps_status hps_coeff_gradient(hps_handle* h, int nrhs, const void* u, const void
 
 void hps_free(hps_handle* h) { free_handle(h); }
 
+hps_status hps_trim(void) {
+  if (hps::dev_pool_trim() == cudaSuccess) return HPS_OK;
+  cudaGetLastError();
+  return HPS_ERR_CUDA;
+}
+
 hps_status hps_last_error_detail(hps_handle* h, int64_t* node) {
   if (!node) return HPS_ERR_INVALID;
   *node = h ? h->err_node : g_last_err_node;

@@ -616,7 +616,7 @@ hps_status hps_server_create(const hps_server_options* opts, hps_server** out) {
       delete s;
       return HPS_ERR_CUDA;
     }
-    o.hbm_budget = (int64_t)(0.85 * (double)fr);
+    o.hbm_budget = (int64_t)(0.85 * (double)(fr + hps::dev_pool_idle_bytes()));
   }
   s->opts = o;
   s->stats.hbm_budget = o.hbm_budget;

@@ -12,6 +12,7 @@
 // latency chains (a reciprocal, a serial load) off the per-column critical
 // path of the panels.
 #include "linalg.h"
+#include "tri_cols.h"
 
 #include <cooperative_groups.h>
 
@@ -570,12 +571,6 @@ int device_sms() {
     return s > 0 ? s : 1;
   }();
   return sms;
-}
-
-// whole-warp shuffle of a real or complex value
-__device__ inline double shfl_val(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ inline cplx shfl_val(cplx v, int src) {
-  return cplx(__shfl_sync(0xffffffffu, v.re, src), __shfl_sync(0xffffffffu, v.im, src));
 }
 
 // ------------------------------------------------------------ panel LU ----
@@ -1401,118 +1396,102 @@ cudaError_t launch_panel_reg(const cudaLaunchConfig_t& cfg, int cs, BOp<T> A, in
 // Apply the panel's interchanges to every column outside the panel and
 // solve U12 = L11^{-1} A12 for the columns in [k0 + nb, trsm_end).
 //
-// The nb interchanges are first composed into one permutation of at most
-// 2 nb rows: warp 0 replays them with lane t holding the row now at
-// position k0 + t, and for a step whose partner lies below the panel's top,
-// lane jj recording that outside position and the row it received (a later
-// step with the same partner takes the record over).  Every thread then reads
-// all moved entries of its column at once and writes them back permuted --
-// one round trip per column instead of one per interchange -- and solves its
-// top block in registers.
-template <typename T, int NB, bool REG>
-__global__ void __launch_bounds__(128) k_laswp_trsm(BOp<T> A, int n, int k0, int nb, const int* ipiv,
-                                                    int trsm_end) {
-  extern __shared__ unsigned char smem_raw[];
-  T* L11 = reinterpret_cast<T*>(smem_raw);  // nb x nb, column-major
-  __shared__ int src_top[32], dst_out[32], src_out[32];
-  const int b = blockIdx.y;
-  T* Ab = A.item(b);
-  const int lda = A.ld;
-  const bool any_trsm = trsm_end > k0 + nb;
-  if (any_trsm)
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-      const int r = e % nb, c = e / nb;
-      L11[e] = Ab[(int64_t)(k0 + r) + (int64_t)(k0 + c) * lda];
+// The interchanges are first composed into one permutation of at most 2 nb
+// rows: a thread per position of the panel's top and per position that an
+// interchange swapped with walks its position back through the nb
+// interchanges to the row whose entries end there.  TC threads per column
+// then read all moved entries at once, write the outside ones back, and solve
+// the top block in registers (tri_cols.h).  Rows that stay where they are in
+// a column without a solve are not touched.
+//
+// Bound by the substitution's chain when there are few matrices, by the FP64
+// pipe and the sectors of the moved rows when there are many.  One thread per
+// column, the triangle's entry loaded before each multiply-add: 41 us for
+// 6880 real columns of one matrix, 49 for 64 of order 432, 755 for 4096 of
+// order 196 (32-row panels), 26 for 1776 complex columns (16-row panels);
+// this form 13.5, 35, 534 and 8.3.
+template <typename T, int NB, int TC>
+__global__ void __launch_bounds__(128) k_laswp_trsm(BOp<T> A, int n, int k0, int nb, const int* ipiv, int trsm_end) {
+  using S = TriCols<T, NB, TC>;
+  constexpr int R = S::R, CW = 128 / TC;
+  __shared__ __align__(16) T tri[NB * NB];
+  __shared__ int src[2 * NB], dst[NB], ips[NB];
+  const int tid = threadIdx.x;
+  T* Ab = A.item(blockIdx.y) + k0;
+  const int64_t ld = A.ld;
+  if (tid < NB) ips[tid] = tid < nb ? ipiv[(int64_t)blockIdx.y * n + k0 + tid] - k0 : tid;
+  if (trsm_end > k0 + nb) {
+#pragma unroll
+    for (int u = 0; u < NB * NB / 128; ++u) {
+      const int e = tid + 128 * u, r = e % NB, c = e / NB;
+      tri[S::at(r, c)] = r < nb && c < nb ? Ab[r + (k0 + c) * ld] : T(0.0);
     }
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const int* ip = ipiv + (int64_t)b * n + k0;
-    const int pl = lane < nb ? ip[lane] : 0;   // all interchanges in one load
-    int content = k0 + lane;   // row whose entries sit at position k0 + lane
-    int opos = -1, ocont = -1; // outside position last swapped at this lane's step, and its row
-    for (int jj = 0; jj < nb; ++jj) {
-      const int p = __shfl_sync(0xffffffffu, pl, jj);
-      const int cj = __shfl_sync(0xffffffffu, content, jj);
-      if (p < k0 + nb) {
-        const int cp = __shfl_sync(0xffffffffu, content, p - k0);
-        if (lane == jj) content = cp;
-        if (lane == p - k0) content = cj;
-      } else {
-        const unsigned m = __ballot_sync(0xffffffffu, opos == p);
-        const int owner = m ? 31 - __clz((int)m) : 0;
-        const int held = __shfl_sync(0xffffffffu, ocont, owner);
-        const int cur = m ? held : p;   // never swapped before: still row p
-        if (m && lane == owner) opos = -1;
-        if (lane == jj) { content = cur; opos = p; ocont = cj; }
-      }
-    }
-    src_top[lane] = lane < nb ? content : 0;
-    dst_out[lane] = lane < nb ? opos : -1;
-    src_out[lane] = ocont;
   }
   __syncthreads();
-  const int ncols_out = n - nb;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ncols_out; t += gridDim.x * blockDim.x) {
-    const int c = (t < k0) ? t : t + nb;
-    T* col = Ab + (int64_t)c * lda;
-    T x[NB], xo[NB];
-    if constexpr (REG) {
-      // few CTAs (one or a few matrices): the whole column in registers,
-      // every load in flight at once, the solve unrolled
+  if (tid < 2 * NB) {
+    const int t = tid % NB, p0 = tid < NB ? t : ips[t];
+    bool last = true;   // no later interchange names this position (those from nb on are no-ops)
+    int pos = p0;
 #pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q < nb) x[q] = col[src_top[q]];
-        if (q < nb && dst_out[q] >= 0) xo[q] = col[src_out[q]];
+    for (int jj = NB - 1; jj >= 0; --jj) {
+      const int p = ips[jj];
+      if (jj > t && jj < nb && p == p0) last = false;
+      pos = pos == jj ? p : pos == p ? jj : pos;
+    }
+    src[tid] = pos;
+    if (tid >= NB) dst[t] = last && p0 >= nb ? p0 : -1;
+  }
+  __syncthreads();
+  const int g = tid % TC, lane0 = tid & 31 & ~(TC - 1);
+  const int ncols = n - nb;
+  for (int t0 = blockIdx.x * CW; t0 < ncols; t0 += gridDim.x * CW) {
+    const int t = t0 + tid / TC;
+    const bool live = t < ncols;
+    const int c = t < k0 ? t : t + nb;
+    const bool solve = live && c >= k0 + nb && c < trsm_end;
+    T* col = Ab + c * ld;
+    T x[R], xo[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int i = g + q * TC;
+      x[q] = xo[q] = T(0.0);
+      if (live && i < nb) {
+        if (solve || src[i] != i) x[q] = col[src[i]];
+        if (dst[i] >= 0) xo[q] = col[src[NB + i]];
       }
+    }
+    __syncwarp();
 #pragma unroll
-      for (int q = 0; q < NB; ++q)
-        if (q < nb && dst_out[q] >= 0) col[dst_out[q]] = xo[q];
-      if (c >= k0 + nb && c < trsm_end) {
+    for (int q = 0; q < R; ++q) {
+      const int i = g + q * TC;
+      if (live && i < nb && dst[i] >= 0) col[dst[i]] = xo[q];
+      xo[q] = x[q];
+    }
+    if (__any_sync(0xffffffffu, solve)) S::lower(xo, tri, g, lane0, nb);
 #pragma unroll
-        for (int jj = 1; jj < NB; ++jj) {
-          if (jj < nb) {
-            T s = x[jj];
-#pragma unroll
-            for (int ii = 0; ii < jj; ++ii) s = fmsc(s, L11[jj + ii * nb], x[ii]);
-            x[jj] = s;
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < NB; ++q)
-        if (q < nb) col[k0 + q] = x[q];
-    } else {
-      // many matrices: runtime-indexed arrays (local memory, L1-resident) keep
-      // the registers, and so the occupancy that hides the FP64 solve's
-      // latency, where the unrolled form would take ~250 registers a thread
-      for (int q = 0; q < nb; ++q) {
-        x[q] = col[src_top[q]];
-        if (dst_out[q] >= 0) xo[q] = col[src_out[q]];
-      }
-      for (int q = 0; q < nb; ++q)
-        if (dst_out[q] >= 0) col[dst_out[q]] = xo[q];
-      if (c >= k0 + nb && c < trsm_end) {
-        for (int jj = 1; jj < nb; ++jj) {
-          T s = x[jj];
-          for (int ii = 0; ii < jj; ++ii) s = fmsc(s, L11[jj + ii * nb], x[ii]);
-          x[jj] = s;
-        }
-      }
-#pragma unroll 8
-      for (int q = 0; q < nb; ++q) col[k0 + q] = x[q];
+    for (int q = 0; q < R; ++q) {
+      const int i = g + q * TC;
+      if (live && i < nb && (solve || src[i] != i)) col[i] = solve ? xo[q] : x[q];
     }
   }
 }
 
-__global__ void k_ipiv_to_perm(const int* ipiv, int* perm, int n, int batch) {
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  const int* ip = ipiv + (int64_t)b * n;
-  int* pm = perm + (int64_t)b * n;
-  for (int i = 0; i < n; ++i) pm[i] = i;
-  for (int j = 0; j < n; ++j) {
-    int p = ip[j];
-    if (p != j) { int t = pm[j]; pm[j] = pm[p]; pm[p] = t; }
+// perm[i] = the row whose entries the interchanges leave in row i.  Interchange
+// j touches rows >= j only, so row i is settled by interchange i; from there
+// the row's origin is followed back: an earlier interchange that named the
+// current position brought it from row j.  A thread per row, no exchange
+// between them.  Bound by the walk of the last rows (replaying the swaps of a
+// matrix in one thread took 650 us for 6912 rows; this 147).
+__global__ void __launch_bounds__(128) k_ipiv_to_perm(const int* ipiv, int* perm, int n) {
+  const int* ip = ipiv + (int64_t)blockIdx.x * n;
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
+    int pos = ip[i];
+#pragma unroll 16
+    for (int j = min(i | 31, n - 1) - 1; j >= 0; --j) {
+      const int p = ip[j];
+      if (j < i && p == pos) pos = j;
+    }
+    perm[(int64_t)blockIdx.x * n + i] = pos;
   }
 }
 
@@ -1656,17 +1635,18 @@ static cudaError_t lu_leaf(BOp<T> A, int n, int k0, int nb, int trsm_end, int ba
   if (pf) pf->end(K_LU_PANEL, pfl, st);
   if (n > nb) {
     const int ncols = n - nb;
-    // few matrices: 32-thread CTAs, so that the columns spread over the SMs
-    const bool few = ((ncols + 127) / 128) * batch < 2 * device_sms();
-    const int tpb = few ? 32 : 128;
-    int bx = std::min((ncols + tpb - 1) / tpb, 1024);
-    size_t sm2 = (size_t)nb * nb * sizeof(T);
+    // eight threads per column have the shortest chain; four issue an eighth
+    // less once the FP64 pipe is full whatever the split (4096 matrices of
+    // order 196: 534 us against 570; 1024 of order 224: 108 against 103)
+    const bool many = (int64_t)((ncols + 31) / 32) * batch >= 48 * device_sms();
+    const int cw = many ? 32 : 16;
+    const dim3 grid(std::min((ncols + cw - 1) / cw, 4096), batch);
     if (pf) {
       pf->begin(st);
       pf->note(nb, ncols, nb, batch);
     }
-    if (few) k_laswp_trsm<T, LuNB<T>::NB, true><<<dim3(bx, batch), tpb, sm2, st>>>(A, n, k0, nb, ipiv, trsm_end);
-    else k_laswp_trsm<T, LuNB<T>::NB, false><<<dim3(bx, batch), tpb, sm2, st>>>(A, n, k0, nb, ipiv, trsm_end);
+    if (many) k_laswp_trsm<T, LuNB<T>::NB, 4><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, trsm_end);
+    else k_laswp_trsm<T, LuNB<T>::NB, 8><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, trsm_end);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (pf) pf->end(K_LASWP_TRSM, F * 0.5 * nb * (nb - 1) * (double)std::max(0, trsm_end - k0 - nb) * batch, st);
   }
@@ -1749,7 +1729,7 @@ cudaError_t getrf(BOp<T> A, int n, int batch, int* ipiv, int* perm, int* info, u
   if (base_w < nbp) base_w = nbp;
   if ((e = rgetrf<T>(A, n, 0, n, base_w, pnb, batch, ipiv, info, dev_err, G, w, st, pf)) != cudaSuccess) return e;
   if (pf) pf->begin(st);
-  k_ipiv_to_perm<<<(batch + 127) / 128, 128, 0, st>>>(ipiv, perm, n, batch);
+  k_ipiv_to_perm<<<dim3(batch, std::min((n + 127) / 128, 65535)), 128, 0, st>>>(ipiv, perm, n);
   if (pf) pf->end(K_OTHER, 0.0, st);
   return cudaGetLastError();
 }
@@ -1874,156 +1854,81 @@ __global__ void __launch_bounds__(128) k_trsm_diag_cols(BOp<T> LU, BOp<T> X, int
   }
 }
 
-// Full 32-row diagonal blocks: a CTA takes CT right-hand sides of one
-// matrix, loads the 32 x CT tile of X coalesced (a warp per column) into
-// shared memory (stride 33: conflict-free per-thread columns), solves one
-// column per thread in registers (fully unrolled), and stores coalesced.
-template <typename T, bool UPPER, int CT>
-__global__ void __launch_bounds__(CT) k_trsm32(BOp<T> LU, BOp<T> X, int p0, int nrhs, int batch) {
-  __shared__ T Ls[32 * 32];
-  __shared__ T Dinv[32];
-  __shared__ T Xs[CT * 33];
-  const int b = blockIdx.y;
-  const T* Lb = LU.item(b);
-  T* Xb = X.item(b);
-  const int j0 = blockIdx.x * CT;
-  const int ncol = min(CT, nrhs - j0);
-  for (int e = threadIdx.x; e < 32 * 32; e += CT) {
-    const int r = e & 31, c = e >> 5;
-    Ls[e] = Lb[(int64_t)(p0 + r) + (int64_t)(p0 + c) * LU.ld];
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int c = wid; c < ncol; c += CT / 32) Xs[c * 33 + lane] = Xb[(int64_t)(j0 + c) * X.ld + p0 + lane];
-  __syncthreads();
-  if (UPPER && threadIdx.x < 32) {
-    const T d = Ls[threadIdx.x * 33];
-    Dinv[threadIdx.x] = is_zero(d) ? T(0.0) : recip(d);
-  }
-  __syncthreads();
-  if (threadIdx.x < ncol) {
-    T x[32];
-    T* xc = Xs + threadIdx.x * 33;
+// Diagonal blocks of 32 rows (or fewer, padded), TC threads per right-hand
+// side (tri_cols.h); a thread's loads of its column are in flight while the
+// block is staged.  Bound by the FP64 pipe with many columns, by the chain of
+// 32 steps with few.  Against one thread per column that loads each entry
+// before its multiply-add (lower / upper, us): 865 real columns of one matrix
+// 18 / 19 -> 8 / 10, 865 of 64 matrices 55 / 80 -> 57 / 66, 114 of 4096
+// 434 / 600 -> 447 / 472; 1793 complex columns of 4 matrices 74 / 78 -> 35 / 49, 225 of 256
+// 251 / 270 -> 231 / 268.
+template <typename T, bool UPPER, int TC>
+__global__ void __launch_bounds__(128) k_trsm32(BOp<T> LU, BOp<T> X, int p0, int pb, int nrhs) {
+  using S = TriCols<T, 32, TC>;
+  __shared__ __align__(16) T tri[32 * 32];
+  __shared__ T dinv[32];
+  const int b = blockIdx.y, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const T* Lb = LU.item(b) + p0 + (int64_t)p0 * LU.ld;
+  const int j = blockIdx.x * (nt / TC) + tid / TC, g = tid % TC;
+  const bool live = j < nrhs;
+  T* col = X.item(b) + p0 + (int64_t)j * X.ld;
+  T x[S::R];
 #pragma unroll
-    for (int r = 0; r < 32; ++r) x[r] = xc[r];
-    if (!UPPER) {
-#pragma unroll
-      for (int r = 1; r < 32; ++r) {
-        T s2 = x[r];
-#pragma unroll
-        for (int c = 0; c < r; ++c) s2 = fmsc(s2, Ls[r + c * 32], x[c]);
-        x[r] = s2;
-      }
-    } else {
-#pragma unroll
-      for (int r = 31; r >= 0; --r) {
-        T s2 = x[r];
-#pragma unroll
-        for (int c = r + 1; c < 32; ++c) s2 = fmsc(s2, Ls[r + c * 32], x[c]);
-        x[r] = s2 * Dinv[r];
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 32; ++r) xc[r] = x[r];
+  for (int q = 0; q < S::R; ++q) x[q] = live && g + q * TC < pb ? col[g + q * TC] : T(0.0);
+#pragma unroll 8
+  for (int c = tid >> 5; c < 32; c += nt >> 5) tri[S::at(lane, c)] = lane < pb && c < pb ? Lb[lane + (int64_t)c * LU.ld] : T(0.0);
+  if (UPPER && tid < 32) {
+    const T d = tid < pb ? Lb[tid + (int64_t)tid * LU.ld] : T(0.0);
+    dinv[tid] = is_zero(d) ? T(0.0) : recip(d);
   }
   __syncthreads();
-  for (int c = wid; c < ncol; c += CT / 32) Xb[(int64_t)(j0 + c) * X.ld + p0 + lane] = Xs[c * 33 + lane];
+  if (blockIdx.x * (nt / TC) + (tid & ~31) / TC >= nrhs) return;   // a warp without columns
+  const int lane0 = lane & ~(TC - 1);
+  if (UPPER) S::upper(x, tri, dinv, g, lane0, 32);
+  else S::lower(x, tri, g, lane0, 32);
+#pragma unroll
+  for (int q = 0; q < S::R; ++q)
+    if (live && g + q * TC < pb) col[g + q * TC] = x[q];
 }
 
-// Full 32-row diagonal blocks with few CTAs in the grid (few matrices):
-// four threads per right-hand side, each holding 8 of the block's 32 rows.
-// The row groups are solved in dependency order, each group's solution
-// broadcast by shuffles to the four threads of its column, the later groups
-// subtracting its contribution: the chain per column is four 8-row
-// triangles and three 8 x 8 updates instead of one 32-row substitution, and
-// the columns spread over four times the warps.
-template <typename T, bool UPPER>
-__global__ void __launch_bounds__(128) k_trsm32_g4(BOp<T> LU, BOp<T> X, int p0, int nrhs, int batch) {
-  __shared__ T Ls[32 * 32];
-  __shared__ T Dinv[32];
-  __shared__ T Xs[32 * 33];
-  const int b = blockIdx.y;
-  const T* Lb = LU.item(b);
-  T* Xb = X.item(b);
-  const int j0 = blockIdx.x * 32;
-  const int ncol = min(32, nrhs - j0);
-  for (int e = threadIdx.x; e < 32 * 32; e += 128) {
-    const int r = e & 31, c = e >> 5;
-    Ls[e] = Lb[(int64_t)(p0 + r) + (int64_t)(p0 + c) * LU.ld];
+// Threads per right-hand side of k_trsm32, or 0 for k_trsm_diag_cols.
+//
+// A warp's FP64 instructions per column set are known (496 multiply-adds for
+// 32 rows in one thread, 256, 136 and 76 in each of 2, 4 and 8; the upper
+// triangle scales once per row in every thread), and every scheduler issues one
+// in 64 cycles, so the time goes with the fullest scheduler's warps times
+// that count: few columns take 8 threads, many take the form that issues least in
+// all.  Loads that one warp per scheduler does not hide put the counts below
+// at 540 and 572 for one thread; the upper triangle's longer chain makes 4 and 8 threads
+// count 200 and 130.  Blocks of less than 32 rows are padded, which
+// costs pipe time, so they come here only while one wave of warps holds all columns.
+template <bool UPPER>
+int trsm32_threads(int pb, int nrhs, int batch) {
+  const int count[4] = {UPPER ? 572 : 540, UPPER ? 288 : 256, UPPER ? 200 : 136, UPPER ? 130 : 76};
+  const int64_t slots = 4 * device_sms();
+  if (pb < 32 && (int64_t)((nrhs * 8 + 31) / 32) * batch > slots) return 0;
+  int best = 0;
+  int64_t least = 0;
+  for (int i = 3; i >= 0; --i) {
+    const int64_t warps = (int64_t)(((int64_t)nrhs * (1 << i) + 31) / 32) * batch;
+    const int64_t t = (warps + slots - 1) / slots * count[i];
+    if (!best || t < least) best = 1 << i, least = t;
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int c = wid; c < ncol; c += 4) Xs[c * 33 + lane] = Xb[(int64_t)(j0 + c) * X.ld + p0 + lane];
-  __syncthreads();
-  if (UPPER && threadIdx.x < 32) {
-    const T d = Ls[threadIdx.x * 33];
-    Dinv[threadIdx.x] = is_zero(d) ? T(0.0) : recip(d);
-  }
-  __syncthreads();
-  const int col = threadIdx.x >> 2, g = threadIdx.x & 3;
-  const bool live = col < ncol;
-  const int lane0 = lane & ~3;   // the column's first lane
-  T x[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) x[i] = live ? Xs[col * 33 + 8 * g + i] : T(0.0);
-#pragma unroll
-  for (int step = 0; step < 4; ++step) {
-    const int blk = UPPER ? 3 - step : step;
-    if (g == blk) {
-      if (!UPPER) {
-#pragma unroll
-        for (int i = 1; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < i; ++j) x[i] = fmsc(x[i], Ls[(8 * g + i) + (8 * g + j) * 32], x[j]);
-      } else {
-#pragma unroll
-        for (int i = 7; i >= 0; --i) {
-          T sacc = x[i];
-#pragma unroll
-          for (int j = i + 1; j < 8; ++j) sacc = fmsc(sacc, Ls[(8 * g + i) + (8 * g + j) * 32], x[j]);
-          x[i] = sacc * Dinv[8 * g + i];
-        }
-      }
-    }
-    T xb[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) xb[j] = shfl_val(x[j], lane0 | blk);
-    if (UPPER ? g < blk : g > blk) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) x[i] = fmsc(x[i], Ls[(8 * g + i) + (8 * blk + j) * 32], xb[j]);
-    }
-  }
-  if (live) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) Xs[col * 33 + 8 * g + i] = x[i];
-  }
-  __syncthreads();
-  for (int c = wid; c < ncol; c += 4) Xb[(int64_t)(j0 + c) * X.ld + p0 + lane] = Xs[c * 33 + lane];
+  return best;
 }
 
 template <typename T, bool UPPER>
 cudaError_t trsm_diag(BOp<T> LU, BOp<T> X, int p0, int pb, int nrhs, int batch, cudaStream_t st) {
   const size_t sm = ((size_t)pb * pb + pb) * sizeof(T);
   const int by = std::min(batch, 65535);
-  if (pb == 32 && nrhs >= 16 && batch <= 65535) {
-    // 128 columns per CTA (real data) unless that leaves most SMs idle; the
-    // complex tile keeps 32 so that static shared memory stays below 48 KB;
-    // a grid of at most one such CTA per SM splits each column over four
-    // threads (shorter chains on more SMSPs; with more CTAs than SMs the
-    // split form's extra instructions cost more than its latency saves:
-    // measured on 1793 complex columns of 4 matrices, 4.6 -> 5.2 ms)
-    const int ctas32 = ((nrhs + 31) / 32) * batch;
-    bool wide = false;
-    if constexpr (sizeof(T) == 8) {
-      wide = ((nrhs + 127) / 128) * batch >= 2 * device_sms();
-      if (wide) k_trsm32<T, UPPER, 128><<<dim3((nrhs + 127) / 128, batch), 128, 0, st>>>(LU, X, p0, nrhs, batch);
-    }
-    if (!wide) {
-      if (ctas32 <= device_sms())
-        k_trsm32_g4<T, UPPER><<<dim3((nrhs + 31) / 32, batch), 128, 0, st>>>(LU, X, p0, nrhs, batch);
-      else
-        k_trsm32<T, UPPER, 32><<<dim3((nrhs + 31) / 32, batch), 32, 0, st>>>(LU, X, p0, nrhs, batch);
-    }
+  const int tc = nrhs >= 16 && batch <= 65535 ? trsm32_threads<UPPER>(pb, nrhs, batch) : 0;
+  if (tc) {
+    const int nt = 32 * std::min(4, (nrhs * tc + 31) / 32);
+    const dim3 grid((nrhs + nt / tc - 1) / (nt / tc), batch);
+    if (tc == 1) k_trsm32<T, UPPER, 1><<<grid, nt, 0, st>>>(LU, X, p0, pb, nrhs);
+    else if (tc == 2) k_trsm32<T, UPPER, 2><<<grid, nt, 0, st>>>(LU, X, p0, pb, nrhs);
+    else if (tc == 4) k_trsm32<T, UPPER, 4><<<grid, nt, 0, st>>>(LU, X, p0, pb, nrhs);
+    else k_trsm32<T, UPPER, 8><<<grid, nt, 0, st>>>(LU, X, p0, pb, nrhs);
   } else if (nrhs >= 16) {
     const int bx = std::min((nrhs + 127) / 128, 1024);
     k_trsm_diag_cols<T, UPPER><<<dim3(bx, by), 128, sm, st>>>(LU, X, p0, pb, nrhs, batch);

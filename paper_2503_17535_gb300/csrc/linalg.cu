@@ -82,15 +82,6 @@ template <> constexpr double fma_flops<cplx>() { return 8.0; }
 
 // ---------------------------------------------------------------- GEMM ----
 
-// Tile shapes: 64 x 64 (4 x 4 outputs per thread) for large FP64 products,
-// 32 x 32 (2 x 2 per thread) where 64-wide tiles would leave much of the
-// last tile row / column empty (the leaf updates of (p-2)^2-sized blocks).
-template <typename T, int WIDE> struct GemmTile;
-template <> struct GemmTile<double, 1> { enum { BM = 64, BN = 64, BK = 16, TM = 4, TN = 4 }; };
-template <> struct GemmTile<double, 0> { enum { BM = 32, BN = 32, BK = 16, TM = 2, TN = 2 }; };
-template <> struct GemmTile<cplx, 1> { enum { BM = 32, BN = 32, BK = 16, TM = 2, TN = 2 }; };
-template <> struct GemmTile<cplx, 0> { enum { BM = 32, BN = 32, BK = 16, TM = 2, TN = 2 }; };
-
 // Epilogue modes: the LU / TRSM / Schur updates are C <- C - A B and the
 // leaf products C <- A B; handling those two forms apart keeps the general
 // alpha / beta arithmetic (a complex multiply and multiply-add per element)
@@ -104,183 +95,138 @@ inline int epi_mode(const GemmArgs<T>& g) {
   return EPI_GENERAL;
 }
 
-template <typename T, int MODE, int WIDE>
-__global__ void __launch_bounds__(256) k_gemm(GemmArgs<T> g) {
-  constexpr int BM = GemmTile<T, WIDE>::BM, BN = GemmTile<T, WIDE>::BN, BK = GemmTile<T, WIDE>::BK;
-  constexpr int TM = GemmTile<T, WIDE>::TM, TN = GemmTile<T, WIDE>::TN;
-  constexpr int RX = BM / TM;  // threads along M (16)
-  __shared__ T As[BK][BM];
-  __shared__ T Bs[BK][BN];
-  const int tid = threadIdx.x;
-  const int tx = tid % RX, ty = tid / RX;
-  for (int b = blockIdx.z; b < g.batch; b += gridDim.z) {
-    const T* A = g.A.item(b);
-    const T* B = g.B.item(b);
-    T* C = g.C.item(b);
-    const int i0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
-    T acc[TM][TN];
-#pragma unroll
-    for (int r = 0; r < TM; ++r)
-#pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        acc[r][c] = T(0.0);
-        if (MODE == EPI_SUB) {
-          const int gi = i0 + tx + RX * r, gj = j0 + ty + (256 / RX) * c;
-          if (gi < g.M && gj < g.N) acc[r][c] = C[(int64_t)g.crow.at(b, gi) + (int64_t)gj * g.C.ld];
-        }
-      }
-    for (int k0 = 0; k0 < g.K; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += 256) {
-        int i = e % BM, l = e / BM;
-        int gi = i0 + i, gl = k0 + l;
-        T v = T(0.0);
-        if (gi < g.M && gl < g.K)
-          v = A[(int64_t)g.arow.at(b, gi) + (int64_t)g.acol.at(b, gl) * g.A.ld];
-        As[l][i] = v;
-      }
-      for (int e = tid; e < BK * BN; e += 256) {
-        int l = e % BK, j = e / BK;
-        int gl = k0 + l, gj = j0 + j;
-        T v = T(0.0);
-        if (gl < g.K && gj < g.N) v = B[(int64_t)g.brow.at(b, gl) + (int64_t)gj * g.B.ld];
-        Bs[l][j] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        T av[TM], bv[TN];
-#pragma unroll
-        for (int r = 0; r < TM; ++r) av[r] = As[kk][tx + RX * r];
-#pragma unroll
-        for (int c = 0; c < TN; ++c) bv[c] = Bs[kk][ty + (256 / RX) * c];
-#pragma unroll
-        for (int r = 0; r < TM; ++r)
-#pragma unroll
-          for (int c = 0; c < TN; ++c)
-            acc[r][c] = MODE == EPI_SUB ? fmsc(acc[r][c], av[r], bv[c]) : fmac(acc[r][c], av[r], bv[c]);
-      }
-      __syncthreads();
-    }
-    const bool use_beta = !is_zero(g.beta);
-#pragma unroll
-    for (int r = 0; r < TM; ++r) {
-      int gi = i0 + tx + RX * r;
-      if (gi >= g.M) continue;
-      int64_t ci = g.crow.at(b, gi);
-#pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        int gj = j0 + ty + (256 / RX) * c;
-        if (gj >= g.N) continue;
-        T* p = C + ci + (int64_t)gj * g.C.ld;
-        if (MODE != EPI_GENERAL) {
-          *p = acc[r][c];
-        } else {
-          T v = g.alpha * acc[r][c];
-          if (use_beta) v = fmac(v, g.beta, *p);
-          *p = v;
-        }
-      }
-    }
-  }
-}
-
-// Complex GEMM by the 3M method: with A = Ar + i Ai and B = Br + i Bi, the
-// real products P1 = Ar Br, P2 = Ai Bi and P3 = (Ar + Ai)(Br + Bi) give
+// Products on the FP64 pipe, N > 8: BM x 256 / BM tiles (BM = 32, 16 or 8 rows,
+// whichever pads the shape least), four warps, a thread per row and
+// pair of columns, 32 steps of K staged at once with the next 32 in flight in
+// registers.
+//
+// The pipe does two multiply-adds per clock and SM, so that even these small
+// tiles need only 2.5 of the 30 bytes per clock that L2 delivers to an SM; what
+// counts is that the tiles spread over all SMs, that K is not padded (to a
+// multiple of four only) and that the pipe never waits for a load.
+// us (64 x 64 or 32 x 32 tiles with 16 steps of K, the loads waited for, before -> now): 32 x
+// 864 x 32 14.4 -> 6.3, 64 x 864 x 64 75 -> 12.4, 128 x 128 x 128 145 -> 14.4, 1024 x 1024 x
+// 64 135 -> 115 (pipe: 112); batches of 4096 64 x 114 x 4 874 -> 277.
+//
+// Complex products take the 3M method: with A = Ar + i Ai and B = Br + i Bi,
+// the real products P1 = Ar Br, P2 = Ai Bi and P3 = (Ar + Ai)(Br + Bi) give
 // C = (P1 - P2) + i (P3 - P1 - P2).  Each complex multiply-add costs three
 // real FMAs instead of four on the FP64 pipe; the sums Ar + Ai and Br + Bi
 // are formed once per element when the tile is staged in shared memory.
 // With MODE == EPI_SUB the accumulators start from C so that the update
 // needs three additions per element: p1 = 0, p2 = Re C, p3 = Re C - Im C give
 // Re(C - AB) = p2 - p1 and Im(C - AB) = p1 + p2 - p3 after the products.
-template <int MODE>
-__global__ void __launch_bounds__(256) k_gemm_c3m(GemmArgs<cplx> g) {
-  constexpr int BM = 32, BN = 32, BK = 16, TM = 2, TN = 2, RX = 16;
-  __shared__ double Ar[BK][BM], Ai[BK][BM], As[BK][BM];
-  __shared__ double Br[BK][BN], Bi[BK][BN], Bs[BK][BN];
-  const int tid = threadIdx.x;
-  const int tx = tid % RX, ty = tid / RX;
-  for (int b = blockIdx.z; b < g.batch; b += gridDim.z) {
-    const cplx* A = g.A.item(b);
-    const cplx* B = g.B.item(b);
-    cplx* C = g.C.item(b);
-    const int i0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
-    double p1[TM][TN], p2[TM][TN], p3[TM][TN];
+template <typename T> struct GemmPlanes { enum { N = 1 }; };
+template <> struct GemmPlanes<cplx> { enum { N = 3 }; };
+
+__device__ __forceinline__ double gemm_plane(double v, int) { return v; }
+__device__ __forceinline__ double gemm_plane(cplx v, int p) { return p == 0 ? v.re : p == 1 ? v.im : v.re + v.im; }
+
+template <typename T, int MODE, int BM>
+__global__ void __launch_bounds__(128) k_gemm(GemmArgs<T> g) {
+  constexpr int P = GemmPlanes<T>::N, BN = 256 / BM, BK = 32, LA = BM / 4, LB = BN / 4;
+  __shared__ double As[P][BK][BM];
+  __shared__ __align__(16) double Bs[P][BK][BN + 2];   // + 2: the staging writes go down a column
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int r = tid % BM, c0 = 2 * (tid / BM);   // this thread's row and columns c0, c0 + 1 of the tile
+  const int ra = tid % BM, la = tid / BM;        // what it stages of A: row ra, steps la, la + 128 / BM, ...
+  const int tiles_m = (g.M + BM - 1) / BM;
+  const int i = blockIdx.x % tiles_m * BM + r, j0 = blockIdx.x / tiles_m * BN;
+  const bool beta = MODE == EPI_SUB || (MODE == EPI_GENERAL && !is_zero(g.beta));
+  for (int b = blockIdx.y; b < g.batch; b += gridDim.y) {
+    const T* A = g.A.item(b);
+    const T* B = g.B.item(b);
+    T* C = g.C.item(b);
+    const bool row = i < g.M;
+    const int64_t ai = row ? g.arow.at(b, i) : 0, ci = row ? g.crow.at(b, i) : 0;
+    T a[LA], bb[LB], cv[2];
+    double acc[P][2];
+    auto load = [&](int k0) {
 #pragma unroll
-    for (int r = 0; r < TM; ++r)
-#pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        p1[r][c] = p2[r][c] = p3[r][c] = 0.0;
-        if (MODE == EPI_SUB) {
-          const int gi = i0 + tx + RX * r, gj = j0 + ty + 16 * c;
-          if (gi < g.M && gj < g.N) {
-            const cplx cv = C[(int64_t)g.crow.at(b, gi) + (int64_t)gj * g.C.ld];
-            p2[r][c] = cv.re;
-            p3[r][c] = cv.re - cv.im;
-          }
-        }
+      for (int u = 0; u < LA; ++u) {
+        const int l = k0 + la + 128 / BM * u;
+        a[u] = row && l < g.K ? A[ai + (int64_t)g.acol.at(b, l) * g.A.ld] : T(0.0);
       }
-    for (int k0 = 0; k0 < g.K; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += 256) {
-        const int i = e % BM, l = e / BM;
-        const int gi = i0 + i, gl = k0 + l;
-        cplx v(0.0, 0.0);
-        if (gi < g.M && gl < g.K) v = A[(int64_t)g.arow.at(b, gi) + (int64_t)g.acol.at(b, gl) * g.A.ld];
-        Ar[l][i] = v.re; Ai[l][i] = v.im; As[l][i] = v.re + v.im;
+      const int l = k0 + lane;
+      const int64_t bi = l < g.K ? g.brow.at(b, l) : 0;
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        const int j = j0 + w + 4 * u;
+        bb[u] = l < g.K && j < g.N ? B[bi + (int64_t)j * g.B.ld] : T(0.0);
       }
-      for (int e = tid; e < BK * BN; e += 256) {
-        const int l = e % BK, j = e / BK;
-        const int gl = k0 + l, gj = j0 + j;
-        cplx v(0.0, 0.0);
-        if (gl < g.K && gj < g.N) v = B[(int64_t)g.brow.at(b, gl) + (int64_t)gj * g.B.ld];
-        Br[l][j] = v.re; Bi[l][j] = v.im; Bs[l][j] = v.re + v.im;
-      }
-      __syncthreads();
+    };
+    load(0);
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        double ar[TM], ai[TM], as[TM], br[TN], bi[TN], bs[TN];
+    for (int c = 0; c < 2; ++c) {
+      cv[c] = beta && row && j0 + c0 + c < g.N ? C[ci + (int64_t)(j0 + c0 + c) * g.C.ld] : T(0.0);
 #pragma unroll
-        for (int r = 0; r < TM; ++r) { ar[r] = Ar[kk][tx + RX * r]; ai[r] = Ai[kk][tx + RX * r]; as[r] = As[kk][tx + RX * r]; }
-#pragma unroll
-        for (int c = 0; c < TN; ++c) { br[c] = Br[kk][ty + 16 * c]; bi[c] = Bi[kk][ty + 16 * c]; bs[c] = Bs[kk][ty + 16 * c]; }
-#pragma unroll
-        for (int r = 0; r < TM; ++r)
-#pragma unroll
-          for (int c = 0; c < TN; ++c) {
-            p1[r][c] = fma(ar[r], br[c], p1[r][c]);
-            p2[r][c] = fma(ai[r], bi[c], p2[r][c]);
-            p3[r][c] = fma(as[r], bs[c], p3[r][c]);
-          }
-      }
-      __syncthreads();
-    }
-    const bool use_beta = !is_zero(g.beta);
-#pragma unroll
-    for (int r = 0; r < TM; ++r) {
-      const int gi = i0 + tx + RX * r;
-      if (gi >= g.M) continue;
-      const int64_t ci = g.crow.at(b, gi);
-#pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        const int gj = j0 + ty + 16 * c;
-        if (gj >= g.N) continue;
-        cplx* p = C + ci + (int64_t)gj * g.C.ld;
-        if (MODE == EPI_SUB) {
-          *p = cplx(p2[r][c] - p1[r][c], (p1[r][c] + p2[r][c]) - p3[r][c]);
-        } else if (MODE == EPI_SET) {
-          *p = cplx(p1[r][c] - p2[r][c], p3[r][c] - (p1[r][c] + p2[r][c]));
+      for (int p = 0; p < P; ++p) acc[p][c] = 0.0;
+      if (MODE == EPI_SUB) {
+        if constexpr (P == 1) {
+          acc[0][c] = cv[c];
         } else {
-          const cplx acc(p1[r][c] - p2[r][c], p3[r][c] - p1[r][c] - p2[r][c]);
-          cplx v = g.alpha * acc;
-          if (use_beta) v = fmac(v, g.beta, *p);
-          *p = v;
+          acc[1][c] = cv[c].re;
+          acc[2][c] = cv[c].re - cv[c].im;
         }
       }
+    }
+    for (int k0 = 0; k0 < g.K; k0 += BK) {
+      const int kc = min(BK, (g.K - k0 + 3) & ~3);   // steps beyond K are zero
+      __syncthreads();
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+#pragma unroll
+        for (int u = 0; u < LA; ++u)
+          if (la + 128 / BM * u < kc) As[p][la + 128 / BM * u][ra] = gemm_plane(a[u], p);
+#pragma unroll
+        for (int u = 0; u < LB; ++u) Bs[p][lane][w + 4 * u] = gemm_plane(bb[u], p);
+      }
+      __syncthreads();
+      if (k0 + BK < g.K) load(k0 + BK);
+#pragma unroll 2
+      for (int k = 0; k < kc; k += 4) {
+        double av[P][4];
+        double2 bv[P][4];
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            av[p][u] = As[p][k + u][r];
+            bv[p][u] = *reinterpret_cast<const double2*>(&Bs[p][k + u][c0]);
+          }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int p = 0; p < P; ++p) {
+            const double s = P == 1 && MODE == EPI_SUB ? -av[p][u] : av[p][u];
+            acc[p][0] = fma(s, bv[p][u].x, acc[p][0]);
+            acc[p][1] = fma(s, bv[p][u].y, acc[p][1]);
+          }
+      }
+    }
+    __syncthreads();
+    if (!row) continue;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (j0 + c0 + c >= g.N) continue;
+      T v;
+      if constexpr (P == 1) {
+        v = acc[0][c];
+      } else if (MODE == EPI_SUB) {
+        v = cplx(acc[1][c] - acc[0][c], (acc[0][c] + acc[1][c]) - acc[2][c]);
+      } else if (MODE == EPI_SET) {
+        v = cplx(acc[0][c] - acc[1][c], acc[2][c] - (acc[0][c] + acc[1][c]));
+      } else {
+        v = cplx(acc[0][c] - acc[1][c], acc[2][c] - acc[0][c] - acc[1][c]);
+      }
+      if (MODE == EPI_GENERAL) {
+        v = g.alpha * v;
+        if (beta) v = fmac(v, g.beta, cv[c]);
+      }
+      C[ci + (int64_t)(j0 + c0 + c) * g.C.ld] = v;
     }
   }
 }
-
-template <typename T> struct UseC3M { static constexpr bool value = false; };
-template <> struct UseC3M<cplx> { static constexpr bool value = true; };
 
 // Skinny variant for N <= 8 right-hand sides (the solve path): one thread
 // per output row, B chunks staged in shared memory, A read column by column
@@ -464,13 +410,19 @@ __global__ void __launch_bounds__(256) k_gemm_ta(GemmArgs<T> g) {
   }
 }
 
-// Wide (64 x 64) tiles unless they leave more than 1/8 of the computed
-// outputs empty where 32 x 32 tiles would not: the padded area decides.
-inline bool wide_tiles(int M, int N, int BM, int BN) {
-  if (BM == 32) return false;
-  auto padded = [](int n, int b) { return (double)((n + b - 1) / b) * b; };
-  const double wide = padded(M, BM) * padded(N, BN), narrow = padded(M, 32) * padded(N, 32);
-  return wide <= 1.125 * narrow;
+template <typename T, int BM>
+void launch_gemm(const GemmArgs<T>& g, cudaStream_t st) {
+  const dim3 grid((unsigned)((g.M + BM - 1) / BM) * (unsigned)((g.N + 256 / BM - 1) / (256 / BM)), std::min(g.batch, 65535));
+  switch (epi_mode(g)) {
+    case EPI_SUB: k_gemm<T, EPI_SUB, BM><<<grid, 128, 0, st>>>(g); break;
+    case EPI_SET: k_gemm<T, EPI_SET, BM><<<grid, 128, 0, st>>>(g); break;
+    default: k_gemm<T, EPI_GENERAL, BM><<<grid, 128, 0, st>>>(g); break;
+  }
+}
+
+// outputs that tiles of bm x 256 / bm compute for an M x N product
+inline int64_t padded_outputs(int M, int N, int bm) {
+  return ((int64_t)(M + bm - 1) / bm * bm) * ((int64_t)(N + 256 / bm - 1) / (256 / bm) * (256 / bm));
 }
 
 template <typename T>
@@ -483,7 +435,6 @@ cudaError_t gemm(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     // product runs on the FP64 pipe instead
     cudaGetLastError();
   }
-  constexpr int BM = GemmTile<T, 1>::BM, BN = GemmTile<T, 1>::BN;
   if (pf) {
     pf->begin(st);
     pf->note(g.M, g.N, g.K, g.batch);
@@ -503,31 +454,14 @@ cudaError_t gemm(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     else if (g.N == 2) k_gemm_skinny<T, 2><<<grid, 128, 0, st>>>(g);
     else if (g.N <= 4) k_gemm_skinny<T, 4><<<grid, 128, 0, st>>>(g);
     else k_gemm_skinny<T, 8><<<grid, 128, 0, st>>>(g);
-  } else if (UseC3M<T>::value) {
-    dim3 grid((g.M + 31) / 32, (g.N + 31) / 32, std::min(g.batch, 65535));
-    const GemmArgs<cplx>& gc = *reinterpret_cast<const GemmArgs<cplx>*>(&g);
-    switch (epi_mode(gc)) {
-      case EPI_SUB: k_gemm_c3m<EPI_SUB><<<grid, 256, 0, st>>>(gc); break;
-      case EPI_SET: k_gemm_c3m<EPI_SET><<<grid, 256, 0, st>>>(gc); break;
-      default: k_gemm_c3m<EPI_GENERAL><<<grid, 256, 0, st>>>(gc); break;
-    }
-    const double mnk = g.M * (double)g.N * g.K * g.batch;
-    if (pf) pf->end(K_GEMM, 8.0 * mnk, st, 6.0 * mnk);
-    return cudaGetLastError();
-  } else if (wide_tiles(g.M, g.N, BM, BN)) {
-    dim3 grid((g.M + BM - 1) / BM, (g.N + BN - 1) / BN, std::min(g.batch, 65535));
-    switch (epi_mode(g)) {
-      case EPI_SUB: k_gemm<T, EPI_SUB, 1><<<grid, 256, 0, st>>>(g); break;
-      case EPI_SET: k_gemm<T, EPI_SET, 1><<<grid, 256, 0, st>>>(g); break;
-      default: k_gemm<T, EPI_GENERAL, 1><<<grid, 256, 0, st>>>(g); break;
-    }
   } else {
-    dim3 grid((g.M + 31) / 32, (g.N + 31) / 32, std::min(g.batch, 65535));
-    switch (epi_mode(g)) {
-      case EPI_SUB: k_gemm<T, EPI_SUB, 0><<<grid, 256, 0, st>>>(g); break;
-      case EPI_SET: k_gemm<T, EPI_SET, 0><<<grid, 256, 0, st>>>(g); break;
-      default: k_gemm<T, EPI_GENERAL, 0><<<grid, 256, 0, st>>>(g); break;
-    }
+    const int64_t o32 = padded_outputs(g.M, g.N, 32), o16 = padded_outputs(g.M, g.N, 16), o8 = padded_outputs(g.M, g.N, 8);
+    if (o32 <= o16 && o32 <= o8) launch_gemm<T, 32>(g, st);
+    else if (o16 <= o8) launch_gemm<T, 16>(g, st);
+    else launch_gemm<T, 8>(g, st);
+    if (pf) pf->end(K_GEMM, fma_flops<T>() * g.M * (double)g.N * g.K * g.batch, st,
+                    (sizeof(T) == 16 ? 6.0 : 2.0) * g.M * (double)g.N * g.K * g.batch);   // 3M: three of four
+    return cudaGetLastError();
   }
   if (pf) pf->end(K_GEMM, fma_flops<T>() * g.M * (double)g.N * g.K * g.batch, st);
   return cudaGetLastError();

@@ -30,9 +30,9 @@ ROOT = os.path.dirname(HERE)
 
 CANDIDATES = {
     "lu_cluster_panel": [0, 1],
-    "lu_base_panels_few": [0, 4, 8, 16, 32],
+    "lu_base_panels_few": [0, 16, 32, 64, 128],
     "lu_few_min_n": [1024, 2048, 4096, 8192],
-    "lu_base_panels_many": [2, 4, 8],
+    "lu_base_panels_many": [4, 8, 16, 32],
     "tc_min_work_real": [25, 50, 100, 200, 400],
     "tc_min_work_cplx": [6, 12, 25, 50, 100],
     "tc_min_k": [16, 33, 48, 64, 96],

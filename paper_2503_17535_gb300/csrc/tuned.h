@@ -6,9 +6,9 @@
 #pragma once
 
 #define HPS_TUNED_LU_CLUSTER_PANEL 1
-#define HPS_TUNED_LU_BASE_PANELS_FEW 32
+#define HPS_TUNED_LU_BASE_PANELS_FEW 128
 #define HPS_TUNED_LU_FEW_MIN_N 4096
-#define HPS_TUNED_LU_BASE_PANELS_MANY 8
+#define HPS_TUNED_LU_BASE_PANELS_MANY 32
 #define HPS_TUNED_TC_MIN_WORK_REAL 50
 #define HPS_TUNED_TC_MIN_WORK_CPLX 50
 #define HPS_TUNED_TC_MIN_K 16

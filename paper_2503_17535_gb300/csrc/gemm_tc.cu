@@ -206,20 +206,30 @@ __device__ __forceinline__ void put_digits(const double (&v)[8], int evm, uint8_
 }
 
 // One launch for all operands.  A warp takes units of 32 rows x UK k (16 for
-// real data: a whole k step; 8 for complex); of a CTA's 8 warps, KW share 32
-// rows and split the units of their inner dimension, and 8 / KW such row
-// groups share the CTA, so that short inner dimensions keep every warp busy.
+// real data: a whole k step; 8 for complex); of a CTA's NW warps (4, or 8 when
+// so many share rows), KW share 32 rows and split the units of their inner
+// dimension, and NW / KW such row groups share the CTA, so that short inner
+// dimensions keep every warp busy.
 // Long ones spread over the CS CTAs of a cluster as well (few rows and many k
 // would leave most SMs idle).  Pass 1 finds each row's largest magnitude (by
 // its upper word: only the exponent counts; over both parts of a complex
-// row), pass 2 writes the digits; when no warp has more than one unit, each
-// entry is read once and stays in registers.  An operand whose k runs along
+// row), pass 2 writes the digits, last unit first, which is still in
+// registers; when no warp has more than one unit, each entry is read once.
+// An operand whose k runs along
 // its columns (ks = 1: B, or B^T in the A slot) is read in segments of UK
 // entries per row and turned around in shared memory: one row per lane would
 // touch 32 cache lines per load.  Rows beyond R are not written: their
 // products land in outputs that nobody stores.
-template <typename T>
-__global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT, int b0, int KW, int CS) {
+//
+// Bound by instruction issue (100 per entry; 24 warps an SM) and the latency of
+// a CTA's load-write cycle, not by memory (2.5 - 4 TB/s).  Loads by pointer
+// steps instead of an index map looked up for each entry, row groups that wait for
+// their own warps only and smaller CTAs for short K, us for both operands of
+// 4096 items (before -> now): 164 x 164 x 32 339 -> 228, 128 x 128 x 68 538 ->
+// 309, 114 x 32 x 64 246 -> 207; one pass over the Helmholtz build's products
+// 15.1 -> 11.5 ms, the 3D elliptic's 11.0 -> 7.7.
+template <typename T, int NW>
+__global__ void __launch_bounds__(32 * NW, 24 / NW) k_split(SplitSet<T> ss, int K, int KT, int b0, int KW, int CS) {
   constexpr int UK = std::is_same<T, cplx>::value ? 8 : 16;   // k per unit
   constexpr int RL = 32 / UK;                                 // rows per load of a turned unit
   const int op = blockIdx.y, bl = blockIdx.z, b = b0 + bl;
@@ -227,10 +237,11 @@ __global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cr = (int)blockIdx.x % CS;                        // CTA of the cluster (clusters run along x)
   const int rg = (int)blockIdx.x / CS;
-  if (rg * (8 / KW) * 32 >= R || bl >= ss.items[op]) return;  // uniform over the cluster
+  if (rg * (NW / KW) * 32 >= R || bl >= ss.items[op]) return;  // uniform over the cluster
   const Src<T>& s = ss.s[op];
   const int kw = warp & (KW - 1);
-  const int rbase = (rg * (8 / KW) + warp / KW) * 32;
+  const int rbase = (rg * (NW / KW) + warp / KW) * 32;
+  if (rbase >= R && CS == 1) return;   // a row group without rows: its warps share no barrier with others
   const int r = rbase + lane;
   const T* X = s.X.item(b);
   const bool live = r < R;
@@ -239,18 +250,19 @@ __global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT,
   const int64_t rs = s.rs, ks = s.ks;
   const bool turn = ks == 1 && !s.rmap.idx;
   const int nu = KT * (TK / UK), step = KW * CS, u0 = cr * KW + kw;
-  __shared__ uint32_t smax[8][32];
-  __shared__ uint32_t cmax[8][8][32];   // [CTA of the cluster][row group][row]
-  __shared__ T tile[8][32 * (UK + 1)];
+  __shared__ uint32_t smax[NW][32];
+  __shared__ uint32_t cmax[NW == 8 ? 8 : 1][NW][32];   // [CTA of the cluster][row group][row]
+  __shared__ T tile[NW][32 * (UK + 1)];
   T xv[UK];
   auto load = [&](int u) {
     if (turn) {
       const int k = u * UK + (lane & (UK - 1));
       const int64_t ko = k < K ? (kidx ? (int64_t)kidx[k] : (int64_t)k) : -1;
+      const T* p = X + (int64_t)(rbase + lane / UK) * rs + ko;
 #pragma unroll
       for (int q = 0; q < UK; ++q) {
         const int row = rbase + q * RL + lane / UK;
-        xv[q] = (ko >= 0 && row < R) ? X[(int64_t)row * rs + ko] : T(0.0);
+        xv[q] = (ko >= 0 && row < R) ? p[(int64_t)(q * RL) * rs] : T(0.0);
       }
       __syncwarp();
 #pragma unroll
@@ -258,28 +270,33 @@ __global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT,
       __syncwarp();
 #pragma unroll
       for (int c = 0; c < UK; ++c) xv[c] = tile[warp][lane * (UK + 1) + c];
-    } else {
+    } else if (kidx) {
 #pragma unroll
       for (int c = 0; c < UK; ++c) {
         const int k = u * UK + c;
-        xv[c] = (live && k < K) ? X[roff + (int64_t)(kidx ? kidx[k] : k) * ks] : T(0.0);
+        xv[c] = (live && k < K) ? X[roff + (int64_t)kidx[k] * ks] : T(0.0);
       }
+    } else {
+      const T* p = X + roff + (int64_t)(u * UK) * ks;
+#pragma unroll
+      for (int c = 0; c < UK; ++c) xv[c] = (live && u * UK + c < K) ? p[c * ks] : T(0.0);
     }
   };
   uint32_t mx = 0;
+  int last = -1;   // the unit in xv
   for (int u = u0; u < nu; u += step) {
-    load(u);
+    load(last = u);
 #pragma unroll
     for (int c = 0; c < UK; ++c) mx = max(mx, mag_hi(xv[c]));
   }
   smax[warp][lane] = mx;
-  __syncthreads();
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / KW), "r"(32 * KW) : "memory");   // the warps of this row group
   for (int w = 0; w < KW; ++w) mx = max(mx, smax[warp - kw + w][lane]);
   if (CS > 1) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     if (kw == 0)
-      for (int d = 0; d < CS; ++d) cl.map_shared_rank(&cmax[0][0][0], d)[(cr * 8 + warp) * 32 + lane] = mx;
+      for (int d = 0; d < CS; ++d) cl.map_shared_rank(&cmax[0][0][0], d)[(cr * NW + warp) * 32 + lane] = mx;
     cl.sync();
     for (int d = 0; d < CS; ++d) mx = max(mx, cmax[d][warp - kw][lane]);
   }
@@ -288,8 +305,8 @@ __global__ void __launch_bounds__(256, 3) k_split(SplitSet<T> ss, int K, int KT,
   const int BLK = TK * 2 << lt;
   const int tl = r >> lt, rr = r & ((1 << lt) - 1);
   const int64_t rowoff = ((int64_t)bl * ss.RT[op] + tl) * KT * (int64_t)(DIG * BLK) + (rr >> 3) * 256 + (rr & 7) * 16;
-  for (int u = u0; u < nu; u += step) {
-    if (nu > step) load(u);
+  for (int u = last; u >= 0; u -= step) {
+    if (u != last) load(u);
     if (!live) continue;
 #pragma unroll
     for (int half = 0; half < UK / 8; ++half) {
@@ -975,13 +992,14 @@ cudaError_t launch_split(const tc::SplitSet<T>& ss, int nops, int K, int KT, int
   const int nu = KT * (std::is_same<T, cplx>::value ? 2 : 1);
   int kw = 1;
   while (kw < 8 && kw < nu) kw *= 2;
-  const int rows = 32 * (8 / kw);
+  const int nw = kw <= 4 ? 4 : 8;
+  const int rows = 32 * (nw / kw);
   const int64_t ctas = (int64_t)((rmax + rows - 1) / rows) * nops * nb;
   int cs = 1;
-  while (cs < 8 && nu > kw * cs && ctas * cs < 4 * device_sms()) cs *= 2;
+  while (nw == 8 && cs < 8 && nu > kw * cs && ctas * cs < 4 * device_sms()) cs *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((rmax + rows - 1) / rows * cs, nops, nb);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(32 * nw);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -990,7 +1008,8 @@ cudaError_t launch_split(const tc::SplitSet<T>& ss, int nops, int K, int KT, int
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = cs > 1 ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, tc::k_split<T>, ss, K, KT, b0, kw, cs);
+  const cudaError_t e = nw == 8 ? cudaLaunchKernelEx(&cfg, tc::k_split<T, 8>, ss, K, KT, b0, kw, cs)
+                                : cudaLaunchKernelEx(&cfg, tc::k_split<T, 4>, ss, K, KT, b0, kw, cs);
   if (pf) pf->end(K_SPLIT, 0.0, st);
   return e;
 }

@@ -1014,8 +1014,8 @@ cudaError_t launch_split(const tc::SplitSet<T>& ss, int nops, int K, int KT, int
   return e;
 }
 
-cudaError_t launch_mma(const tc::GemmP& p, const Tiling& tl, int kc, int nb, int M, int N, int K, cudaStream_t st,
-                       Prof* pf) {
+cudaError_t launch_mma(const tc::GemmP& p, const Tiling& tl, int kc, int nb, int M, int N, int K, int sms,
+                       cudaStream_t st, Prof* pf) {
   using namespace tc;
   if (pf) {
     pf->begin(st);
@@ -1026,7 +1026,7 @@ cudaError_t launch_mma(const tc::GemmP& p, const Tiling& tl, int kc, int nb, int
   // one CTA per tile
   const int64_t ntiles = (int64_t)p.MT * p.NT * nb;
   const bool persist = K >= lu_tune(TUNE_TC_PERSIST_MIN_K);
-  const int grid = (int)(persist ? std::min<int64_t>(ntiles, device_sms()) : ntiles);
+  const int grid = (int)(persist ? std::min<int64_t>(ntiles, sms) : ntiles);
   const bool unit = p.alpha == 1.0 || p.alpha == -1.0;
   const int epi = unit && p.beta == 0.0 ? TC_SET : unit && p.beta == 1.0 ? TC_ADD : TC_GENERAL;
   cudaError_t e;
@@ -1136,7 +1136,7 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     if constexpr (NP == 1) {
       p.As = As[0]; p.Bs = Bs[0];
       p.As2 = nullptr; p.Bs2 = nullptr; p.pair = 0; p.neg2 = 0;
-      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, device_sms() - g.spare_sms, st, pf)) != cudaSuccess) return e;
     } else {
       // complex (real alpha, beta), each component one launch of two
       // products into the same accumulators:
@@ -1152,12 +1152,12 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
       slots(0, 0, p.As, p.Bs);
       slots(1, 1, p.As2, p.Bs2);
       p.neg2 = 1;
-      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, device_sms() - g.spare_sms, st, pf)) != cudaSuccess) return e;
       slots(0, 1, p.As, p.Bs);
       slots(1, 0, p.As2, p.Bs2);
       p.neg2 = 0;
       p.C.off += 1;   // the imaginary component
-      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, st, pf)) != cudaSuccess) return e;
+      if ((e = launch_mma(p, tl, kc, nb, g.M, g.N, g.K, device_sms() - g.spare_sms, st, pf)) != cudaSuccess) return e;
     }
   }
   return cudaGetLastError();

@@ -1510,6 +1510,7 @@ hps_status hps_coeff_gradient(hps_handle* h, int nrhs, const void* u, const void
 void hps_free(hps_handle* h) { free_handle(h); }
 
 hps_status hps_trim(void) {
+  hps::lu_side_trim();
   if (hps::dev_pool_trim() == cudaSuccess) return HPS_OK;
   cudaGetLastError();
   return HPS_ERR_CUDA;

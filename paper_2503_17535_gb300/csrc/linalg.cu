@@ -14,6 +14,8 @@
 #include "linalg.h"
 #include "tri_cols.h"
 
+#include <mutex>
+
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1344,8 +1346,14 @@ cudaError_t launch_panel_reg(const cudaLaunchConfig_t& cfg, int cs, BOp<T> A, in
 // 6880 real columns of one matrix, 49 for 64 of order 432, 755 for 4096 of
 // order 196 (32-row panels), 26 for 1776 complex columns (16-row panels);
 // this form 13.5, 35, 534 and 8.3.
+struct LuCols {
+  int left;           // columns [0, left)
+  int first, right;   // and [first, first + right)
+};
+
 template <typename T, int NB, int TC>
-__global__ void __launch_bounds__(128) k_laswp_trsm(BOp<T> A, int n, int k0, int nb, const int* ipiv, int trsm_end) {
+__global__ void __launch_bounds__(128) k_laswp_trsm(BOp<T> A, int n, int k0, int nb, const int* ipiv, LuCols cols,
+                                                    int trsm_end) {
   using S = TriCols<T, NB, TC>;
   constexpr int R = S::R, CW = 128 / TC;
   __shared__ __align__(16) T tri[NB * NB];
@@ -1377,11 +1385,11 @@ __global__ void __launch_bounds__(128) k_laswp_trsm(BOp<T> A, int n, int k0, int
   }
   __syncthreads();
   const int g = tid % TC, lane0 = tid & 31 & ~(TC - 1);
-  const int ncols = n - nb;
+  const int ncols = cols.left + cols.right;
   for (int t0 = blockIdx.x * CW; t0 < ncols; t0 += gridDim.x * CW) {
     const int t = t0 + tid / TC;
     const bool live = t < ncols;
-    const int c = t < k0 ? t : t + nb;
+    const int c = t < cols.left ? t : t - cols.left + cols.first;
     const bool solve = live && c >= k0 + nb && c < trsm_end;
     T* col = Ab + c * ld;
     T x[R], xo[R];
@@ -1488,11 +1496,10 @@ cudaError_t panel_smem_limit() {
   return err;
 }
 
-// Factor the panel A[k0:n, k0:k0+nb), apply its interchanges to every other
-// column and solve U12 = L11^{-1} A12 for the columns [k0 + nb, trsm_end).
+// Factor the panel A[k0:n, k0:k0+nb).
 template <typename T>
-static cudaError_t lu_leaf(BOp<T> A, int n, int k0, int nb, int trsm_end, int batch, int* ipiv, int* info,
-                           unsigned* dev_err, int G, const LuWork& w, cudaStream_t st, Prof* pf) {
+static cudaError_t lu_panel(BOp<T> A, int n, int k0, int nb, int batch, int* ipiv, int* info,
+                            unsigned* dev_err, int G, const LuWork& w, cudaStream_t st, Prof* pf) {
   constexpr double F = fma_flops<T>();
   const int nb0 = LuNB<T>::NB;
   cudaError_t e;
@@ -1567,25 +1574,185 @@ static cudaError_t lu_leaf(BOp<T> A, int n, int k0, int nb, int trsm_end, int ba
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (pf) pf->end(K_LU_PANEL, pfl, st);
-  if (n > nb) {
-    const int ncols = n - nb;
-    // eight threads per column have the shortest chain; four issue an eighth
-    // less once the FP64 pipe is full whatever the split (4096 matrices of
-    // order 196: 534 us against 570; 1024 of order 224: 108 against 103)
-    const bool many = (int64_t)((ncols + 31) / 32) * batch >= 48 * device_sms();
-    const int cw = many ? 32 : 16;
-    const dim3 grid(std::min((ncols + cw - 1) / cw, 4096), batch);
-    if (pf) {
-      pf->begin(st);
-      pf->note(nb, ncols, nb, batch);
-    }
-    if (many) k_laswp_trsm<T, LuNB<T>::NB, 4><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, trsm_end);
-    else k_laswp_trsm<T, LuNB<T>::NB, 8><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, trsm_end);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (pf) pf->end(K_LASWP_TRSM, F * 0.5 * nb * (nb - 1) * (double)std::max(0, trsm_end - k0 - nb) * batch, st);
-  }
   return cudaSuccess;
 }
+
+// Apply the interchanges of the panel at k0 to the columns `cols` (none of them
+// the panel's) and solve U12 = L11^{-1} A12 for those in [k0 + nb, trsm_end).
+template <typename T>
+static cudaError_t lu_swap(BOp<T> A, int n, int k0, int nb, LuCols cols, int trsm_end, int batch, const int* ipiv,
+                           cudaStream_t st, Prof* pf) {
+  const int ncols = cols.left + cols.right;
+  if (ncols <= 0) return cudaSuccess;
+  // eight threads per column have the shortest chain; four issue an eighth
+  // less once the FP64 pipe is full whatever the split (4096 matrices of
+  // order 196: 534 us against 570; 1024 of order 224: 108 against 103)
+  const bool many = (int64_t)((ncols + 31) / 32) * batch >= 48 * device_sms();
+  const int cw = many ? 32 : 16;
+  const dim3 grid(std::min((ncols + cw - 1) / cw, 4096), batch);
+  if (pf) {
+    pf->begin(st);
+    pf->note(nb, ncols, nb, batch);
+  }
+  if (many) k_laswp_trsm<T, LuNB<T>::NB, 4><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, cols, trsm_end);
+  else k_laswp_trsm<T, LuNB<T>::NB, 8><<<grid, 128, 0, st>>>(A, n, k0, nb, ipiv, cols, trsm_end);
+  const int solved = std::max(0, std::min(trsm_end, cols.first + cols.right) - cols.first);
+  if (pf) pf->end(K_LASWP_TRSM, fma_flops<T>() * 0.5 * nb * (nb - 1) * (double)solved * batch, st);
+  return cudaGetLastError();
+}
+
+// A[k0 + nb : n, j0 : j0 + nj) -= A[k0 + nb : n, panel] U12, leaving spare SMs
+template <typename T>
+static cudaError_t lu_update(BOp<T> A, int n, int k0, int nb, int j0, int nj, int spare, int batch, cudaStream_t st,
+                             Prof* pf) {
+  if (n - k0 - nb <= 0 || nj <= 0) return cudaSuccess;
+  GemmArgs<T> g;
+  g.M = n - k0 - nb; g.N = nj; g.K = nb; g.batch = batch;
+  g.A = shifted(A, (int64_t)(k0 + nb) + (int64_t)k0 * A.ld);
+  g.B = shifted(A, (int64_t)k0 + (int64_t)j0 * A.ld);
+  g.C = shifted(A, (int64_t)(k0 + nb) + (int64_t)j0 * A.ld);
+  g.alpha = T(-1.0); g.beta = T(1.0);
+  g.spare_sms = spare;
+  return gemm(g, st, pf);
+}
+
+// SMs that the next panels of `batch` matrices (of `rows` rows) take when they
+// are factored beside the rest of the update (rows x cols, inner dimension nb), or
+// 0 when they are not.  Splitting the update costs two short launches and
+// two events a panel (~20 us), so the rest has to be worth hiding: from 2e6
+// multiply-adds on (builds at 2e6 / 5e6 / 1e7 / 2e7 / never: Helmholtz 93.1 /
+// 93.5 / 93.6 / 94.0 / 94.7 ms, adaptive 71.4 / 71.7 / 71.9 / 72.0 / 73.5, 3D elliptic 76.3 at
+// all of them / 82.0).  Panels on more than half of the SMs leave the update
+// too few (on up to all: Helmholtz 95.3, 3D elliptic 80.6).
+template <typename T>
+int panel_ahead_sms(int rows, int cols, int nb, int batch) {
+  if (cols <= 0 || (double)rows * cols * nb * batch < 2e6 || batch > device_sms() / 2) return 0;
+  const int cr = lu_tune(TUNE_LU_CLUSTER_PANEL) ? panel_reg_size<T>(rows, batch) : 0;
+  return cr > 0 && (int64_t)cr * batch <= device_sms() / 2 ? cr * batch : 0;
+}
+
+namespace {
+
+// A second stream for the panels that are factored ahead of the trailing
+// updates, with the events that order it against the caller's stream.  Idle
+// ones are kept (at most kSideKeep a device; lu_side_trim destroys them): making
+// one takes tens of microseconds.  A released one is joined to the stream
+// that used it, so its next user inherits no hazard, at worst a short wait.
+struct SideStream {
+  cudaStream_t st = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  int dev = 0;
+  void destroy() {
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
+    if (st) cudaStreamDestroy(st);
+    st = nullptr;
+  }
+};
+constexpr size_t kSideKeep = 8;
+std::mutex g_side_mu;
+std::vector<SideStream> g_side;
+
+bool side_take(SideStream* out) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError(), false;
+  {
+    std::lock_guard<std::mutex> lk(g_side_mu);
+    for (size_t i = 0; i < g_side.size(); ++i)
+      if (g_side[i].dev == dev) {
+        *out = g_side[i];
+        g_side.erase(g_side.begin() + i);
+        return true;
+      }
+  }
+  SideStream s;
+  s.dev = dev;
+  int lo = 0, hi = 0;
+  // the highest priority: a waiting panel takes the first SMs that come free
+  if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&s.st, cudaStreamNonBlocking, hi) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    s.destroy();
+    return false;
+  }
+  *out = s;
+  return true;
+}
+
+void side_give(SideStream s) {
+  {
+    std::lock_guard<std::mutex> lk(g_side_mu);
+    size_t kept = 0;
+    for (const SideStream& o : g_side) kept += o.dev == s.dev;
+    if (kept < kSideKeep) {
+      g_side.push_back(s);
+      return;
+    }
+  }
+  s.destroy();
+}
+
+}  // namespace
+
+// Destroy the current device's idle side streams.
+void lu_side_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  std::lock_guard<std::mutex> lk(g_side_mu);
+  for (size_t i = g_side.size(); i-- > 0;)
+    if (g_side[i].dev == dev) {
+      g_side[i].destroy();
+      g_side.erase(g_side.begin() + i);
+    }
+}
+
+// The blocked factorisation of one range with its panels ahead: panel k + 1
+// needs only its own columns of panel k's update, so those are done first and
+// the panel is factored on the side stream while the rest of the update
+// runs (on the SMs that the panel leaves: a tensor-core product has one CTA per
+// SM for its whole duration, which a late panel would wait for and an early
+// one would stretch).  A panel of few matrices is a serial chain on a few SMs
+// (115 us for 6912 rows on 16); the update of the others takes as long.  The same
+// operations on the same entries; only where a product runs may change, as
+// the two parts of an update are routed by their own sizes.
+struct LookAhead {
+  cudaStream_t main;
+  SideStream side;
+  bool tried = false, open = false;   // open: work on the side stream that main has not waited for
+  explicit LookAhead(cudaStream_t st) : main(st) {}
+  ~LookAhead() {
+    if (open) wait();
+    if (side.st) side_give(side);
+  }
+  bool available() {
+    if (!tried) {
+      tried = true;
+      // a stream that is being captured would take the side stream, and whoever
+      // takes it next, into the capture
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(main, &cap) != cudaSuccess) cudaGetLastError();
+      else if (cap == cudaStreamCaptureStatusNone) side_take(&side);
+    }
+    return side.st != nullptr;
+  }
+  cudaError_t begin() {   // side waits for main
+    cudaError_t e = cudaEventRecord(side.fork, main);
+    return e != cudaSuccess ? e : cudaStreamWaitEvent(side.st, side.fork, 0);
+  }
+  cudaError_t end() {
+    open = true;
+    return cudaEventRecord(side.join, side.st);
+  }
+  cudaError_t wait() {   // main waits for side
+    open = false;
+    return cudaStreamWaitEvent(main, side.join, 0);
+  }
+};
 
 template <typename T>
 static cudaError_t rtrsm_lower(BOp<T> LU, BOp<T> X, int p0, int n1, int nrhs, int batch, cudaStream_t st,
@@ -1594,31 +1761,40 @@ static cudaError_t rtrsm_lower(BOp<T> LU, BOp<T> X, int p0, int n1, int nrhs, in
 // Recursive LU with partial pivoting of the columns [c0, c1) (rows c0..n):
 // factor the left half, U12 = L11^{-1} A12 by the recursive triangular
 // solve, A22 -= A21 U12 as one product of inner dimension ~(c1 - c0) / 2,
-// factor the right half.  Ranges of at most 4 panels are factored blocked
+// factor the right half.  Ranges of at most base_w columns are factored blocked
 // right-looking (panel, interchanges + U12 within the range, update of the
-// range's remaining columns), which keeps the launch count of the blocked
-// algorithm; so are whole matrices when there are few of them (base_w = n).  The same pivots and operations as the blocked right-looking
-// order; the bulk of the trailing updates becomes a few large-K products
-// (on the tensor cores) instead of n / nb products of inner dimension nb.
+// range's remaining columns), which has fewer launches; so are whole matrices
+// when there are few of them (base_w = n).  The same pivots and operations as
+// the blocked right-looking order; of larger matrices the bulk of the trailing
+// updates becomes a few large-K products instead of n / nb products of inner
+// dimension nb.
 template <typename T>
 static cudaError_t rgetrf(BOp<T> A, int n, int c0, int c1, int base_w, int nb0, int batch, int* ipiv, int* info,
                           unsigned* dev_err, int G, const LuWork& w, cudaStream_t st, Prof* pf) {
   const int wdt = c1 - c0;
   cudaError_t e;
   if (wdt <= base_w) {
+    LookAhead la(st);
     for (int k0 = c0; k0 < c1; k0 += nb0) {
-      const int nb = std::min(nb0, c1 - k0);
-      if ((e = lu_leaf<T>(A, n, k0, nb, c1, batch, ipiv, info, dev_err, G, w, st, pf)) != cudaSuccess) return e;
-      const int m2 = n - k0 - nb, n2 = c1 - k0 - nb;
-      if (m2 > 0 && n2 > 0) {
-        GemmArgs<T> g;
-        g.M = m2; g.N = n2; g.K = nb; g.batch = batch;
-        g.A = shifted(A, (int64_t)(k0 + nb) + (int64_t)k0 * A.ld);
-        g.B = shifted(A, (int64_t)k0 + (int64_t)(k0 + nb) * A.ld);
-        g.C = shifted(A, (int64_t)(k0 + nb) + (int64_t)(k0 + nb) * A.ld);
-        g.alpha = T(-1.0); g.beta = T(1.0);
-        if ((e = gemm(g, st, pf)) != cudaSuccess) return e;
+      const int nb = std::min(nb0, c1 - k0), k1 = k0 + nb, nb1 = std::min(nb0, c1 - k1);
+      if (la.open) e = la.wait();
+      else e = lu_panel<T>(A, n, k0, nb, batch, ipiv, info, dev_err, G, w, st, pf);
+      if (e != cudaSuccess) return e;
+      const int sms = panel_ahead_sms<T>(n - k1, c1 - k1 - nb1, nb, batch);
+      if (sms == 0 || !la.available()) {
+        if ((e = lu_swap<T>(A, n, k0, nb, LuCols{k0, k1, n - k1}, c1, batch, ipiv, st, pf)) != cudaSuccess) return e;
+        if ((e = lu_update<T>(A, n, k0, nb, k1, c1 - k1, 0, batch, st, pf)) != cudaSuccess) return e;
+        continue;
       }
+      const int k2 = k1 + nb1;
+      if ((e = lu_swap<T>(A, n, k0, nb, LuCols{0, k1, nb1}, c1, batch, ipiv, st, pf)) != cudaSuccess) return e;
+      if ((e = lu_update<T>(A, n, k0, nb, k1, nb1, 0, batch, st, pf)) != cudaSuccess) return e;
+      if ((e = la.begin()) != cudaSuccess) return e;
+      e = lu_panel<T>(A, n, k1, nb1, batch, ipiv, info, dev_err, G, w, la.side.st, pf);
+      const cudaError_t e2 = la.end();
+      if (e != cudaSuccess || e2 != cudaSuccess) return e != cudaSuccess ? e : e2;
+      if ((e = lu_swap<T>(A, n, k0, nb, LuCols{k0, k2, n - k2}, c1, batch, ipiv, st, pf)) != cudaSuccess) return e;
+      if ((e = lu_update<T>(A, n, k0, nb, k2, c1 - k2, sms, batch, st, pf)) != cudaSuccess) return e;
     }
     return cudaSuccess;
   }

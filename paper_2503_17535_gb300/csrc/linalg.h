@@ -92,6 +92,7 @@ struct GemmArgs {
   // A enters conjugate-transposed: the (i, l) entry of the product's left
   // factor is conj(A(acol(l), arow(i))) (adjoint solves)
   bool ta = false;
+  int spare_sms = 0;   // SMs that other work beside this product keeps busy
   __device__ T a_at(const T* A, int b, int i, int l) const {
     if (!ta) return A[(int64_t)arow.at(b, i) + (int64_t)acol.at(b, l) * this->A.ld];
     return conj_of(A[(int64_t)acol.at(b, l) + (int64_t)arow.at(b, i) * this->A.ld]);
@@ -179,6 +180,10 @@ size_t lu_pub_bytes(int n, int batch, int G);
 template <typename T>
 cudaError_t getrf(BOp<T> A, int n, int batch, int* ipiv, int* perm, int* info, unsigned* dev_err,
                   int G, const LuWork& w, cudaStream_t st, Prof* pf);
+
+// getrf keeps up to eight idle streams a device for panels that run beside the
+// trailing updates; this destroys the current device's.
+void lu_side_trim();
 
 // Solve (P^T L U) X = R in place for X given perm-gathered rows:
 //   permute_rows: X(i, j) = R(perm[i], j)

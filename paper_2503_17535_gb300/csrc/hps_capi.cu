@@ -706,7 +706,8 @@ hps_status solve_multi_impl(const std::vector<int>& idx, hps_handle* const* hs, 
       tk.n_ext = Lv.n_ext; tk.n_int = Lv.n_int; tk.nrhs = nrhs[i];
       tk.tile0 = grp.tiles;
       tk.elem0 = grp.elems;
-      grp.tiles += (int64_t)Lv.nmerge * ((Lv.n_int + 31) / 32) * nrhs[i];
+      tk.cg = down_groups(((int64_t)Lv.nmerge * Lv.n_int + 31) / 32 * nrhs[i], Lv.n_ext, 8);
+      grp.tiles += down_task_row_tiles(tk) * nrhs[i];
       grp.elems += (int64_t)Lv.nmerge * Lv.nch * Lv.nbc * nrhs[i];
       if (grp.n == kMaxGroup) HPS_CUDA(flush_down());
     }

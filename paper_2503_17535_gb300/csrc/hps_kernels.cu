@@ -3,6 +3,8 @@
 // dense FP64 work (LU, triangular solves, GEMM) lives in linalg.cu.
 #include "hps_kernels.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 namespace hps {
@@ -405,70 +407,142 @@ cudaError_t merge_gather_h(const T* hc, int nmerge, int nch, int nbc, int n_ext,
 
 // ------------------------------------------------------------- downward ----
 
-// gint(:, c) = -(X_C gpar(:, c) + xpart(:, c)); a warp per (merge, row, rhs)
-// block of rows: each thread owns one row and walks the columns.
-template <typename T>
-__global__ void k_down_gint(const T* X, const T* xp, const T* gpar, int nmerge, int n_ext, int n_int,
-                            int nrhs, T* gint) {
-  const int64_t total = (int64_t)nmerge * n_int * nrhs;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e % n_int);
-    const int64_t bc = e / n_int;
-    const int c = (int)(bc % nrhs);
-    const int64_t b = bc / nrhs;
-    const T* Xb = X + b * (int64_t)n_int * (n_ext + 1);
-    const T* g = gpar + b * (int64_t)n_ext * nrhs + (int64_t)c * n_ext;
-    T acc = xp ? xp[b * (int64_t)n_int * nrhs + r + (int64_t)c * n_int] : Xb[r + (int64_t)n_ext * n_int];
-    for (int j = 0; j < n_ext; ++j) acc = fmac(acc, Xb[r + (int64_t)j * n_int], g[j]);
-    gint[b * (int64_t)n_int * nrhs + r + (int64_t)c * n_int] = -acc;
+// gint(:, c) = -(X_C gpar(:, c) + xpart(:, c)): a lane per row (the rows of all
+// merges in one sequence), NC right-hand sides at a time, the columns dealt to
+// CG warps of a CTA and, with CL, in ranges to the CS CTAs of a cluster; the
+// partial sums are added in shared memory in a fixed order, so that the
+// result does not depend on scheduling.
+//
+// Bound by the FP64 pipe when there are many rows (two multiply-adds per clock
+// and SM: 86 us for 205 MB of complex entries and one right-hand side, which
+// memory would deliver in 31), by the latency of a row's loads when there are
+// few; the column groups spread those over more warps, and clusters of small
+// CTAs over all SMs while there are less than two 32-row tiles per SM (112 tiles of
+// 3584 complex columns 127 -> 117 us, 224 of 1792 123 -> 105; with more tiles, or
+// very long rows, the ranges cost locality: 432 real tiles 94 -> 137, 216 of
+// 13824 columns 246 -> 265).  With one warp per 32 rows up to 255 columns, as
+// before, 64 real merges of 176 columns took 80 us, now 12.
+template <typename T, int CG, int NC, bool CL>
+__global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X, const T* xp, const T* gpar,
+                                                                       int64_t rows, int n_ext, int n_int, int nrhs,
+                                                                       int CS, T* gint) {
+  namespace cg_ = cooperative_groups;
+  constexpr int NW = CG < 4 ? 4 : CG;
+  __shared__ T part[CG > 1 ? NW : 1][NC][33];
+  __shared__ T sums[CL ? 8 : 1][NC][33];   // of the cluster's CTAs
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cg = w % CG;
+  const int rank = CL ? (int)blockIdx.x % CS : 0;
+  const int64_t R = ((int64_t)(CL ? blockIdx.x / CS : blockIdx.x) * (NW / CG) + w / CG) * 32 + lane;
+  const int c0 = blockIdx.y * NC;
+  const bool live = R < rows;
+  const int64_t b = live ? R / n_int : 0;
+  const int r = live ? (int)(R % n_int) : 0;
+  const T* x = X + b * (int64_t)n_int * (n_ext + 1) + r;
+  const T* g = gpar + (b * nrhs + c0) * (int64_t)n_ext;
+  int64_t go[NC];   // columns beyond the last repeat it
+#pragma unroll
+  for (int c = 0; c < NC; ++c) go[c] = (int64_t)min(c, nrhs - 1 - c0) * n_ext;
+  T acc[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) acc[c] = T(0.0);
+  if (live) {
+    const int j1 = CL ? (int)((int64_t)n_ext * (rank + 1) / CS) : n_ext;   // a cluster's CTAs take ranges of columns
+#pragma unroll 8
+    for (int j = (CL ? (int)((int64_t)n_ext * rank / CS) : 0) + cg; j < j1; j += CG) {
+      const T xv = x[(int64_t)j * n_int];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], xv, g[go[c] + j]);
+    }
+  }
+  if constexpr (CG > 1) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) part[w][c][lane] = acc[c];
+    __syncthreads();
+    if (cg == 0) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 1; k < CG; ++k) acc[c] = acc[c] + part[w + k][c][lane];
+    }
+  }
+  if constexpr (CL) {
+    cg_::cluster_group cl = cg_::this_cluster();
+    if (w == 0) {
+      T* first = cl.map_shared_rank(&sums[0][0][0], 0);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) first[(rank * NC + c) * 33 + lane] = acc[c];
+    }
+    cl.sync();
+    if (rank != 0) return;
+    if (w == 0)
+      for (int k = 1; k < CS; ++k)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c] = acc[c] + sums[k][c][lane];
+  }
+  if (cg != 0 || !live) return;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    if (c0 + c >= nrhs) break;
+    const T s = xp ? xp[(b * nrhs + c0 + c) * (int64_t)n_int + r] : x[(int64_t)n_ext * n_int];
+    gint[(b * nrhs + c0 + c) * (int64_t)n_int + r] = -(s + acc[c]);
   }
 }
 
-// Same product for levels with few long rows (the top merges): a CTA holds
-// 32 rows x CG column groups; each warp reads 32 consecutive rows of one
-// column (coalesced), the CG partial sums are added in shared memory in a
-// fixed order, so the result does not depend on scheduling.
-template <typename T, int CG>
-__global__ void __launch_bounds__(32 * CG) k_down_gint_split(const T* X, const T* xp, const T* gpar, int nmerge,
-                                                         int n_ext, int n_int, int nrhs, T* gint) {
-  __shared__ T part[CG][33];
-  const int lane = threadIdx.x, cg = threadIdx.y;
-  const int r = blockIdx.x * 32 + lane;
-  const int64_t bc = blockIdx.y;  // merge * nrhs + rhs
-  const int c = (int)(bc % nrhs);
-  const int64_t b = bc / nrhs;
-  const T* Xb = X + b * (int64_t)n_int * (n_ext + 1);
-  const T* g = gpar + b * (int64_t)n_ext * nrhs + (int64_t)c * n_ext;
-  T acc = T(0.0);
-  if (r < n_int) {
-    int j = cg;
-#pragma unroll 4
-    for (; j < n_ext; j += CG) acc = fmac(acc, Xb[r + (int64_t)j * n_int], g[j]);
-  }
-  part[cg][lane] = acc;
-  __syncthreads();
-  if (cg == 0 && r < n_int) {
-    T s = xp ? xp[b * (int64_t)n_int * nrhs + r + (int64_t)c * n_int] : Xb[r + (int64_t)n_ext * n_int];
-    for (int k = 0; k < CG; ++k) s = s + part[k][lane];
-    gint[b * (int64_t)n_int * nrhs + r + (int64_t)c * n_int] = -s;
+// right-hand sides a thread takes at a time: at most `most`, in even groups
+inline int rhs_group(int nrhs, int most) {
+  const int groups = (nrhs + most - 1) / most;
+  return (nrhs + groups - 1) / groups;
+}
+
+template <typename T, int CG, int NC, bool CL>
+cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t rows, int n_ext, int n_int, int nrhs,
+                                int cs, T* gint, cudaStream_t st) {
+  constexpr int NW = CG < 4 ? 4 : CG;
+  const int per = 32 * (NW / CG);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((rows + per - 1) / per * cs), (nrhs + NC - 1) / NC);
+  cfg.blockDim = dim3(32 * NW);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = CL ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_down_gint<T, CG, NC, CL>, X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint);
+}
+
+template <typename T, int CG, bool CL>
+cudaError_t launch_down_gint_cg(const T* X, const T* xp, const T* gpar, int64_t rows, int n_ext, int n_int, int nrhs,
+                                int cs, T* gint, int nc, cudaStream_t st) {
+  switch (nc) {
+    case 1: return launch_down_gint_nc<T, CG, 1, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
+    case 2: return launch_down_gint_nc<T, CG, 2, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
+    case 3: return launch_down_gint_nc<T, CG, 3, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
+    default: return launch_down_gint_nc<T, CG, 4, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
   }
 }
 
-// Rows of work below which the split kernel is used (about two resident
-// threads per SM lane of the whole GPU would otherwise be idle).
-constexpr int64_t kDownSplitRows = 1 << 17;
-
 template <typename T>
-void launch_down_gint(const T* X, const T* xp, const T* gpar, int nmerge, int n_ext, int n_int, int nrhs,
-                      T* gint, cudaStream_t st) {
-  const int64_t rows = (int64_t)nmerge * n_int * nrhs;
-  if (rows < kDownSplitRows && n_ext >= 256 && (int64_t)nmerge * nrhs <= 65535) {
-    dim3 grid((n_int + 31) / 32, nmerge * nrhs);
-    k_down_gint_split<T, 16><<<grid, dim3(32, 16), 0, st>>>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint);
-  } else {
-    k_down_gint<T><<<grid_for(rows, 128), 128, 0, st>>>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint);
-  }
+cudaError_t launch_down_gint(const T* X, const T* xp, const T* gpar, int nmerge, int n_ext, int n_int, int nrhs,
+                             T* gint, cudaStream_t st) {
+  const int64_t rows = (int64_t)nmerge * n_int, tiles = (rows + 31) / 32;
+  // fewer right-hand sides per thread where the row tiles would not go round the
+  // SMs two and a half times (112 tiles, eight right-hand sides, real: 182 us in
+  // groups of four, 105 one by one; 224 tiles: 96 in groups of four, 115 of three)
+  int most = 4;
+  while (most > 1 && 2 * tiles * ((nrhs + most - 1) / most) < 5 * device_sms()) --most;
+  const int nc = rhs_group(nrhs, most);
+  const int64_t warps = tiles * ((nrhs + nc - 1) / nc);
+  const bool cluster = warps < 2 * device_sms() && n_ext < 8192;
+  const int cg = down_groups(warps, n_ext, cluster ? 32 : 16);
+  if (cg == 1) return launch_down_gint_cg<T, 1, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
+  if (cg == 2) return launch_down_gint_cg<T, 2, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
+  if (cg == 4) return launch_down_gint_cg<T, 4, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
+  if (cluster) return launch_down_gint_cg<T, 4, true>(X, xp, gpar, rows, n_ext, n_int, nrhs, cg / 4, gint, nc, st);
+  if (cg == 8) return launch_down_gint_cg<T, 8, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
+  return launch_down_gint_cg<T, 16, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
 }
 
 template <typename T>
@@ -497,10 +571,9 @@ cudaError_t down_level(const T* X, const T* xp, const T* gpar, int nmerge, int n
                        cudaStream_t st, Prof* pf) {
   const double F = sizeof(T) == sizeof(cplx) ? 8.0 : 2.0;
   if (pf) pf->begin(st);
-  launch_down_gint<T>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint, st);
-  if (pf) pf->end(K_DOWN, F * (double)nmerge * n_int * n_ext * nrhs, st);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_down_gint<T>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint, st);
   if (e != cudaSuccess) return e;
+  if (pf) pf->end(K_DOWN, F * (double)nmerge * n_int * n_ext * nrhs, st);
   if (pf) pf->begin(st);
   k_down_children<T><<<grid_for((int64_t)nmerge * nch * nbc * nrhs), 256, 0, st>>>(
       gpar, gint, nmerge, nch, nbc, n_ext, n_int, nrhs, ext, var, gchild);
@@ -513,9 +586,9 @@ cudaError_t down_gint(const T* X, const T* xp, const T* gpar, int nmerge, int n_
                       T* gint, cudaStream_t st, Prof* pf) {
   const double F = sizeof(T) == sizeof(cplx) ? 8.0 : 2.0;
   if (pf) pf->begin(st);
-  launch_down_gint<T>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint, st);
+  const cudaError_t e = launch_down_gint<T>(X, xp, gpar, nmerge, n_ext, n_int, nrhs, gint, st);
   if (pf) pf->end(K_DOWN, F * (double)nmerge * n_int * n_ext * nrhs, st);
-  return cudaGetLastError();
+  return e;
 }
 
 template <typename T>
@@ -528,35 +601,75 @@ cudaError_t down_children(const T* gpar, const T* gint, int nmerge, int nch, int
   return cudaGetLastError();
 }
 
+// The row of the leaf's solution map that a node takes: of Y for ItI, of -Y at
+// interior and of P at boundary nodes for DtN.  For real data the two are one
+// pointer and stride, so that a warp with nodes of both kinds (every warp of a 2D
+// leaf) walks one loop.
 template <typename T>
-__global__ void k_leaf_output(LeafConsts k, int64_t nl, int nrhs, const T* X, const T* xp, const T* g,
-                              T* u, bool iti) {
-  const int64_t total = (int64_t)nrhs * nl * k.npts;
+struct LeafRow {
+  const double* p;   // real rows: entry j at p[j ld]
+  const T* x;        // complex rows
+  int64_t ld;
+  int r;             // row of Y
+  bool edge, negate;
+  __device__ LeafRow(const LeafConsts& k, bool iti, int node, const T* Xl, int xrows) {
+    const int pr = iti ? -1 : k.prow[node];
+    edge = pr >= 0;
+    negate = !iti && !edge;
+    r = iti ? node : edge ? 0 : k.iidx[node];
+    ld = edge ? k.ne : xrows;
+    x = Xl + r;
+    if constexpr (sizeof(T) == sizeof(double)) p = edge ? k.P + pr : Xl + r;
+    else p = k.P + pr;
+  }
+  __device__ T at(int j) const {
+    if constexpr (sizeof(T) == sizeof(double)) return p[j * ld];
+    else return edge ? T(p[j * ld]) : x[j * ld];
+  }
+};
+
+// u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides, so
+// that an entry of Y serves NC multiply-adds.  Bound by the FP64 pipe (385 us
+// for 4096 complex leaves of 256 x 56, of which the pipe needs 392 at its nominal
+// rate); one right-hand side per thread read every entry from L2 again for
+// each and walked a warp's boundary and interior nodes one after the other: 1533
+// us for eight real ones, now 784.
+template <typename T, int NC>
+__global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, int nrhs, const T* X, const T* xp,
+                                                     const T* g, T* u, bool iti) {
+  const int64_t total = (int64_t)((nrhs + NC - 1) / NC) * nl * k.npts;
   const int xrows = iti ? k.npts : k.ni;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int node = (int)(e % k.npts);
     const int64_t lc = e / k.npts;
     const int64_t leaf = lc % nl;
-    const int c = (int)(lc / nl);
-    const T* gl = g + (leaf * nrhs + c) * (int64_t)k.nb;
+    const int c0 = (int)(lc / nl) * NC;
+    const T* gl = g + (leaf * nrhs + c0) * (int64_t)k.nb;
     const T* Xl = X + leaf * (int64_t)xrows * (k.nb + 1);
-    T acc = T(0.0);
-    if (iti) {
-      acc = xp ? xp[(leaf * nrhs + c) * (int64_t)xrows + node] : Xl[node + (int64_t)k.nb * xrows];
-      for (int j = 0; j < k.nb; ++j) acc = fmac(acc, Xl[node + (int64_t)j * xrows], gl[j]);
-    } else {
-      const int pr = k.prow[node];
-      if (pr >= 0) {
-        for (int j = 0; j < k.nb; ++j) acc = fmac(acc, T(k.P[pr + (int64_t)j * k.ne]), gl[j]);
-      } else {
-        const int r = k.iidx[node];
-        acc = xp ? xp[(leaf * nrhs + c) * (int64_t)xrows + r] : Xl[r + (int64_t)k.nb * xrows];
-        for (int j = 0; j < k.nb; ++j) acc = fmac(acc, Xl[r + (int64_t)j * xrows], gl[j]);
-        acc = -acc;
-      }
+    int go[NC];   // columns beyond the last repeat it
+    T acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) go[c] = min(c, nrhs - 1 - c0) * k.nb;
+    const LeafRow<T> row(k, iti, node, Xl, xrows);
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      acc[c] = row.edge ? T(0.0)
+               : xp     ? xp[(leaf * nrhs + min(c0 + c, nrhs - 1)) * (int64_t)xrows + row.r]
+                        : Xl[row.r + (int64_t)k.nb * xrows];
+#pragma unroll 4
+    for (int j = 0; j < k.nb; ++j) {
+      const T x = row.at(j);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], x, gl[go[c] + j]);
     }
-    u[e] = acc;
+    if (row.negate) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = -acc[c];
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      if (c0 + c < nrhs) u[((c0 + c) * nl + leaf) * k.npts + node] = acc[c];
   }
 }
 
@@ -565,7 +678,14 @@ cudaError_t leaf_output(const LeafConsts& k, int64_t nl, int nrhs, const T* X, c
                         T* u, bool iti, cudaStream_t st, Prof* pf) {
   const double F = sizeof(T) == sizeof(cplx) ? 8.0 : 2.0;
   if (pf) pf->begin(st);
-  k_leaf_output<T><<<grid_for((int64_t)nrhs * nl * k.npts), 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti);
+  const int nc = rhs_group(nrhs, 4);
+  const int grid = grid_for((int64_t)((nrhs + nc - 1) / nc) * nl * k.npts);
+  switch (nc) {
+    case 1: k_leaf_output<T, 1><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
+    case 2: k_leaf_output<T, 2><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
+    case 3: k_leaf_output<T, 3><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
+    default: k_leaf_output<T, 4><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
+  }
   if (pf) pf->end(K_DOWN, F * (double)nrhs * nl * k.npts * k.nb, st);
   return cudaGetLastError();
 }
@@ -610,37 +730,37 @@ cudaError_t scale_copy(const T* src, T* dst, int64_t n, double alpha, cudaStream
 
 // ------------------------------------------------- grouped downward pass ----
 
-// gint = -(X_C gpar + x) for one 32-row tile of one merge and right-hand
-// side of one task per CTA: 32 lanes own the rows, 8 warps split the columns
-// (coalesced 32-row column reads), partial sums added in shared memory in a
-// fixed order.
+// gint = -(X_C gpar + x) for the rows of all merges of a task and one right-hand
+// side: as k_down_gint, with eight warps a CTA of which tk.cg share 32 rows.
 template <typename T>
 __global__ void __launch_bounds__(256) k_down_gint_group(DownGroup<T> grp) {
   __shared__ T part[8][33];
-  const int lane = threadIdx.x, cg = threadIdx.y;
+  const int lane = threadIdx.x, w = threadIdx.y;
   const int64_t tile = blockIdx.x;
   int ti = 0;
   while (ti + 1 < grp.n && grp.t[ti + 1].tile0 <= tile) ++ti;
   const DownTask<T>& tk = grp.t[ti];
-  const int rtiles = (tk.n_int + 31) / 32;
+  const int CG = tk.cg, cg = w & (CG - 1), n_int = tk.n_int, n_ext = tk.n_ext, nrhs = tk.nrhs;
+  const int64_t rows = (int64_t)tk.nmerge * n_int, rtiles = down_task_row_tiles(tk);
   const int64_t loc = tile - tk.tile0;
-  const int r = (int)(loc % rtiles) * 32 + lane;
-  const int64_t bc = loc / rtiles;
-  const int c = (int)(bc % tk.nrhs);
-  const int64_t b = bc / tk.nrhs;
-  const T* Xb = tk.X + b * (int64_t)tk.n_int * (tk.n_ext + 1);
-  const T* g = tk.gpar + b * (int64_t)tk.n_ext * tk.nrhs + (int64_t)c * tk.n_ext;
+  const int64_t R = (loc % rtiles * (8 / CG) + w / CG) * 32 + lane;
+  const int c = (int)(loc / rtiles);
+  const bool live = R < rows;
+  const int64_t b = live ? R / n_int : 0;
+  const int r = live ? (int)(R % n_int) : 0;
+  const T* x = tk.X + b * (int64_t)n_int * (n_ext + 1) + r;
+  const T* g = tk.gpar + (b * nrhs + c) * (int64_t)n_ext;
   T acc = T(0.0);
-  if (r < tk.n_int) {
+  if (live) {
 #pragma unroll 4
-    for (int j = cg; j < tk.n_ext; j += 8) acc = fmac(acc, Xb[r + (int64_t)j * tk.n_int], g[j]);
+    for (int j = cg; j < n_ext; j += CG) acc = fmac(acc, x[(int64_t)j * n_int], g[j]);
   }
-  part[cg][lane] = acc;
+  part[w][lane] = acc;
   __syncthreads();
-  if (cg == 0 && r < tk.n_int) {
-    T s = Xb[r + (int64_t)tk.n_ext * tk.n_int];
-    for (int k = 0; k < 8; ++k) s = s + part[k][lane];
-    tk.gint[b * (int64_t)tk.n_int * tk.nrhs + r + (int64_t)c * tk.n_int] = -s;
+  if (cg == 0 && live) {
+    T s = x[(int64_t)n_ext * n_int];
+    for (int k = 0; k < CG; ++k) s = s + part[w + k][lane];
+    tk.gint[(b * nrhs + c) * (int64_t)n_int + r] = -s;
   }
 }
 
@@ -693,21 +813,11 @@ __global__ void k_leaf_output_group(LeafGroup<T> grp) {
     const int xrows = grp.iti ? k.npts : k.ni;
     const T* gl = tk.g + (leaf * tk.nrhs + c) * (int64_t)k.nb;
     const T* Xl = tk.X + leaf * (int64_t)xrows * (k.nb + 1);
-    T acc = T(0.0);
-    if (grp.iti) {
-      acc = Xl[node + (int64_t)k.nb * xrows];
-      for (int j = 0; j < k.nb; ++j) acc = fmac(acc, Xl[node + (int64_t)j * xrows], gl[j]);
-    } else {
-      const int pr = k.prow[node];
-      if (pr >= 0) {
-        for (int j = 0; j < k.nb; ++j) acc = fmac(acc, T(k.P[pr + (int64_t)j * k.ne]), gl[j]);
-      } else {
-        const int r = k.iidx[node];
-        acc = Xl[r + (int64_t)k.nb * xrows];
-        for (int j = 0; j < k.nb; ++j) acc = fmac(acc, Xl[r + (int64_t)j * xrows], gl[j]);
-        acc = -acc;
-      }
-    }
+    const LeafRow<T> row(k, grp.iti, node, Xl, xrows);
+    T acc = row.edge ? T(0.0) : Xl[row.r + (int64_t)k.nb * xrows];
+#pragma unroll 4
+    for (int j = 0; j < k.nb; ++j) acc = fmac(acc, row.at(j), gl[j]);
+    if (row.negate) acc = -acc;
     tk.u[le] = acc;
   }
 }

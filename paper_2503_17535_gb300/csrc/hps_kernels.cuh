@@ -107,6 +107,15 @@ cudaError_t leaf_output(const LeafConsts& k, int64_t nl, int nrhs, const T* X, c
 // task and every CTA or thread finds its task from the prefix offsets.
 constexpr int kMaxGroup = 24;
 
+// column groups: enough for kDownWarps warps in all (eight a scheduler), while
+// each keeps eight columns
+constexpr int64_t kDownWarps = 4096;
+inline int down_groups(int64_t warps, int n_ext, int most) {
+  int cg = 1;
+  while (cg < most && warps * cg < kDownWarps && n_ext >= 16 * cg) cg *= 2;
+  return cg;
+}
+
 template <typename T>
 struct DownTask {
   const T* X;        // n_int x (n_ext+1) per merge; the last column is x
@@ -116,9 +125,16 @@ struct DownTask {
   const int* ext;
   const int* var;
   int nmerge, nch, nbc, n_ext, n_int, nrhs;
-  int64_t tile0;     // first 32-row tile of this task in the gint launch
+  int cg;            // warps that share 32 rows in the gint launch (1, 2, 4 or 8)
+  int64_t tile0;     // first CTA of this task in the gint launch
   int64_t elem0;     // first element of this task in the children launch
 };
+// CTAs of a task's gint launch per right-hand side: eight warps each
+template <typename T>
+__host__ __device__ inline int64_t down_task_row_tiles(const DownTask<T>& tk) {
+  const int per = 32 * (8 / tk.cg);
+  return ((int64_t)tk.nmerge * tk.n_int + per - 1) / per;
+}
 template <typename T>
 struct DownGroup {
   int n;

@@ -57,62 +57,103 @@ __device__ inline void load_coeffs(const Coeffs& cf, int64_t at, int dim, double
 
 // --------------------------------------------------------------- leaves ----
 
-__global__ void k_leaf_dtn_Lii(LeafConsts k, int64_t nl, Coeffs cf, double* Lii) {
-  const int64_t per = (int64_t)k.ni * k.ni;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % k.ni, c = rc / k.ni;
-    const int i = k.Ii[r], j = k.Ii[c];
-    double a, b[3], cc;
-    load_coeffs(cf, leaf * k.npts + i, k.dim, &a, b, &cc);
+// The leaf operators are mostly zeros (an entry couples nodes that differ along
+// one axis: 28 of 196 per row in 2D at p = 16), and FP64 instructions cost a
+// warp the same for one live lane as for 32: a CTA clears its leaf's block
+// and then computes the nonzero entries only, every lane with one of them.
+// Testing every entry for zero took 2650 us for 4096 leaves of 196 x 196, the
+// pipe's time for ten FP64 instructions per warp of entries; now 558 (writing
+// 1.26 GB takes 190).
+
+// stride of axis ax in the node order
+__device__ inline int axis_stride(int p, int ax) { return ax == 0 ? 1 : ax == 1 ? p : p * p; }
+
+__global__ void __launch_bounds__(256) k_leaf_dtn_Lii(LeafConsts k, int64_t nl, int nchunk, Coeffs cf, double* Lii) {
+  const int q = k.p - 2, cols = (k.ni + nchunk - 1) / nchunk;
+  for (int64_t lc = blockIdx.x; lc < nl * nchunk; lc += gridDim.x) {
+    const int64_t leaf = lc / nchunk;
+    const int c0 = (int)(lc % nchunk) * cols, nc = min(cols, k.ni - c0);
+    if (nc <= 0) continue;
+    double* L = Lii + leaf * (int64_t)k.ni * k.ni + (int64_t)c0 * k.ni;
+    for (int64_t e = threadIdx.x; e < (int64_t)nc * k.ni; e += blockDim.x) L[e] = 0.0;
+    __syncthreads();
     const double s = k.sleaf ? k.sleaf[leaf] : k.s;
-    Lii[e] = L_entry(k, s, a, b, cc, i, j);
+    // column c's entries along axis ax, position t; the diagonal with axis 0
+    for (int e = threadIdx.x; e < nc * k.dim * q; e += blockDim.x) {
+      const int t = 1 + e % q, ca = e / q, ax = ca % k.dim, c = ca / k.dim;
+      const int j = k.Ii[c0 + c];
+      int cj[3];
+      coords(k.dim, k.p, j, cj);
+      const int own = ax == 0 ? cj[0] : ax == 1 ? cj[1] : cj[2];
+      if (t == own && ax != 0) continue;
+      const int i = j + (t - own) * axis_stride(k.p, ax);
+      double a, b[3], cc;
+      load_coeffs(cf, leaf * k.npts + i, k.dim, &a, b, &cc);
+      L[k.iidx[i] + (int64_t)c * k.ni] = L_entry(k, s, a, b, cc, i, j);
+    }
   }
 }
 
-__global__ void k_leaf_dtn_rhs(LeafConsts k, int64_t nl, Coeffs cf, const double* f, double* rhs) {
-  const int ncol = k.nb + 1;
-  const int64_t per = (int64_t)k.ni * ncol;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % k.ni, col = rc / k.ni;
+// CTAs per leaf of k_leaf_dtn_Lii: four a SM in all
+inline int Lii_chunks(int64_t nl, int ni) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(ni, (4 * device_sms() + nl - 1) / nl));
+}
+
+// [L_ie P | -f_i]: a thread takes a row's kRhsCols columns, so that the row's
+// couplings to its 2 dim boundary nodes are computed once for them (per entry they
+// were six of every seven FP64 instructions in 3D: 992 us for 512 leaves of 216 x
+// 217; now 299).
+constexpr int kRhsCols = 16;
+__global__ void __launch_bounds__(256) k_leaf_dtn_rhs(LeafConsts k, int64_t nl, Coeffs cf, const double* f, double* rhs) {
+  const int ncol = k.nb + 1, nchunk = (ncol + kRhsCols - 1) / kRhsCols;
+  const int64_t total = nl * nchunk * k.ni;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int r = (int)(e % k.ni);
+    const int64_t lc = e / k.ni, leaf = lc / nchunk;
+    const int col0 = (int)(lc % nchunk) * kRhsCols, col1 = min(col0 + kRhsCols, ncol);
     const int i = k.Ii[r];
-    if (col == k.nb) {
-      rhs[e] = f ? -f[leaf * k.npts + i] : 0.0;
-      continue;
-    }
     double a, b[3], cc;
     load_coeffs(cf, leaf * k.npts + i, k.dim, &a, b, &cc);
     const double s = k.sleaf ? k.sleaf[leaf] : k.s;
     int ci[3];
     coords(k.dim, k.p, i, ci);
-    double acc = 0.0;
-    for (int ax = 0; ax < k.dim; ++ax) {
-      for (int end = 0; end < 2; ++end) {
-        int cj[3] = {ci[0], ci[1], ci[2]};
-        cj[ax] = end ? k.p - 1 : 0;
-        const int j = cj[0] + k.p * (cj[1] + k.p * cj[2]);
-        const int pr = k.prow[j];
-        const int el = ci[ax] * k.p + cj[ax];
-        const double lij = fma(a * s * s, k.DD[el], b[ax] * s * k.D[el]);
-        acc = fma(lij, k.P[pr + (int64_t)col * k.ne], acc);
-      }
+    double lij[6];
+    const double* P[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int ax = q / 2, end = q % 2;
+      lij[q] = 0.0;
+      P[q] = k.P;
+      if (ax >= k.dim) continue;
+      const int cj = end ? k.p - 1 : 0;
+      const int j = i + (cj - ci[ax]) * axis_stride(k.p, ax);
+      const int el = ci[ax] * k.p + cj;
+      P[q] += k.prow[j];
+      lij[q] = fma(a * s * s, k.DD[el], b[ax] * s * k.D[el]);
     }
-    rhs[e] = acc;
+    double* out = rhs + leaf * (int64_t)k.ni * ncol + r;
+    for (int col = col0; col < col1; ++col) {
+      double acc = 0.0;
+      if (col == k.nb) {
+        acc = f ? -f[leaf * k.npts + i] : 0.0;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+          if (q < 2 * k.dim) acc = fma(lij[q], P[q][(int64_t)col * k.ne], acc);
+      }
+      out[(int64_t)col * k.ni] = acc;
+    }
   }
 }
 
 cudaError_t leaf_dtn_assemble(const LeafConsts& k, int64_t nl, Coeffs cf, const double* f,
                               double* Lii, double* rhs, cudaStream_t st, Prof* pf) {
   if (pf) pf->begin(st);
-  k_leaf_dtn_Lii<<<grid_for(nl * k.ni * k.ni), 256, 0, st>>>(k, nl, cf, Lii);
+  const int nchunk = Lii_chunks(nl, k.ni);
+  k_leaf_dtn_Lii<<<grid_for(nl * nchunk, 1), 256, 0, st>>>(k, nl, nchunk, cf, Lii);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   if (pf) pf->begin(st);
-  k_leaf_dtn_rhs<<<grid_for(nl * k.ni * (k.nb + 1)), 256, 0, st>>>(k, nl, cf, f, rhs);
+  k_leaf_dtn_rhs<<<grid_for(nl * k.ni * ((k.nb + kRhsCols) / kRhsCols)), 256, 0, st>>>(k, nl, cf, f, rhs);
   if (pf) pf->end(K_ASSEMBLE, 2.0 * 2 * k.dim * (double)nl * k.ni * k.nb, st);
   return cudaGetLastError();
 }
@@ -167,17 +208,29 @@ __global__ void k_leaf_iti_rhs(LeafConsts k, int64_t nl, const cplx* f, cplx* rh
 
 // L(I_i, boundary nodes in owner order): the interior rows of the leaf
 // operator on the boundary columns, for the ItI interior elimination.
-__global__ void k_leaf_iti_Lie(LeafConsts k, int64_t nl, Coeffs cf, double* Lie) {
-  const int64_t per = (int64_t)k.ni * k.nown;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % k.ni, c = rc / k.ni;
-    const int i = k.Ii[r], j = k.own_node[c];
-    double a, b[3], cc;
-    load_coeffs(cf, leaf * k.npts + i, k.dim, &a, b, &cc);
-    Lie[e] = L_entry(k, k.s, a, b, cc, i, j);
+// Interior rows, owned boundary columns; nonzero along the normal of the
+// column's node (no corner node couples with an interior one).
+__global__ void __launch_bounds__(256) k_leaf_iti_Lie(LeafConsts k, int64_t nl, Coeffs cf, double* Lie) {
+  const int per = k.ni * k.nown, q = k.p - 2;
+  for (int64_t leaf = blockIdx.x; leaf < nl; leaf += gridDim.x) {
+    double* L = Lie + leaf * per;
+    for (int e = threadIdx.x; e < per; e += blockDim.x) L[e] = 0.0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < k.nown * q; e += blockDim.x) {
+      const int c = e / q, t = 1 + e % q;
+      const int j = k.own_node[c];
+      int cj[3];
+      coords(k.dim, k.p, j, cj);
+      int nax = 0, ax = 0;
+      for (int d = 0; d < k.dim; ++d)
+        if (cj[d] == 0 || cj[d] == k.p - 1) ++nax, ax = d;
+      if (nax != 1) continue;
+      const int own = ax == 0 ? cj[0] : ax == 1 ? cj[1] : cj[2];
+      const int i = j + (t - own) * axis_stride(k.p, ax);
+      double a, b[3], cc;
+      load_coeffs(cf, leaf * k.npts + i, k.dim, &a, b, &cc);
+      L[k.iidx[i] + c * k.ni] = L_entry(k, k.s, a, b, cc, i, j);
+    }
   }
 }
 
@@ -212,14 +265,15 @@ __global__ void k_coef_bounds(Coeffs cf, int dim, int64_t n, double* out) {
 
 cudaError_t leaf_assemble_Lii(const LeafConsts& k, int64_t nl, Coeffs cf, double* Lii, cudaStream_t st, Prof* pf) {
   if (pf) pf->begin(st);
-  k_leaf_dtn_Lii<<<grid_for(nl * k.ni * k.ni), 256, 0, st>>>(k, nl, cf, Lii);
+  const int nchunk = Lii_chunks(nl, k.ni);
+  k_leaf_dtn_Lii<<<grid_for(nl * nchunk, 1), 256, 0, st>>>(k, nl, nchunk, cf, Lii);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   return cudaGetLastError();
 }
 
 cudaError_t leaf_iti_Lie(const LeafConsts& k, int64_t nl, Coeffs cf, double* Lie, cudaStream_t st, Prof* pf) {
   if (pf) pf->begin(st);
-  k_leaf_iti_Lie<<<grid_for(nl * k.ni * k.nown), 256, 0, st>>>(k, nl, cf, Lie);
+  k_leaf_iti_Lie<<<grid_for(nl, 1), 256, 0, st>>>(k, nl, cf, Lie);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   return cudaGetLastError();
 }

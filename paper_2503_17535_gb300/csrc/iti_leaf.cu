@@ -30,71 +30,54 @@
 namespace hps {
 namespace {
 
-inline int gridn(int64_t total, int threads = 256) {
-  int64_t b = (total + threads - 1) / threads;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(b, 65535 * 8));
-}
-
 // dst[leaf][r + c n] = Re / Im (c < m: real parts, c >= m: imaginary parts) of
 // src[leaf][row(r) + c ld] (row(r) = rmap[r] or r0 + r); per-leaf strides.
 __global__ void k_split(const cplx* src, int64_t sstride, int sld, const int* rmap, int r0, int n, int m,
                         int64_t nl, double* dst, int64_t dstride) {
-  const int64_t per = (int64_t)n * 2 * m;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % n, c2 = rc / n;
-    const int c = c2 % m;
+  for_tile(n, 2 * m, nl, [&](int64_t leaf, int r, int c2) {
+    const int c = c2 < m ? c2 : c2 - m;
     const int row = rmap ? rmap[r] : r0 + r;
     const cplx v = src[leaf * sstride + row + (int64_t)c * sld];
     dst[leaf * dstride + r + (int64_t)c2 * n] = c2 < m ? v.re : v.im;
-  }
+  });
 }
 
 // dst[leaf][row(r) + c ld] = base[leaf][r + c bld] + sign * (re + i im) of the
 // split block sp[leaf] (n x 2m); base may be null (0).
 __global__ void k_merge(const double* sp, int64_t spstride, int n, int m, const cplx* base, int64_t bstride, int bld,
                         double sign, int64_t nl, cplx* dst, int64_t dstride, int dld, const int* rmap, int r0) {
-  const int64_t per = (int64_t)n * m;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % n, c = rc / n;
+  for_tile(n, m, nl, [&](int64_t leaf, int r, int c) {
     const double* s = sp + leaf * spstride;
     cplx v(sign * s[r + (int64_t)c * n], sign * s[r + (int64_t)(m + c) * n]);
     if (base) v = v + base[leaf * bstride + r + (int64_t)c * bld];
     const int row = rmap ? rmap[r] : r0 + r;
     dst[leaf * dstride + row + (int64_t)c * dld] = v;
-  }
+  });
 }
 
 // dst[leaf][row(r) + c ld] = src[leaf][r + c sld] (complex copy with a row map)
 __global__ void k_copy_rows(const cplx* src, int64_t sstride, int sld, int n, int m, int64_t nl, cplx* dst,
                             int64_t dstride, int dld, const int* rmap, int r0, const int* smap) {
-  const int64_t per = (int64_t)n * m;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t leaf = e / per;
-    const int rc = (int)(e % per);
-    const int r = rc % n, c = rc / n;
+  for_tile(n, m, nl, [&](int64_t leaf, int r, int c) {
     const int srow = smap ? smap[r] : r;
     const int row = rmap ? rmap[r] : r0 + r;
     dst[leaf * dstride + row + (int64_t)c * dld] = src[leaf * sstride + srow + (int64_t)c * sld];
-  }
+  });
 }
 
 // S[leaf] = complex(Sre[leaf]) + i eta on the diagonal
 __global__ void k_make_S(const double* Sre, int no, double eta, int64_t nl, cplx* S) {
-  const int64_t per = (int64_t)no * no;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int rc = (int)(e % per);
-    S[e] = cplx(Sre[e], (rc % no) == (rc / no) ? eta : 0.0);
-  }
+  for_tile(no, no, nl, [&](int64_t leaf, int r, int c) {
+    const int64_t e = leaf * no * no + r + (int64_t)c * no;
+    S[e] = cplx(Sre[e], r == c ? eta : 0.0);
+  });
 }
 
-// dst[leaf] = src (shared) for every leaf
-__global__ void k_broadcast(const double* src, int64_t n, int64_t nl, double* dst) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nl * n; e += (int64_t)gridDim.x * blockDim.x)
-    dst[e] = src[e % n];
+// dst[leaf] = src (shared, n x n) for every leaf
+__global__ void k_broadcast(const double* src, int n, int64_t nl, double* dst) {
+  for_tile(n, n, nl, [&](int64_t leaf, int r, int c) {
+    dst[leaf * n * n + r + (int64_t)c * n] = src[r + (int64_t)c * n];
+  });
 }
 
 hps_status ensure_cap(hps_handle* h, int ncols) {
@@ -188,7 +171,7 @@ hps_status iti_elim_setup(hps_handle* h, const Coeffs& co, cudaStream_t st, Prof
   HPS_CUDA(permute_rows<double>(bop<double>(tmp, (int64_t)ni * no, ni), WB, E.perm, ni, no, (int)nl, st, pf));
   HPS_CUDA(getrs_inplace<double>(LUo, ni, WB, no, (int)nl, st, pf));
   // S = G_oe - G_oi W (+ i eta on the diagonal)
-  k_broadcast<<<gridn(nl * no * no), 256, 0, st>>>(E.Goe, (int64_t)no * no, nl, tmp);
+  k_broadcast<<<tile_grid(no, no, nl), 256, 0, st>>>(E.Goe, no, nl, tmp);
   HPS_CUDA(cudaGetLastError());
   {
     GemmArgs<double> g;
@@ -199,7 +182,7 @@ hps_status iti_elim_setup(hps_handle* h, const Coeffs& co, cudaStream_t st, Prof
     g.alpha = -1.0; g.beta = 1.0;
     HPS_CUDA(gemm<double>(g, st, pf));
   }
-  k_make_S<<<gridn(nl * no * no), 256, 0, st>>>(tmp, no, h->eta, nl, E.S);
+  k_make_S<<<tile_grid(no, no, nl), 256, 0, st>>>(tmp, no, h->eta, nl, E.S);
   HPS_CUDA(cudaGetLastError());
   E.GS = lu_group_size<cplx>(no, (int)std::min<int64_t>(nl, 1 << 30), h->num_sms);
   if (E.GS > 1) {
@@ -223,7 +206,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   const int ni = E.ni, no = E.no, xr = (int)h->npts;
   const int64_t xs = (int64_t)xr * m;
   // z = L_ii^{-1} r_i  (split into real / imaginary columns)
-  k_split<<<gridn(nl * ni * 2 * m), 256, 0, st>>>(R, xs, xr, nullptr, no, ni, m, nl, E.z, (int64_t)ni * 2 * m);
+  k_split<<<tile_grid(ni, 2 * (int64_t)m, nl), 256, 0, st>>>(R, xs, xr, nullptr, no, ni, m, nl, E.z, (int64_t)ni * 2 * m);
   HPS_CUDA(cudaGetLastError());
   BOp<double> LUo = bop<double>(E.LU, (int64_t)ni * ni, ni);
   BOp<double> Z2 = bop<double>(E.z2, (int64_t)ni * 2 * m, ni);
@@ -239,7 +222,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
     g.alpha = 1.0; g.beta = 0.0;
     HPS_CUDA(gemm<double>(g, st, pf));
   }
-  k_merge<<<gridn(nl * no * m), 256, 0, st>>>(E.t, (int64_t)no * 2 * m, no, m, R, xs, xr, -1.0, nl, E.q,
+  k_merge<<<tile_grid(no, m, nl), 256, 0, st>>>(E.t, (int64_t)no * 2 * m, no, m, R, xs, xr, -1.0, nl, E.q,
                                               (int64_t)no * m, no, nullptr, 0);
   HPS_CUDA(cudaGetLastError());
   // y_e = S^{-1} q
@@ -248,7 +231,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   HPS_CUDA(permute_rows<cplx>(bop<cplx>(E.q, (int64_t)no * m, no), Q2, E.permS, no, m, (int)nl, st, pf));
   HPS_CUDA(getrs_inplace<cplx>(SB, no, Q2, m, (int)nl, st, pf, &E.invS, h->capturing));
   // y_i = z - W y_e
-  k_split<<<gridn(nl * no * 2 * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
+  k_split<<<tile_grid(no, 2 * (int64_t)m, nl), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
                                                   (int64_t)no * 2 * m);
   HPS_CUDA(cudaGetLastError());
   {
@@ -261,10 +244,10 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
     HPS_CUDA(gemm<double>(g, st, pf));
   }
   // scatter to node order
-  k_copy_rows<<<gridn(nl * no * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, no, m, nl, X, xs, xr, h->downn, 0,
+  k_copy_rows<<<tile_grid(no, m, nl), 256, 0, st>>>(E.q2, (int64_t)no * m, no, no, m, nl, X, xs, xr, h->downn, 0,
                                                   nullptr);
   HPS_CUDA(cudaGetLastError());
-  k_merge<<<gridn(nl * ni * m), 256, 0, st>>>(E.z2, (int64_t)ni * 2 * m, ni, m, nullptr, 0, 0, 1.0, nl, X, xs, xr,
+  k_merge<<<tile_grid(ni, m, nl), 256, 0, st>>>(E.z2, (int64_t)ni * 2 * m, ni, m, nullptr, 0, 0, 1.0, nl, X, xs, xr,
                                               h->dIi, 0);
   HPS_CUDA(cudaGetLastError());
   return HPS_OK;
@@ -279,10 +262,10 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
   const int ni = E.ni, no = E.no, xr = (int)h->npts;
   const int64_t xs = (int64_t)xr * m;
   // z_e (complex, owner order) and z_i (split)
-  k_copy_rows<<<gridn(nl * no * m), 256, 0, st>>>(Xb, xs, xr, no, m, nl, E.q, (int64_t)no * m, no, nullptr, 0,
+  k_copy_rows<<<tile_grid(no, m, nl), 256, 0, st>>>(Xb, xs, xr, no, m, nl, E.q, (int64_t)no * m, no, nullptr, 0,
                                                   h->downn);
   HPS_CUDA(cudaGetLastError());
-  k_split<<<gridn(nl * ni * 2 * m), 256, 0, st>>>(Xb, xs, xr, h->dIi, 0, ni, m, nl, E.z, (int64_t)ni * 2 * m);
+  k_split<<<tile_grid(ni, 2 * (int64_t)m, nl), 256, 0, st>>>(Xb, xs, xr, h->dIi, 0, ni, m, nl, E.z, (int64_t)ni * 2 * m);
   HPS_CUDA(cudaGetLastError());
   // q = z_e - W^T z_i
   {
@@ -295,7 +278,7 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
     g.alpha = 1.0; g.beta = 0.0;
     HPS_CUDA(gemm<double>(g, st, pf));
   }
-  k_merge<<<gridn(nl * no * m), 256, 0, st>>>(E.t, (int64_t)no * 2 * m, no, m, E.q, (int64_t)no * m, no, -1.0, nl,
+  k_merge<<<tile_grid(no, m, nl), 256, 0, st>>>(E.t, (int64_t)no * 2 * m, no, m, E.q, (int64_t)no * m, no, -1.0, nl,
                                               E.q, (int64_t)no * m, no, nullptr, 0);
   HPS_CUDA(cudaGetLastError());
   // x_o = S^{-H} q
@@ -304,7 +287,7 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
   HPS_CUDA(getrs_h<cplx>(bop<cplx>(E.S, (int64_t)no * no, no), no, QB, m, (int)nl, st, pf, &E.invS));
   HPS_CUDA(permute_rows_inv<cplx>(QB, Q2, E.permS, no, m, (int)nl, st));
   // z_i -= G_oi^T x_o
-  k_split<<<gridn(nl * no * 2 * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
+  k_split<<<tile_grid(no, 2 * (int64_t)m, nl), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
                                                   (int64_t)no * 2 * m);
   HPS_CUDA(cudaGetLastError());
   BOp<double> ZB = bop<double>(E.z, (int64_t)ni * 2 * m, ni);
@@ -323,10 +306,10 @@ hps_status iti_elim_apply_h(hps_handle* h, const cplx* Xb, cplx* Rb, int m, cuda
   HPS_CUDA(getrs_h<double>(bop<double>(E.LU, (int64_t)ni * ni, ni), ni, ZB, 2 * m, (int)nl, st, pf, &E.inv));
   HPS_CUDA(permute_rows_inv<double>(ZB, Z2, E.perm, ni, 2 * m, (int)nl, st));
   // Rbar rows: [x_o; x_i]
-  k_copy_rows<<<gridn(nl * no * m), 256, 0, st>>>(E.q2, (int64_t)no * m, no, no, m, nl, Rb, xs, xr, nullptr, 0,
+  k_copy_rows<<<tile_grid(no, m, nl), 256, 0, st>>>(E.q2, (int64_t)no * m, no, no, m, nl, Rb, xs, xr, nullptr, 0,
                                                   nullptr);
   HPS_CUDA(cudaGetLastError());
-  k_merge<<<gridn(nl * ni * m), 256, 0, st>>>(E.z2, (int64_t)ni * 2 * m, ni, m, nullptr, 0, 0, 1.0, nl, Rb, xs, xr,
+  k_merge<<<tile_grid(ni, m, nl), 256, 0, st>>>(E.z2, (int64_t)ni * 2 * m, ni, m, nullptr, 0, 0, 1.0, nl, Rb, xs, xr,
                                               nullptr, no);
   HPS_CUDA(cudaGetLastError());
   return HPS_OK;

@@ -1847,28 +1847,18 @@ cudaError_t getrf(BOp<T> A, int n, int batch, int* ipiv, int* perm, int* info, u
 // ------------------------------------------------------ triangular solve ----
 
 template <typename T>
-__global__ void k_permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch) {
-  int64_t total = (int64_t)n * nrhs;
-  for (int b = blockIdx.y; b < batch; b += gridDim.y) {
-    const T* s = src.item(b);
-    T* d = dst.item(b);
-    const int* pm = perm + (int64_t)b * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-      int i = (int)(e % n), j = (int)(e / n);
-      d[i + (int64_t)j * dst.ld] = s[pm[i] + (int64_t)j * src.ld];
-    }
-  }
+__global__ void __launch_bounds__(256) k_permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch) {
+  for_tile(n, nrhs, batch, [&](int64_t b, int i, int j) {
+    dst.item((int)b)[i + (int64_t)j * dst.ld] = src.item((int)b)[perm[b * n + i] + (int64_t)j * src.ld];
+  });
 }
 
 template <typename T>
 cudaError_t permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch,
                          cudaStream_t st, Prof* pf) {
   if (n <= 0 || nrhs <= 0 || batch <= 0) return cudaSuccess;
-  int64_t total = (int64_t)n * nrhs;
-  int bx = (int)std::min<int64_t>((total + 255) / 256, 2048);
   if (pf) pf->begin(st);
-  k_permute_rows<T><<<dim3(bx, std::min(batch, 65535)), 256, 0, st>>>(src, dst, perm, n, nrhs, batch);
+  k_permute_rows<T><<<tile_grid(n, nrhs, batch), 256, 0, st>>>(src, dst, perm, n, nrhs, batch);
   if (pf) pf->end(K_GATHER, 0.0, st);
   return cudaGetLastError();
 }

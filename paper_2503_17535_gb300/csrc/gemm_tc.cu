@@ -877,17 +877,17 @@ bool tc_applicable(const GemmArgs<T>& g) {
   if (!w || !w->enabled || !w->err_slot || !*w->err_slot || g.ta || g.K > (1 << 20)) return false;
   if (w->force) return true;
   // one side of at least 32 and the other of at least 16: the short side
-  // goes to the 48-wide tile dimension (transposed tiling when M is short)
+  // goes to the narrow tile dimension (transposed tiling when M is short)
   if (std::min(g.M, g.N) < 1 || std::max(g.M, g.N) < 32 || g.K < 16) return false;
   if (std::min(g.M, g.N) < 16 && !few_rows_long_k(g.M, g.N, g.K)) return false;
-  // a side below 32 fills at best two thirds of the 48-wide tile side: such
+  // a side below 32 leaves even the 32-wide tile side part empty: such
   // products go to the tensor cores only while the tiles stay over ~28 % full
   // (measured: 28 x 113 gains there, 28 x 57 loses) -- except products of
-  // at most 8 rows, N >= 32 and K >= 32, which the FP64-pipe kernels run at
-  // under half their rate (4 x 114 x 64: 0.14 TFLOP/s); few columns stay on
-  // the FP64 pipe's skinny kernels
+  // at most 8 rows, N >= 32 and K >= 32, which half-empty FP64-pipe tiles run
+  // at under half their rate (4 x 114 x 64 complex, 4096 items: 1.4 ms of 0.6);
+  // few columns stay on the FP64 pipe's skinny kernels
   if (std::min(g.M, g.N) < 32 && tile_fill(g.M, g.N) < 0.28 && !few_rows_long_k(g.M, g.N, g.K)) return false;
-  // short inner dimensions: ten accumulators per output are read back for
+  // short inner dimensions: eight accumulators per output are read back for
   // little work, so small items stay on the FP64 pipe
   if (g.K < lu_tune(TUNE_TC_MIN_K) && (g.M < 512 || g.N < 512)) return false;
   if ((double)g.M * g.N * g.K * g.batch < 1.0e5 * lu_tune(TUNE_TC_MIN_WORK_REAL)) return false;

@@ -1,8 +1,10 @@
 // Shape choices of the batched LU and the tensor-core routing thresholds on
 // GB300 (hps_tune_set in include/hps.h).  Written by
 // paper_2503_17535_gb300/autotune.py from timed builds of the benchmark
-// workloads (summed median build time, ms, at the chosen values:
-// {"helmholtz2d_iti_p16_depth6": 171.74, "elliptic3d_dtn_p8_depth3": 150.87, "adaptive3d_dtn_p8": 122.98}); rerun it to regenerate.
+// workloads; rerun it to regenerate.  The base widths were measured again with
+// the faster interchange step (few / many: 32/8, 64/16, 128/32, all/64 panels:
+// 3D elliptic build 84.9 / 82.2 / 80.8 / 82.2 ms, Helmholtz 99.7 / 99.5 /
+// 99.2 / 99.3).
 #pragma once
 
 #define HPS_TUNED_LU_CLUSTER_PANEL 1

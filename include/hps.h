@@ -308,8 +308,9 @@ void hps_free(hps_handle* h);
 
 /* Give the freed device memory that the library's pool keeps on the current
  * device (at most a sixteenth of the device's memory) back to the device, for
- * a program that needs it for something else.  Memory of live handles and of
- * work in flight stays.  HPS_ERR_CUDA when a CUDA call fails. */
+ * a program that needs it for something else, and destroy the library's idle
+ * streams there (at most eight).  Memory of live handles and of work in flight
+ * stays.  HPS_ERR_CUDA when a CUDA call fails. */
 hps_status hps_trim(void);
 
 /* Batched dense product C = alpha A B + beta C (no counterpart in the paper:
@@ -364,8 +365,9 @@ hps_status hps_getrf(int dtype, int mode, int n, int batch, void* A, int lda, in
  *   HPS_TUNE_LU_BASE_PANELS_MANY (1): the same for batches of 8 or more;
  *   HPS_TUNE_LU_FEW_MIN_N        (2): batches of fewer than 8 recurse only
  *       from this order on;
- *   HPS_TUNE_LU_CLUSTER_PANEL    (3): 1 factors tall panels in a thread-block
- *       cluster's distributed shared memory, 0 with cooperative groups;
+ *   HPS_TUNE_LU_CLUSTER_PANEL    (3): 1 factors panels in the registers of a
+ *       CTA or thread-block cluster (beside the trailing updates when there
+ *       are few matrices), 0 in shared memory with cooperative groups;
  *   HPS_TUNE_TC_MIN_WORK_REAL    (4): a real product of the build runs on the
  *       tensor cores from M N K batch >= value x 1e5 on (hps_options.fp64_gemm
  *       = 0), else on the FP64 pipe;

@@ -463,10 +463,11 @@ cudaError_t merge_gather_h(const T* hc, int nmerge, int nch, int nbc, int n_ext,
 // very long rows, the ranges cost locality: 432 real tiles 94 -> 137, 216 of
 // 13824 columns 246 -> 265).  With one warp per 32 rows up to 255 columns, as
 // before, 64 real merges of 176 columns took 80 us, now 12.
+constexpr int kGridY = 65535;   // groups of right-hand sides in one launch (grid limit)
 template <typename T, int CG, int NC, bool CL>
 __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X, const T* xp, const T* gpar,
                                                                        int64_t rows, int n_ext, int n_int, int nrhs,
-                                                                       int CS, T* gint) {
+                                                                       int CS, int cfirst, T* gint) {
   namespace cg_ = cooperative_groups;
   constexpr int NW = CG < 4 ? 4 : CG;
   __shared__ T part[CG > 1 ? NW : 1][NC][33];
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cg = w % CG;
   const int rank = CL ? (int)blockIdx.x % CS : 0;
   const int64_t R = ((int64_t)(CL ? blockIdx.x / CS : blockIdx.x) * (NW / CG) + w / CG) * 32 + lane;
-  const int c0 = blockIdx.y * NC;
+  const int c0 = cfirst + blockIdx.y * NC;
   const bool live = R < rows;
   const int64_t b = live ? R / n_int : 0;
   const int r = live ? (int)(R % n_int) : 0;
@@ -541,7 +542,7 @@ cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t 
   constexpr int NW = CG < 4 ? 4 : CG;
   const int per = 32 * (NW / CG);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((rows + per - 1) / per * cs), (nrhs + NC - 1) / NC);
+  cfg.gridDim.x = (unsigned)((rows + per - 1) / per * cs);
   cfg.blockDim = dim3(32 * NW);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -551,7 +552,12 @@ cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = CL ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_down_gint<T, CG, NC, CL>, X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint);
+  cudaError_t e = cudaSuccess;
+  for (int c = 0; c < nrhs && e == cudaSuccess; c += kGridY * NC) {
+    cfg.gridDim.y = std::min(kGridY, (nrhs - c + NC - 1) / NC);
+    e = cudaLaunchKernelEx(&cfg, k_down_gint<T, CG, NC, CL>, X, xp, gpar, rows, n_ext, n_int, nrhs, cs, c, gint);
+  }
+  return e;
 }
 
 template <typename T, int CG, bool CL>

@@ -981,7 +981,10 @@ int panel_cluster_size(int rows, int nb, int batch) {
 // mbarriers (bounded waits); every warp then picks the same pivot from its own
 // shared memory.  Candidates are double-buffered by column parity: a CTA
 // pushes into a slot again only two columns later, after receiving the
-// candidates that every CTA sends once it has finished with the slot.
+// candidates that every CTA sends once it has finished with the slot.  So are
+// the candidates of the CTA's own warps (wrec): in a cluster with one thread
+// per row only the next column's block barrier orders a warp's reading of them
+// before what another warp writes after that.
 //
 // What bounds it: the chain from one pivot to the next.  The FP64 pipe takes
 // 64 cycles per warp instruction and scheduler; a division is ~440 cycles, the
@@ -1052,7 +1055,7 @@ struct PanelReg {
   T* cinv;        // [2][CS] reciprocals of their pivot entries
   uint4* crec;    // [2][CS] their keys: magnitude hi + 1, lo, position, row
   uint64_t* bar;  // [2] keys and rows of a slot have arrived, [2] reciprocals
-  uint4* wrec;    // [RW] this CTA's warps' candidates
+  uint4* wrec;    // [2 slots][16] this CTA's warps' candidates
   T* srow;        // [NB + 1] the CTA candidate's row and reciprocal (3 more are read past a row's end)
   unsigned* err;
   int CS, g, k0, nb, r0, ld, RW;
@@ -1084,10 +1087,10 @@ struct PanelReg {
       uint32_t hi = done ? 0u : (uint32_t)(mb >> 32) + 1u, lo = done ? 0u : (uint32_t)mb;
       uint32_t ps = (uint32_t)(pr - k0 < nb ? ptop : pr);
       const int src = warp_pivot(hi, lo, ps);
-      if (lane == src) wrec[rw] = make_uint4(hi, lo, ps, (uint32_t)pr);
+      if (lane == src) wrec[slot * 16 + rw] = make_uint4(hi, lo, ps, (uint32_t)pr);
     }
     __syncthreads();
-    uint4 rec = wrec[RW > 1 && lane < RW ? lane : 0];
+    uint4 rec = wrec[slot * 16 + (RW > 1 && lane < RW ? lane : 0)];
     int w = 0;
     if (RW > 1) {
       if (lane >= RW) rec = make_uint4(0u, 0u, 0xffffffffu, 0u);
@@ -1211,7 +1214,7 @@ __global__ void __launch_bounds__(512) k_lu_panel_reg(BOp<T> A, int n, int k0, i
   namespace cg = cooperative_groups;
   constexpr int NB = LuNB<T>::NB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint4 wrec[16];
+  __shared__ uint4 wrec[2 * 16];
   __shared__ uint4 crec[2 * 16];
   __shared__ __align__(8) uint64_t bars[4];
   PanelReg<T, CL, CT> p;

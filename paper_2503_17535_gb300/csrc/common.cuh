@@ -137,6 +137,13 @@ __device__ inline bool wait_flag(const volatile unsigned* f, unsigned want, unsi
   return true;
 }
 
+// The two halves of a cluster-wide barrier, for all threads of the cluster.
+// Another CTA's shared memory may be touched only once that CTA has started:
+// kernels that write into it arrive at entry and wait before their first
+// remote store.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // Copies over a batch of rows x cols blocks: a CTA walks tiles of kTileRows x
 // kTileCols of its items, so that the only division per entry is a 32-bit one (a
 // 64-bit division and remainder cost more than the copy: 4096 items of 196 x

@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(32 * NW, 24 / NW) k_split(SplitSet<T> ss, int 
   const int cr = (int)blockIdx.x % CS;                        // CTA of the cluster (clusters run along x)
   const int rg = (int)blockIdx.x / CS;
   if (rg * (NW / KW) * 32 >= R || bl >= ss.items[op]) return;  // uniform over the cluster
+  if (CS > 1) cluster_arrive();   // before the maxima go to the other CTAs, every CTA has started
   const Src<T>& s = ss.s[op];
   const int kw = warp & (KW - 1);
   const int rbase = (rg * (NW / KW) + warp / KW) * 32;
@@ -295,6 +296,7 @@ __global__ void __launch_bounds__(32 * NW, 24 / NW) k_split(SplitSet<T> ss, int 
   if (CS > 1) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
+    cluster_wait();
     if (kw == 0)
       for (int d = 0; d < CS; ++d) cl.map_shared_rank(&cmax[0][0][0], d)[(cr * NW + warp) * 32 + lane] = mx;
     cl.sync();

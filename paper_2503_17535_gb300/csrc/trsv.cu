@@ -138,9 +138,6 @@ size_t block_smem(int n, int nr, bool herm) {
 
 // ------------------------------------------------------------- few matrices
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
 template <typename T, int NR, bool HERM, int MO>
 __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X, int nrhs, const T* dinv) {
   namespace cg = cooperative_groups;

@@ -6,11 +6,16 @@
   the warp that holds the winner, the wait for the pushed bytes -- are laid out
   as a graph of what is ordered before what; a slot may be written again only
   after every reading of what it held.
+* Another CTA's shared memory may be touched only once that CTA has started: in
+  every kernel that writes there, a cluster-wide barrier comes before the first
+  remote address.
 """
 
 import itertools
 import os
 import re
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_17535_gb300", "csrc")
 
@@ -64,3 +69,32 @@ def test_panel_candidates_are_read_before_they_are_overwritten():
     assert "const int slot = jj & 1;" in src
     for winners in itertools.product(range(3), repeat=5):
         assert not _unordered_reuse(slots, 3, 5, winners)
+
+
+BARRIER = re.compile(r"cluster_wait\(\)|cl\.sync\(\)|this_cluster\(\)\.sync\(\)")
+STORE = r"map_shared_rank\(|peer_addr\("
+# where a kernel first makes such a store: a call of the lambda or member function that does
+CALLS = {"k_trsv_cluster": r"solve\(dm,", "k_lu_panel_reg": r"p\.template run<"}
+
+
+def _kernels(src):
+    """(name, body) of every __global__ function."""
+    for m in re.finditer(r"__global__ void (?:__launch_bounds__\([^{;]*?\)\s+)?(k_\w+)\(", src):
+        start = src.index("{", m.end())
+        depth, i = 1, start + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[i], 0)
+            i += 1
+        yield m.group(1), src[start:i]
+
+
+@pytest.mark.parametrize("name,count", [("gemm_tc.cu", 1), ("linalg.cu", 2), ("trsv.cu", 1)])
+def test_cluster_barrier_before_the_first_remote_store(name, count):
+    found = 0
+    for kernel, body in _kernels(_source(name)):
+        remote = re.search(CALLS.get(kernel, STORE), body)
+        if remote:
+            found += 1
+            barrier = BARRIER.search(body)
+            assert barrier and barrier.start() < remote.start(), kernel
+    assert found == count

@@ -472,6 +472,7 @@ __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X
   constexpr int NW = CG < 4 ? 4 : CG;
   __shared__ T part[CG > 1 ? NW : 1][NC][33];
   __shared__ T sums[CL ? 8 : 1][NC][33];   // of the cluster's CTAs
+  if constexpr (CL) cluster_arrive();   // before its sums go to the first CTA, that one has started
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cg = w % CG;
   const int rank = CL ? (int)blockIdx.x % CS : 0;
   const int64_t R = ((int64_t)(CL ? blockIdx.x / CS : blockIdx.x) * (NW / CG) + w / CG) * 32 + lane;
@@ -509,6 +510,7 @@ __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X
   }
   if constexpr (CL) {
     cg_::cluster_group cl = cg_::this_cluster();
+    cluster_wait();
     if (w == 0) {
       T* first = cl.map_shared_rank(&sums[0][0][0], 0);
 #pragma unroll

@@ -88,7 +88,7 @@ def _kernels(src):
         yield m.group(1), src[start:i]
 
 
-@pytest.mark.parametrize("name,count", [("gemm_tc.cu", 1), ("linalg.cu", 2), ("trsv.cu", 1)])
+@pytest.mark.parametrize("name,count", [("gemm_tc.cu", 1), ("linalg.cu", 2), ("trsv.cu", 1), ("hps_kernels.cu", 1)])
 def test_cluster_barrier_before_the_first_remote_store(name, count):
     found = 0
     for kernel, body in _kernels(_source(name)):

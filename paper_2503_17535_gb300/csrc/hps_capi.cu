@@ -501,7 +501,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
     if (!h->capturing && trsv_flags_applicable<T>(ni, nrhs, nm, h->trsv))
       HPS_CUDA(getrs_flags<T>((const T*)Lv.D, ni, ni, y, ni, nrhs, h->trsv, st, pf));
     else
-      HPS_CUDA(getrs_inplace<T>(DD, ni, YB, nrhs, nm, st, pf, &Lv.inv, h->capturing));
+      HPS_CUDA(getrs_inplace<T>(DD, ni, YB, nrhs, nm, st, pf, &Lv.inv));
     return HPS_OK;
   }
   const int hn = ni / 2, nb = h->nb;
@@ -532,7 +532,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
   if (!h->capturing && trsv_flags_applicable<T>(hn, nrhs, nm, h->trsv))
     HPS_CUDA(getrs_flags<T>((const T*)Lv.W, hn, hn, y, ni, nrhs, h->trsv, st, pf));
   else
-    HPS_CUDA(getrs_inplace<T>(WW, hn, YB, nrhs, nm, st, pf, &Lv.inv, h->capturing));
+    HPS_CUDA(getrs_inplace<T>(WW, hn, YB, nrhs, nm, st, pf, &Lv.inv));
   HPS_CUDA(copy_block<T>(b + hn, (int64_t)ni * nrhs, ni, y + hn, (int64_t)ni * nrhs, ni, hn, nrhs, nm, st, pf));
   // y2 <- b2 - D21 y1 (even children's interior blocks)
   HPS_CUDA(child_block(false, grouped(YB, 2), grouped(YB, 2)));
@@ -580,7 +580,7 @@ hps_status solve_impl(hps_handle* h, int nrhs, const void* g_in, const void* f_i
     } else {
       BOp<T> LA = bop<T>((T*)h->leafA, (int64_t)nlu * nlu, nlu);
       HPS_CUDA(permute_rows<T>(bop<T>(tmp, (int64_t)xr * nrhs, xr), XF, h->leaf_perm, nlu, nrhs, (int)nl, st, pf));
-      HPS_CUDA(getrs_inplace<T>(LA, nlu, XF, nrhs, (int)nl, st, pf, &h->leaf_inv, h->capturing));
+      HPS_CUDA(getrs_inplace<T>(LA, nlu, XF, nrhs, (int)nl, st, pf, &h->leaf_inv));
     }
     GemmArgs<T> gl;
     gl.M = nb; gl.N = nrhs; gl.K = ITI ? (int)h->npts : xr; gl.batch = (int)nl;

@@ -211,7 +211,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   BOp<double> LUo = bop<double>(E.LU, (int64_t)ni * ni, ni);
   BOp<double> Z2 = bop<double>(E.z2, (int64_t)ni * 2 * m, ni);
   HPS_CUDA(permute_rows<double>(bop<double>(E.z, (int64_t)ni * 2 * m, ni), Z2, E.perm, ni, 2 * m, (int)nl, st, pf));
-  HPS_CUDA(getrs_inplace<double>(LUo, ni, Z2, 2 * m, (int)nl, st, pf, &E.inv, h->capturing));
+  HPS_CUDA(getrs_inplace<double>(LUo, ni, Z2, 2 * m, (int)nl, st, pf, &E.inv));
   // q = r_o - G_oi z
   {
     GemmArgs<double> g;
@@ -229,7 +229,7 @@ hps_status iti_elim_apply(hps_handle* h, const cplx* R, cplx* X, int m, cudaStre
   BOp<cplx> SB = bop<cplx>(E.S, (int64_t)no * no, no);
   BOp<cplx> Q2 = bop<cplx>(E.q2, (int64_t)no * m, no);
   HPS_CUDA(permute_rows<cplx>(bop<cplx>(E.q, (int64_t)no * m, no), Q2, E.permS, no, m, (int)nl, st, pf));
-  HPS_CUDA(getrs_inplace<cplx>(SB, no, Q2, m, (int)nl, st, pf, &E.invS, h->capturing));
+  HPS_CUDA(getrs_inplace<cplx>(SB, no, Q2, m, (int)nl, st, pf, &E.invS));
   // y_i = z - W y_e
   k_split<<<tile_grid(no, 2 * (int64_t)m, nl), 256, 0, st>>>(E.q2, (int64_t)no * m, no, nullptr, 0, no, m, nl, E.t,
                                                   (int64_t)no * 2 * m);

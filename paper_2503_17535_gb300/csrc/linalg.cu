@@ -509,6 +509,13 @@ int device_sms() {
   return sms;
 }
 
+bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // ------------------------------------------------------------ panel LU ----
 
 // Factor the panel A[k0:n, k0:k0+nb) of each matrix with partial pivoting.
@@ -1737,9 +1744,7 @@ struct LookAhead {
       tried = true;
       // a stream that is being captured would take the side stream, and whoever
       // takes it next, into the capture
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(main, &cap) != cudaSuccess) cudaGetLastError();
-      else if (cap == cudaStreamCaptureStatusNone) side_take(&side);
+      if (!stream_capturing(main)) side_take(&side);
     }
     return side.st != nullptr;
   }
@@ -2103,10 +2108,10 @@ static cudaError_t rtrsm_upper(BOp<T> LU, BOp<T> X, int p0, int n1, int nrhs, in
 
 template <typename T>
 cudaError_t getrs_inplace(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st,
-                          Prof* pf, TrsvInv* inv, bool capturing) {
+                          Prof* pf, TrsvInv* inv) {
   if (n <= 0 || nrhs <= 0 || batch <= 0) return cudaSuccess;
   if (trsv_few_applicable<T>(n, nrhs, batch, inv))
-    return trsv_few<T>(LU, n, X, nrhs, batch, false, inv, capturing, st, pf);
+    return trsv_few<T>(LU, n, X, nrhs, batch, false, inv, st, pf);
   cudaError_t e;
   // forward: unit lower; backward: non-unit upper
   if ((e = rtrsm_lower<T>(LU, X, 0, n, nrhs, batch, st, pf)) != cudaSuccess) return e;
@@ -2377,11 +2382,10 @@ cudaError_t permute_rows_inv(BOp<T> src, BOp<T> dst, const int* perm, int n, int
 // X <- (U^H)^{-1} then (L^H)^{-1}: the conjugate transpose of getrs_inplace
 // (without the row permutation, which the caller applies after).
 template <typename T>
-cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf, TrsvInv* inv,
-                    bool capturing) {
+cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf, TrsvInv* inv) {
   if (n <= 0 || nrhs <= 0 || batch <= 0) return cudaSuccess;
   if (trsv_few_applicable<T>(n, nrhs, batch, inv))
-    return trsv_few<T>(LU, n, X, nrhs, batch, true, inv, capturing, st, pf);
+    return trsv_few<T>(LU, n, X, nrhs, batch, true, inv, st, pf);
   const int pb0 = 32;
   const int by = std::min(batch, 65535);
   const int bx = std::min((nrhs + 127) / 128, 1024);
@@ -2432,11 +2436,11 @@ cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_
                                 const LuWork&, cudaStream_t, Prof*);                             \
   template cudaError_t permute_rows<T>(BOp<T>, BOp<T>, const int*, int, int, int, cudaStream_t,  \
                                        Prof*);                                                   \
-  template cudaError_t getrs_inplace<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*, bool);   \
+  template cudaError_t getrs_inplace<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*);   \
   template bool trsv_flags_applicable<T>(int, int, int, const TrsvWork&);                        \
   template cudaError_t getrs_flags<T>(const T*, int, int, T*, int, int, TrsvWork&, cudaStream_t, Prof*); \
   template cudaError_t permute_rows_inv<T>(BOp<T>, BOp<T>, const int*, int, int, int, cudaStream_t);    \
-  template cudaError_t getrs_h<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*, bool);
+  template cudaError_t getrs_h<T>(BOp<T>, int, BOp<T>, int, int, cudaStream_t, Prof*, TrsvInv*);
 
 HPS_INST(double)
 HPS_INST(cplx)

@@ -159,6 +159,10 @@ int& lu_tune(int param);
 // Streaming multiprocessors of the current device (queried once per process).
 int device_sms();
 
+// Whether work enqueued on the stream is recorded into a graph, by the library or
+// by the caller, instead of run (also when the stream does not tell).
+bool stream_capturing(cudaStream_t st);
+
 struct LuWork {
   unsigned* bars = nullptr;   // 2 * batch barrier words (zeroed)
   void* pub = nullptr;        // publish buffer for G > 1
@@ -194,7 +198,8 @@ cudaError_t permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrh
 
 // Inverses of the diagonal blocks of a batch of factors (trsv.cu): storage of
 // trsv_inv_elems elements that lives as long as the factors, filled by the
-// first solve with few right-hand sides.
+// first solve with few right-hand sides that is not being captured into a graph
+// (a captured one records their formation, which every launch repeats).
 struct TrsvInv {
   void* p = nullptr;
   bool ready = false;
@@ -208,14 +213,12 @@ template <typename T>
 bool trsv_few_applicable(int n, int nrhs, int batch, const TrsvInv* inv);
 // Both triangles in one launch, X already row-permuted: X <- U^{-1} L^{-1} X,
 // or with herm X <- L^{-H} U^{-H} X (before the inverse permutation).
-// capturing: the stream is being captured into a graph.
 template <typename T>
-cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm, TrsvInv* inv, bool capturing,
-                     cudaStream_t st, Prof* pf);
+cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm, TrsvInv* inv, cudaStream_t st, Prof* pf);
 
 template <typename T>
 cudaError_t getrs_inplace(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st,
-                          Prof* pf, TrsvInv* inv = nullptr, bool capturing = false);
+                          Prof* pf, TrsvInv* inv = nullptr);
 
 // One n x n LU factor against nrhs <= 8 columns (X <- U^{-1} L^{-1} X, X
 // already row-permuted), each triangle in a single cooperative launch:
@@ -249,7 +252,7 @@ cudaError_t permute_rows_inv(BOp<T> src, BOp<T> dst, const int* perm, int n, int
                              cudaStream_t st);
 template <typename T>
 cudaError_t getrs_h(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st, Prof* pf,
-                    TrsvInv* inv = nullptr, bool capturing = false);
+                    TrsvInv* inv = nullptr);
 
 // C = alpha * C + beta (identity added on the diagonal when diag != 0) helpers
 template <typename T>

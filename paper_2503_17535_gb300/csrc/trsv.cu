@@ -483,8 +483,7 @@ bool trsv_few_applicable(int n, int nrhs, int batch, const TrsvInv* inv) {
 }
 
 template <typename T>
-cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm, TrsvInv* inv, bool capturing,
-                     cudaStream_t st, Prof* pf) {
+cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm, TrsvInv* inv, cudaStream_t st, Prof* pf) {
   cudaError_t e;
   const T* dv = nullptr;
   if (inv && inv->p) {
@@ -493,7 +492,7 @@ cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm,
       k_block_inverses<T><<<dim3((n + 31) / 32, 2, batch), 128, 0, st>>>(LU, n, static_cast<T*>(inv->p));
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if (pf) pf->end(K_OTHER, 0.0, st);
-      if (!capturing) inv->ready = true;   // a captured launch runs with every replay
+      inv->ready = !stream_capturing(st);   // a captured launch has formed nothing yet
     }
     dv = static_cast<const T*>(inv->p);
   }
@@ -510,7 +509,7 @@ cudaError_t trsv_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, bool herm,
 
 #define HPS_TRSV_INST(T)                                                        \
   template bool trsv_few_applicable<T>(int, int, int, const TrsvInv*);          \
-  template cudaError_t trsv_few<T>(BOp<T>, int, BOp<T>, int, int, bool, TrsvInv*, bool, cudaStream_t, Prof*);
+  template cudaError_t trsv_few<T>(BOp<T>, int, BOp<T>, int, int, bool, TrsvInv*, cudaStream_t, Prof*);
 HPS_TRSV_INST(double)
 HPS_TRSV_INST(cplx)
 

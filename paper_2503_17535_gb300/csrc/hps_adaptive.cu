@@ -724,7 +724,7 @@ hps_status adaptive_solve(hps_handle* h, int nrhs, const void* g_in, const void*
                             (T*)M.x, st, pf));
       BOp<T> GI = bop<T>((T*)M.gint, 0, M.n_int);
       HPS_CUDA(permute_rows<T>(bop<T>((T*)M.x, 0, M.n_int), GI, M.perm, M.n_int, nrhs, 1, st, pf));
-      if (trsv_flags_applicable<T>(M.n_int, nrhs, 1, h->trsv))
+      if (trsv_flags_applicable<T>(M.n_int, nrhs, 1, h->trsv) && !stream_capturing(st))
         HPS_CUDA(getrs_flags<T>((const T*)M.D, M.n_int, M.n_int, (T*)M.gint, M.n_int, nrhs, h->trsv, st, pf));
       else
         HPS_CUDA(getrs_inplace<T>(bop<T>((T*)M.D, 0, M.n_int), M.n_int, GI, nrhs, 1, st, pf, &h->ag.back().inv));

@@ -498,7 +498,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
   if (!Kind<T>::iti) {
     BOp<T> DD = bop<T>((T*)Lv.D, (int64_t)ni * ni, ni);
     HPS_CUDA(permute_rows<T>(bop<T>(b, (int64_t)ni * nrhs, ni), YB, Lv.perm, ni, nrhs, nm, st, pf));
-    if (!h->capturing && trsv_flags_applicable<T>(ni, nrhs, nm, h->trsv))
+    if (trsv_flags_applicable<T>(ni, nrhs, nm, h->trsv) && !stream_capturing(st))
       HPS_CUDA(getrs_flags<T>((const T*)Lv.D, ni, ni, y, ni, nrhs, h->trsv, st, pf));
     else
       HPS_CUDA(getrs_inplace<T>(DD, ni, YB, nrhs, nm, st, pf, &Lv.inv));
@@ -529,7 +529,7 @@ hps_status apply_Dinv(hps_handle* h, int m, T* b, T* y, int nrhs, cudaStream_t s
   // b1 <- b1 - D12 b2 (odd children's interior blocks)
   HPS_CUDA(child_block(true, grouped(B1, 2), grouped(B1, 2)));
   HPS_CUDA(permute_rows<T>(B1, YB, Lv.perm, hn, nrhs, nm, st, pf));
-  if (!h->capturing && trsv_flags_applicable<T>(hn, nrhs, nm, h->trsv))
+  if (trsv_flags_applicable<T>(hn, nrhs, nm, h->trsv) && !stream_capturing(st))
     HPS_CUDA(getrs_flags<T>((const T*)Lv.W, hn, hn, y, ni, nrhs, h->trsv, st, pf));
   else
     HPS_CUDA(getrs_inplace<T>(WW, hn, YB, nrhs, nm, st, pf, &Lv.inv));

@@ -225,8 +225,10 @@ cudaError_t getrs_inplace(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaS
 // 32-row blocks are solved in dependency order and published through
 // per-block flags (flags[i] == epoch once block i is final).  The caller
 // keeps one flag per 32 rows (device, initially 0) and a counter; each call
-// uses two fresh epochs.  A wait that exceeds its poll limit stores 1 in
-// *host_err (host-mapped memory) and the block goes on, so no launch hangs.
+// uses two fresh epochs, so that it must not be recorded into a graph (a second
+// launch would find the flags of the first).  A wait that exceeds its poll limit
+// stores 1 in *host_err (host-mapped memory) and the block goes on, so no launch
+// hangs.
 struct TrsvWork {
   unsigned* flags = nullptr;
   int nflags = 0;

@@ -7,7 +7,9 @@ itself, and every launch of the graph must give the solution of the data that
 are then behind its pointers.
 
 Reference: the same solve of a second operator that was never captured.  The
-same kernels run on the same data, so the results are equal."""
+same kernels run on the same data, so the results are equal, except where a
+captured solve takes the blocked triangular solves (single factors beyond 2048
+rows), which are as accurate: 1e-11, both are backward-stable solves."""
 
 import numpy as np
 import pytest
@@ -53,7 +55,7 @@ def _operator(P, kind, p, L, lazy, seed):
 
 
 CASES = [("dtn2", 9, 3, False), ("iti", 10, 3, False), ("iti", 10, 2, True), ("dtn3", 6, 2, False), ("dtn3", 6, 1, True),
-         ("adaptive", 6, 0, False)]
+         ("adaptive", 6, 0, False), ("dtn3", 9, 2, True)]
 
 
 @pytest.mark.parametrize("kind,p,L,lazy", CASES, ids=["%s-p%d-L%d-%s" % (c[0], c[1], c[2], "lazy" if c[3] else "explicit")
@@ -61,6 +63,8 @@ CASES = [("dtn2", 9, 3, False), ("iti", 10, 3, False), ("iti", 10, 2, True), ("d
 def test_solves_around_a_callers_graph(P, kind, p, L, lazy):
     build, rhs, out = _operator(P, kind, p, L, lazy, 100 * p + L)
     (g, f), (g2, f2) = rhs(), rhs()
+    blocked = (kind, p) == ("dtn3", 9)   # a root of 2352 rows
+    same = lambda u, v: bool(((u - v).abs().max() <= (1e-11 if blocked else 0.0) * v.abs().max()))  # noqa: E731
     h = build()
     u, v = out(), out()
     P.hps_solve(h, g, u)   # the workspace
@@ -74,7 +78,7 @@ def test_solves_around_a_callers_graph(P, kind, p, L, lazy):
     w, w2 = out(), out()
     P.hps_solve(ref, g, w, f=f)
     P.hps_solve(ref, g2, w2, f=f2)
-    assert torch.equal(v, w)
+    assert same(v, w)
     # a graph captured before any new-source solve, launched for three sources
     h = build()
     P.hps_solve(h, g, u)
@@ -88,6 +92,6 @@ def test_solves_around_a_callers_graph(P, kind, p, L, lazy):
         fin.copy_(fk)
         u.fill_(float("nan"))
         graph.replay()
-        assert torch.equal(u, wk)
+        assert same(u, wk)
     P.hps_solve(h, g2, v, f=f2)
-    assert torch.equal(v, w2)
+    assert same(v, w2)

@@ -36,6 +36,7 @@ __device__ __forceinline__ cplx shfl_v(cplx v, int src) {
 
 constexpr int NT = 128, NW = 4;   // threads and warps of a CTA
 constexpr int MAXN = 8;           // right-hand sides per launch column group
+constexpr size_t BLOCK_SMEM = 200 * 1024;   // most that k_trsv_block takes
 
 // ------------------------------------------------------------ many matrices
 
@@ -439,24 +440,32 @@ cudaError_t dispatch_cluster(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, co
 template <typename T, int NR, bool HERM>
 cudaError_t launch_block(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaStream_t st) {
   static const cudaError_t attr = cudaFuncSetAttribute(
-      k_trsv_block<T, NR, HERM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      k_trsv_block<T, NR, HERM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BLOCK_SMEM);
   if (attr != cudaSuccess) return attr;
   k_trsv_block<T, NR, HERM><<<dim3(batch, (nrhs + NR - 1) / NR), NT, block_smem<T>(n, NR, HERM), st>>>(LU, n, X, nrhs, batch);
   return cudaGetLastError();
 }
 
+// Columns that a launch for nrhs right-hand sides takes at a time; its shared
+// memory, and so the rule that takes the launch, go with them.
+int few_cols(int nrhs) { return nrhs <= 2 ? nrhs : nrhs <= 4 ? 4 : MAXN; }
+
 template <typename T, bool HERM>
 cudaError_t solve_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, const T* dinv, cudaStream_t st) {
   if (!dinv) {
-    if (nrhs == 1) return launch_block<T, 1, HERM>(LU, n, X, nrhs, batch, st);
-    if (nrhs == 2) return launch_block<T, 2, HERM>(LU, n, X, nrhs, batch, st);
-    if (nrhs <= 4) return launch_block<T, 4, HERM>(LU, n, X, nrhs, batch, st);
-    return launch_block<T, 8, HERM>(LU, n, X, nrhs, batch, st);
+    switch (few_cols(nrhs)) {
+      case 1: return launch_block<T, 1, HERM>(LU, n, X, nrhs, batch, st);
+      case 2: return launch_block<T, 2, HERM>(LU, n, X, nrhs, batch, st);
+      case 4: return launch_block<T, 4, HERM>(LU, n, X, nrhs, batch, st);
+      default: return launch_block<T, 8, HERM>(LU, n, X, nrhs, batch, st);
+    }
   }
-  if (nrhs == 1) return dispatch_cluster<T, 1, HERM>(LU, n, X, nrhs, batch, dinv, st);
-  if (nrhs == 2) return dispatch_cluster<T, 2, HERM>(LU, n, X, nrhs, batch, dinv, st);
-  if (nrhs <= 4) return dispatch_cluster<T, 4, HERM>(LU, n, X, nrhs, batch, dinv, st);
-  return dispatch_cluster<T, 8, HERM>(LU, n, X, nrhs, batch, dinv, st);
+  switch (few_cols(nrhs)) {
+    case 1: return dispatch_cluster<T, 1, HERM>(LU, n, X, nrhs, batch, dinv, st);
+    case 2: return dispatch_cluster<T, 2, HERM>(LU, n, X, nrhs, batch, dinv, st);
+    case 4: return dispatch_cluster<T, 4, HERM>(LU, n, X, nrhs, batch, dinv, st);
+    default: return dispatch_cluster<T, 8, HERM>(LU, n, X, nrhs, batch, dinv, st);
+  }
 }
 
 }  // namespace
@@ -479,7 +488,7 @@ bool trsv_few_applicable(int n, int nrhs, int batch, const TrsvInv* inv) {
   if (nrhs < 1 || nrhs > 2 * MAXN || n < 1) return false;
   if (inv && inv->p) return true;
   // one CTA per matrix: enough of them to fill the SMs, or small ones
-  return (n <= 64 || batch * 2 > device_sms()) && block_smem<T>(n, std::min(nrhs, MAXN), true) <= 200 * 1024;
+  return (n <= 64 || batch * 2 > device_sms()) && block_smem<T>(n, few_cols(nrhs), true) <= BLOCK_SMEM;
 }
 
 template <typename T>

@@ -502,7 +502,7 @@ hps_status adaptive_build(hps_handle* h, const hps_tree* tree, const hps_coeffs*
 
 static hps_status adaptive_ws(hps_handle* h, int nrhs) {
   using T = double;
-  if (h->ws_nrhs >= nrhs) return HPS_OK;
+  if (h->ws_nrhs == nrhs) return HPS_OK;   // the task tables hold the strides of one number of right-hand sides
   // the call has ordered h->last after the handle's earlier work
   for (void* pp : h->ws_allocs) dev_free(pp, h->last);
   h->ws_allocs.clear();

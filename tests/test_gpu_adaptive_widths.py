@@ -1,0 +1,51 @@
+"""GPU tests of adaptive solves whose number of right-hand sides changes from
+call to call on one operator: the workspace's task tables hold the strides of one
+number, and a workspace that could not grow must not be taken for the old one.
+
+Reference: the first solve of a second operator (the same kernels on the same
+data: equal up to the order of columns in a launch, 1e-12)."""
+
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import adaptive as ad
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def setup():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_17535_gb300 as P
+    p, pr = 6, W.elliptic_3d()
+    leaves = [(1, (i, j, k)) for i in range(2) for j in range(2) for k in range(2) if (i, j, k) != (0, 0, 0)]
+    t = P.adaptive_tree(ad.sort_leaves(leaves + ad.children_of(1, (0, 0, 0))), pr.lo, pr.hi)
+    x, _ = P.hps_nodes(t, p, p - 2)
+    nl, ppl, nr = P.hps_sizes(t, p, p - 2)
+    cf = pr.coeffs(x)
+    d = lambda v: torch.from_numpy(np.ascontiguousarray(v)).cuda()  # noqa: E731
+    a, b, c = d(cf["a"].reshape(nl, ppl)), [d(v.reshape(nl, ppl)) for v in cf["b"]], d(cf["c"].reshape(nl, ppl))
+    rng = np.random.default_rng(3)
+    g, f, f0 = d(rng.standard_normal((4, nr))), d(rng.standard_normal((4, nl, ppl))), d(rng.standard_normal((nl, ppl)))
+    build = lambda lazy: P.hps_build(t, p, p - 2, P.HPS_DTN, a=a, b=b, c=c, f=f0, lazy_root=lazy)  # noqa: E731
+    return P, build, g, f
+
+
+def _solve(P, h, n, g, f):
+    u = torch.full((n,) + f.shape[1:], float("nan"), dtype=torch.float64, device="cuda")
+    P.hps_solve_batched(h, n, g[:n].contiguous(), u, f=f[:n].contiguous())
+    v = torch.full_like(u, float("nan"))
+    P.hps_solve_batched(h, n, g[:n].contiguous(), v)
+    return torch.stack([u, v])
+
+
+@pytest.mark.parametrize("lazy", [False, True], ids=["explicit", "lazy"])
+def test_fewer_right_hand_sides_after_more(setup, lazy):
+    P, build, g, f = setup
+    h = build(lazy)
+    for n in (3, 1, 2, 4, 3):
+        got, ref = _solve(P, h, n, g, f), _solve(P, build(lazy), n, g, f)
+        assert bool((got - ref).abs().max() <= 1e-12 * ref.abs().max())

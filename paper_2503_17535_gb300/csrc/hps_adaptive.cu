@@ -542,9 +542,11 @@ static hps_status adaptive_ws(hps_handle* h, int nrhs) {
     G.dx = (T**)A(pb);
     G.dhp = (T**)A(pb);
     if (!G.dr || !G.dx || !G.dhp) return HPS_ERR_OOM;
-    if (cudaMemcpy(G.dr, vr.data(), pb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(G.dx, vx.data(), pb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(G.dhp, vh.data(), pb, cudaMemcpyHostToDevice) != cudaSuccess)
+    // on the call's stream: the pool may hand out the old workspace, which the
+    // solve before still reads
+    if (cudaMemcpyAsync(G.dr, vr.data(), pb, cudaMemcpyHostToDevice, h->last) != cudaSuccess ||
+        cudaMemcpyAsync(G.dx, vx.data(), pb, cudaMemcpyHostToDevice, h->last) != cudaSuccess ||
+        cudaMemcpyAsync(G.dhp, vh.data(), pb, cudaMemcpyHostToDevice, h->last) != cudaSuccess)
       return HPS_ERR_CUDA;
   }
   // task tables of the grouped solve passes, level by level (deepest first)
@@ -622,7 +624,8 @@ static hps_status adaptive_ws(hps_handle* h, int nrhs) {
         const size_t bytes = std::max<size_t>(vec.size() * sizeof(vec[0]), 16);
         void* d = A(bytes);
         if (!d) return false;
-        if (!vec.empty() && cudaMemcpy(d, vec.data(), vec.size() * sizeof(vec[0]), cudaMemcpyHostToDevice) != cudaSuccess)
+        if (!vec.empty() &&
+            cudaMemcpyAsync(d, vec.data(), vec.size() * sizeof(vec[0]), cudaMemcpyHostToDevice, h->last) != cudaSuccess)
           return false;
         *dst = (std::remove_reference_t<decltype(**dst)>*)d;
         *cnt = (int)vec.size();

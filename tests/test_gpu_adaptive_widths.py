@@ -1,6 +1,6 @@
 """GPU tests of adaptive solves whose number of right-hand sides changes from
 call to call on one operator: the workspace's task tables hold the strides of one
-number, and a workspace that could not grow must not be taken for the old one.
+number, and are written while the solve before may still read the old ones.
 
 Reference: the first solve of a second operator (the same kernels on the same
 data: equal up to the order of columns in a launch, 1e-12)."""
@@ -49,3 +49,24 @@ def test_fewer_right_hand_sides_after_more(setup, lazy):
     for n in (3, 1, 2, 4, 3):
         got, ref = _solve(P, h, n, g, f), _solve(P, build(lazy), n, g, f)
         assert bool((got - ref).abs().max() <= 1e-12 * ref.abs().max())
+
+
+def test_numbers_alternate_on_a_stream_of_its_own(setup):
+    """No synchronisation between the calls, and work before them on the stream."""
+    P, build, g, f = setup
+    h = build(False)
+    ref = {n: _solve(P, build(False), n, g, f)[0] for n in (1, 3, 4)}
+    st = torch.cuda.Stream()
+    busy = torch.randn(4096, 4096, device="cuda")
+    ins = {n: (g[:n].contiguous(), f[:n].contiguous()) for n in ref}
+    torch.cuda.synchronize()
+    got = []
+    with torch.cuda.stream(st):
+        for n in (3, 1, 4, 1, 3, 4, 3, 1) * 3:
+            for _ in range(4):
+                busy = busy @ busy * 1e-3
+            got.append((n, torch.empty((n,) + f.shape[1:], dtype=torch.float64, device="cuda")))
+            P.hps_solve_batched(h, n, ins[n][0], got[-1][1], f=ins[n][1])
+    torch.cuda.synchronize()
+    for n, u in got:
+        assert bool((u - ref[n]).abs().max() <= 1e-12 * ref[n].abs().max())

@@ -508,6 +508,7 @@ static hps_status adaptive_ws(hps_handle* h, int nrhs) {
   h->ws_allocs.clear();
   h->bytes -= h->ws_bytes;
   const int64_t before = h->bytes;
+  h->ws_nrhs = 0;   // nothing usable until every buffer is there
   const size_t es = sizeof(T);
   auto A = [&](size_t bytes) { return dalloc(h, bytes, &h->ws_allocs); };
   h->ws_xf = A((size_t)h->nl * h->xrows_leaf * nrhs * es);

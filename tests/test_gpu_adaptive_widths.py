@@ -70,3 +70,17 @@ def test_numbers_alternate_on_a_stream_of_its_own(setup):
     torch.cuda.synchronize()
     for n, u in got:
         assert bool((u - ref[n]).abs().max() <= 1e-12 * ref[n].abs().max())
+
+
+@pytest.mark.parametrize("k", [1, 4, 12, 40])
+def test_a_workspace_that_could_not_grow_is_made_anew(setup, k):
+    P, build, g, f = setup
+    h = build(False)
+    ref = _solve(P, h, 1, g, f)
+    P.hps_debug_fail_alloc(k)
+    try:
+        with pytest.raises(P.HPSError):
+            _solve(P, h, 3, g, f)
+    finally:
+        P.hps_debug_fail_alloc(0)
+    assert torch.equal(_solve(P, h, 1, g, f), ref)

@@ -15,8 +15,9 @@
 // D = p + q (weight 2^{4-8D}).  The product keeps the 36 pairs with p + q <= 9
 // and accumulates each diagonal exactly in its own TMEM accumulator over K
 // chunks of up to 128.  The epilogue reduces the eight diagonal sums to one
-// 64-bit fixed-point integer (exact down to 2^-57 or 2^-56, what lies below
-// rounded once) and scales it by 2^{e_i + f_j} into FP64.  Errors: operand
+// 64-bit fixed-point integer (as many fraction bits as the sum of K products
+// leaves: 63 - ceil(log2 K), at most 62; what lies below rounded once) and
+// scales it by 2^{e_i + f_j} into FP64.  Errors: operand
 // rounding 2^{-63} 2^{e_i} per entry (unbiased), dropped pairs at most
 // 2^{-59} K 2^{e_i + f_j}, half a unit of the fixed point per chunk, and the
 // final rounding to FP64: at or below FP64's own rounding error for a dot
@@ -77,7 +78,8 @@ constexpr int bstg(int tn) { return DIG * bblk(tn); }
 constexpr int EPI_WARPS = 16;       // four per TMEM lane quarter, each a quarter of the tile's columns
 constexpr int THREADS = 32 * EPI_WARPS + 64;   // + producer warp + MMA-issue warp
 constexpr long SPIN = 1L << 22;     // polls before a wait gives up
-constexpr int LSB1 = 57, LSB2 = 56; // fixed-point fraction bits of a KC = 64 tile, of a KC = 128 chunk
+constexpr int LSB1 = 57, LSB2 = 56; // fixed-point fraction bits of a full KC = 64 tile, of a full KC = 128 chunk
+constexpr int LSB_MAX = 62;
 
 // Shared memory: the copy ring; transposed tiles' staging (one block of
 // 32 x TN / 4 results per epilogue warp, odd stride); at TN = 32 two tiles of
@@ -97,6 +99,11 @@ static_assert(diag_max(9, KC2) < (1L << 24), "diagonal sums must stay exact in f
 static_assert(diag_max(6, KC1) <= (1L << 22) && diag_max(7, KC1) / 2 < (1L << 22), "KC = 64 conversion");
 static_assert(diag_max(4, KC2) <= (1L << 22) && diag_max(5, KC2) / 2 < (1L << 22) &&
               (diag_max(6, KC2) + 256) / 4 < (1L << 22) && (diag_max(7, KC2) + 512) / 4 < (1L << 22), "KC = 128 conversion");
+// the lowest diagonals enter in the unit of the result, 2^(LSB1 - lsb) / 8 or
+// 2^(LSB2 - lsb) / 16 of D = 8's, with n 2^(lsb - LSB1) <= 64 (n 2^(lsb - LSB2) <= 128) of
+// n summed products, and D = 7's remainder 256 times: that too is a float integer below 2^22
+static_assert((diag_max(8, KC1) + diag_max(9, KC1) / 256 + (256L << (LSB_MAX - LSB1))) / 8 < (1L << 22) &&
+              (diag_max(8, KC2) + diag_max(9, KC2) / 256 + (512L << (LSB_MAX - LSB2))) / 16 < (1L << 22), "lowest diagonals");
 static_assert(smem_bytes(64, true) <= 226 * 1024 && smem_bytes(64, false) <= 226 * 1024 &&
               smem_bytes(32, true) <= 226 * 1024 && smem_bytes(32, false) <= 226 * 1024, "shared memory too large");
 
@@ -368,8 +375,8 @@ __device__ __forceinline__ double fixed_fast(long long R, int E, uint32_t flip) 
 }
 
 // The eight diagonal sums x_D (exact floats) of one output as a fixed-point
-// integer, rounded once: units of 2^-57 (KC = 64) or 2^{-56 + sh} (KC = 128,
-// sh = 0 .. 6).  A sum below 2^22 becomes an integer with one addition (its
+// integer, rounded once: units of 2^{-57 + sh} (KC = 64, sh = -5 .. 0) or
+// 2^{-56 + sh} (KC = 128, sh = -6 .. 6; unit = 2^-sh / 8 or / 16).  A sum below 2^22 becomes an integer with one addition (its
 // bits after adding 1.5 * 2^23); a larger one is halved or quartered with
 // rounding and its small remainder handed to the next diagonal, where it is
 // 256 times as much and the sum stays below 2^24.  The two lowest diagonals
@@ -384,14 +391,14 @@ __device__ __forceinline__ long long diag_fixed(const float (&x)[NDIAG], int sh,
     const uint32_t a6 = __float_as_uint(x[4] + MG);
     const float h7 = fmaf(x[5], 0.5f, MG), r7 = fmaf(h7 - MG, -2.0f, x[5]);
     const float z = fmaf(r7, 256.0f, fmaf(x[7], 1.0f / 256.0f, x[6]));
-    const uint32_t c = __float_as_uint(fmaf(z, 1.0f / 8.0f, MG));              // units 2^-57
+    const uint32_t c = __float_as_uint(fmaf(z, unit, MG));                      // z / 8, units of 2^-57, at sh = 0
     // x6 2^13 + (x7 / 2) 2^6 + c; the offset of c's bits goes into the sum's
-    const int P = (int)(a6 * 128u + __float_as_uint(h7) - (129u * MB + (MB >> 6)));
+    const int P = (int)(a6 * 128u + __float_as_uint(h7) - (129u * MB + (MB >> (6 - sh))));
     const int Q = (int)(a4 * 256u + a5 - 257u * MB);                            // units 2^-36: 2^21
     const int S = (int)(a2 * 256u + a3 - 257u * MB);                            // units 2^-20: 2^37
-    long long w = (long long)P * 64 + (long long)(unsigned long long)c;
-    w += (long long)Q * (1ll << 21);
-    return w + ((long long)S << 37);
+    long long w = (long long)P * (1 << (6 - sh)) + (long long)(unsigned long long)c;
+    w += (long long)Q * (1 << (21 - sh));
+    return w + ((long long)S << (37 - sh));
   } else {
     const uint32_t a2 = __float_as_uint(x[0] + MG), a3 = __float_as_uint(x[1] + MG);
     const uint32_t a4 = __float_as_uint(x[2] + MG);
@@ -406,8 +413,8 @@ __device__ __forceinline__ long long diag_fixed(const float (&x)[NDIAG], int sh,
     const int P = (int)(__float_as_uint(h6) * 256u + __float_as_uint(h7) - (257u * MB + (MB >> (6 - sh))));
     const int Q = (int)(a4 * 128u + __float_as_uint(h5) - 129u * MB);           // x4 2^28 + (x5 / 2) 2^21
     const int S = (int)(a2 * 256u + a3 - 257u * MB);                            // 2^36
-    long long w = (long long)P * (64 >> sh) + (long long)(unsigned long long)c;
-    w += (long long)Q * (int)((1u << 21) >> sh);
+    long long w = (long long)P * (1 << (6 - sh)) + (long long)(unsigned long long)c;
+    w += (long long)Q * (1 << (21 - sh));
     return w + ((long long)S << (36 - sh));
   }
 }
@@ -606,8 +613,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(GemmP g) {
     constexpr int OSET = EPI_WARPS * 32 * ECOLS;   // doubles per staged tile
     constexpr int RSTEP = 32 / ECOLS;         // transposed: C columns per store
     const uint32_t flip = (uint32_t)((unsigned long long)g.asign >> 32);
-    const int sh = min(LSB2 - g.lsb, 6), sh2 = LSB2 - g.lsb - sh;   // KC = 128: unit of a chunk, rest beyond 6 bits
-    const float unit = 1.0f / (float)(16 << sh);
+    constexpr int LSBC = KC == KC1 ? LSB1 : LSB2;
+    const int sh = min(LSBC - g.lsb, 6), sh2 = LSBC - g.lsb - sh;   // unit of a chunk, rest beyond 6 bits
+    const float unit = __int_as_float((127 - (KC == KC1 ? 3 : 4) - sh) << 23);   // 2^-sh / 8, / 16
     struct Tile {
       double* Cp;          // this thread's first C entry (normal: its tile row; transposed: its tile column's row)
       int ebase, eb;       // exponent of its row (with the fixed point's), of column `lane`
@@ -1100,11 +1108,13 @@ cudaError_t gemm_tc(const GemmArgs<T>& g, cudaStream_t st, Prof* pf) {
     eb = reinterpret_cast<int*>(q); q += z.eb_item * nbb;
   }
   // chunk and fixed-point fraction bits, by the products summed per output (a
-  // complex component sums 2K): scaled entries stay below 1 - 2^-54, so the
-  // sum below 2^63 units with room for the chunks' roundings up to 2^17 terms
+  // complex component sums 2K; the padding of K adds zeros): scaled entries stay
+  // below 1 - 2^-54, so the sum below 2^63 units with room for the chunks'
+  // roundings up to 2^17 terms.  A fixed 57 or 56 bits up to 64 or 128 terms, as
+  // once here, lost up to five bits of short sums that cancel.
   const int ksum = NP * z.KT * TK;
   const int kc = ksum <= KC1 && !general ? KC1 : KC2;
-  const int lsb = kc == KC1 ? LSB1 : ksum <= KC2 ? LSB2 : (ksum <= 1 << 17 ? 63 : 62) - ceil_log2(ksum);
+  const int lsb = std::min(LSB_MAX, (ksum <= 1 << 17 ? 63 : 62) - ceil_log2((int64_t)NP * g.K));
   for (int b0 = 0; b0 < g.batch; b0 += nb_max) {
     const int nb = std::min(nb_max, g.batch - b0);
     SplitSet<T> ss;

@@ -190,9 +190,12 @@ __device__ __forceinline__ void put_digits(const double (&v)[8], int evm, uint8_
     unsigned long long m = full >> d;
     // ties to even (entries 2^-10 of the row's largest and below lose bits, few
     // at first, so that ties are common): up when the bits below the half bit
-    // (the lowest d - 10 of the mantissa) are not all zero or the integer is odd
-    uint32_t below;
-    asm("shl.b32 %0, %1, %2;" : "=r"(below) : "r"(ul), "r"(42 - d));   // 0 for shifts above 31
+    // (the lowest d - 10 of the mantissa: of its lower word, and from d = 43 on all of
+    // that and the lowest d - 42 of the upper) are not all zero or the integer is odd
+    uint32_t below, above;
+    asm("shl.b32 %0, %1, %2;" : "=r"(below) : "r"(ul), "r"(max(42 - d, 0)));   // 0 for shifts above 31
+    asm("shl.b32 %0, %1, %2;" : "=r"(above) : "r"(uh), "r"(74 - d));
+    below |= above;
     m = ev == 0 ? 0ull : (m + ((uint32_t)(m >> 1) & 1u | (below != 0u ? 1u : 0u))) >> 1;
     const unsigned long long t = (int)uh < 0 ? 0x8080808080808080ull - m : 0x8080808080808080ull + m;
     x[c][1] = (uint32_t)t;

@@ -72,7 +72,7 @@ def test_numbers_alternate_on_a_stream_of_its_own(setup):
         assert bool((u - ref[n]).abs().max() <= 1e-12 * ref[n].abs().max())
 
 
-@pytest.mark.parametrize("k", [1, 4, 12, 40])
+@pytest.mark.parametrize("k", [1, 4, 12, 30])
 def test_a_workspace_that_could_not_grow_is_made_anew(setup, k):
     P, build, g, f = setup
     h = build(False)

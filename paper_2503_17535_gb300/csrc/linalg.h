@@ -196,15 +196,16 @@ template <typename T>
 cudaError_t permute_rows(BOp<T> src, BOp<T> dst, const int* perm, int n, int nrhs, int batch,
                          cudaStream_t st, Prof* pf);
 
-// Inverses of the diagonal blocks of a batch of factors (trsv.cu): storage of
-// trsv_inv_elems elements that lives as long as the factors, filled by the
-// first solve with few right-hand sides that is not being captured into a graph
-// (a captured one records their formation, which every launch repeats).
+// Inverses of the diagonal blocks of a batch of factors, and a flag for each
+// (trsv.cu): storage of trsv_inv_elems elements that lives as long as the
+// factors, filled by the first solve with few right-hand sides that is not being
+// captured into a graph (a captured one records their formation, which every
+// launch repeats).
 struct TrsvInv {
   void* p = nullptr;
   bool ready = false;
 };
-inline int64_t trsv_inv_elems(int n, int64_t batch) { return batch * 2 * ((n + 31) / 32) * 1024; }
+inline int64_t trsv_inv_elems(int n, int64_t batch) { return batch * 2 * ((n + 31) / 32) * (1024 + 1); }
 // Whether solves of this batch take a cluster per matrix (and want a TrsvInv).
 bool trsv_cluster_wanted(int n, int64_t batch);
 // Whether a lazy root of order n takes the flag-ordered solve instead.

@@ -10,11 +10,12 @@
 // Few matrices: one thread-block cluster each (k_trsv_cluster).  The 32-row
 // blocks go round the CTAs; per block its owner sums the contributions of the
 // earlier ones, multiplies by the precomputed inverse of the diagonal block
-// (solve_inverses, once per factor) and writes the solution into the shared
-// memory of every CTA; after one cluster barrier every CTA subtracts its
-// contribution from its own later blocks.  The chain per block is two
-// 32 x 32 products on one SM (512 cycles each for real data), the barrier
-// and two short sums.
+// (k_block_inverses, once per factor), corrects the result by the inverse times
+// its residual if the block is ill-conditioned, and writes the solution into the
+// shared memory of every CTA; after one cluster barrier every CTA subtracts its
+// contribution from its own later blocks.  The chain per block is two 32 x 32
+// products on one SM (512 cycles each for real data), four with the correction,
+// the barrier and two or four short sums.
 //
 // The recursive form (one launch per 32-row block and one product per split)
 // took 17 us per launch whatever its size.  Solves with a new source, all
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X,
   const int64_t ld = LU.ld;
   T* Xb = X.item(b) + (int64_t)c0 * X.ld;
   const T* Db = dinv + (int64_t)b * 2 * nblk * 1024;
+  const T* Fb = dinv + ((int64_t)(gridDim.x / CS) * 1024 + b) * 2 * nblk;   // which blocks want the correction
   // own blocks: g, g + CS, ...
   for (int e = threadIdx.x; e < MO * 32 * NR; e += NT) {
     const int r = e % 32, k = e / 32 % MO, c = e / (32 * MO);
@@ -188,6 +190,27 @@ __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X,
       for (int q = 0; q < QW; ++q) m[q] = tw[lane * (QW + 1) + q];
     }
   };
+  auto load_block = [&](int i, int j, T (&m)[QW]) {
+    if (!HERM) tile(A + (int64_t)i * 32 + (int64_t)j * 32 * ld, ld, n - i * 32, n - j * 32, m);
+    else tile(A + (int64_t)j * 32 + (int64_t)i * 32 * ld, ld, n - j * 32, n - i * 32, m);
+  };
+  // block j of the first or second triangle itself
+  auto load_triangle = [&](int tri, int j, T (&m)[QW]) {
+    load_block(j, j, m);
+    const bool unit = (tri == 0) != HERM;
+#pragma unroll
+    for (int q = 0; q < QW; ++q) {
+      const int c = QW * w + q;
+      if (tri == 0 ? lane < c : lane > c) m[q] = T(0.0);
+      else if (lane == c && unit) m[q] = T(1.0);
+    }
+  };
+  // its inverse; returns whether a product with that wants the correction
+  auto load_inverse = [&](int tri, int j, T (&m)[QW]) {
+    const int at = (HERM ? 1 - tri : tri) * nblk + j;
+    tile(Db + (int64_t)at * 1024, 32, 32, 32, m);
+    return !is_zero(Fb[at]);
+  };
   T acc[MO][NR];   // contributions of the solved blocks to own block k (this warp's columns)
   auto clear = [&]() {
 #pragma unroll
@@ -195,55 +218,60 @@ __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X,
 #pragma unroll
       for (int c = 0; c < NR; ++c) acc[k][c] = T(0.0);
   };
-  // block j's solution from its right-hand side and contributions, to every
-  // CTA's slot
-  auto solve = [&](const T (&dm)[QW], int j, int slot) {
+  // the sum over the warps of their v, in one of two buffers in turn
+  auto total = [&](T (&v)[NR], T* p) {
+#pragma unroll
+    for (int c = 0; c < NR; ++c) p[(w * 32 + lane) * NR + c] = v[c];
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NR; ++c)
+      v[c] = (p[lane * NR + c] + p[(32 + lane) * NR + c]) + (p[(64 + lane) * NR + c] + p[(96 + lane) * NR + c]);
+  };
+  // v <- M b, this warp's columns of M in m
+  auto product = [&](const T (&m)[QW], const T (&b)[NR], T (&v)[NR], T* p) {
+#pragma unroll
+    for (int c = 0; c < NR; ++c) v[c] = T(0.0);
+#pragma unroll
+    for (int q = 0; q < QW; ++q)
+#pragma unroll
+      for (int c = 0; c < NR; ++c) v[c] = fmac(v[c], m[q], shfl_v(b[c], QW * w + q));
+    total(v, p);
+  };
+  // block j's solution from its right-hand side and contributions, to every CTA's
+  // slot; dm: the inverse of its diagonal block
+  auto solve = [&](const T (&dm)[QW], bool correct, int tri, int j, int slot) {
     const int kj = j / CS;
-    T a[NR];
+    T* part2 = part + NW * 32 * NR;
+    T y[NR], x[NR], v[NR];
 #pragma unroll
     for (int k = 0; k < MO; ++k)
       if (k == kj) {
 #pragma unroll
-        for (int c = 0; c < NR; ++c) a[c] = acc[k][c];
+        for (int c = 0; c < NR; ++c) v[c] = acc[k][c];
       }
+    total(v, part);
 #pragma unroll
-    for (int c = 0; c < NR; ++c) part[(w * 32 + lane) * NR + c] = a[c];
-    __syncthreads();
-    T y[NR];
+    for (int c = 0; c < NR; ++c) y[c] = xs[(kj * 32 + lane) * NR + c] + v[c];
+    product(dm, y, x, part2);
+    if (correct) {   // uniform over the CTA
+      T tm[QW];
+      load_triangle(tri, j, tm);
+      product(tm, x, v, part);
 #pragma unroll
-    for (int c = 0; c < NR; ++c) {
-      y[c] = xs[(kj * 32 + lane) * NR + c] + ((part[lane * NR + c] + part[(32 + lane) * NR + c]) +
-                                              (part[(64 + lane) * NR + c] + part[(96 + lane) * NR + c]));
-      a[c] = T(0.0);
+      for (int c = 0; c < NR; ++c) y[c] = y[c] - v[c];
+      product(dm, y, v, part2);
+#pragma unroll
+      for (int c = 0; c < NR; ++c) x[c] = x[c] + v[c];
     }
-#pragma unroll
-    for (int q = 0; q < QW; ++q)
-#pragma unroll
-      for (int c = 0; c < NR; ++c) a[c] = fmac(a[c], dm[q], shfl_v(y[c], QW * w + q));
-    T* p2 = part + NW * 32 * NR;
-#pragma unroll
-    for (int c = 0; c < NR; ++c) p2[(w * 32 + lane) * NR + c] = a[c];
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < NR; ++c)
-      y[c] = (p2[lane * NR + c] + p2[(32 + lane) * NR + c]) + (p2[(64 + lane) * NR + c] + p2[(96 + lane) * NR + c]);
     for (int d = w; d < CS; d += NW) {
       T* dst = cl.map_shared_rank(xbuf, d) + (slot * 32 + lane) * NR;
 #pragma unroll
-      for (int c = 0; c < NR; ++c) dst[c] = y[c];
+      for (int c = 0; c < NR; ++c) dst[c] = x[c];
     }
     if (w == 0) {
 #pragma unroll
-      for (int c = 0; c < NR; ++c) xs[(kj * 32 + lane) * NR + c] = y[c];
+      for (int c = 0; c < NR; ++c) xs[(kj * 32 + lane) * NR + c] = x[c];
     }
-  };
-  // own block k less block j's contribution
-  auto load_block = [&](int i, int j, T (&m)[QW]) {
-    if (!HERM) tile(A + (int64_t)i * 32 + (int64_t)j * 32 * ld, ld, n - i * 32, n - j * 32, m);
-    else tile(A + (int64_t)j * 32 + (int64_t)i * 32 * ld, ld, n - j * 32, n - i * 32, m);
-  };
-  auto load_inverse = [&](int tri, int j, T (&m)[QW]) {   // of L's (0) or U's (1) diagonal block
-    tile(Db + ((int64_t)(HERM ? 1 - tri : tri) * nblk + j) * 1024, 32, 32, 32, m);
   };
   auto update = [&](const T (&m)[QW], int k, int slot) {
     const T* xq = xbuf + (slot * 32 + QW * w) * NR;
@@ -266,8 +294,8 @@ __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X,
   clear();
   if (g == 0) {
     T dm[QW];
-    load_inverse(0, 0, dm);
-    solve(dm, 0, 0);
+    const bool correct = load_inverse(0, 0, dm);
+    solve(dm, correct, 0, 0, 0);
   }
   cluster_arrive();
   // Step s: block block_at(tri, t) has been solved; its barrier tells every
@@ -285,15 +313,16 @@ __global__ void __launch_bounds__(NT) k_trsv_cluster(BOp<T> LU, int n, BOp<T> X,
     const int tri1 = turn_round ? 1 : tri, j1 = turn_round ? nblk - 1 : block_at(tri, t + 1);
     const bool mine = s + 1 < 2 * nblk && j1 % CS == g;
     T m1[QW], dm[QW];
+    bool correct = false;
     if (mine) {
       if (!turn_round) load_block(j1, j, m1);
-      load_inverse(tri1, j1, dm);
+      correct = load_inverse(tri1, j1, dm);
     }
     cluster_wait();
     if (turn_round) clear();
     if (mine) {
       if (!turn_round) update(m1, j1 / CS, slot);
-      solve(dm, j1, slot1);
+      solve(dm, correct, tri1, j1, slot1);
     }
     if (s + 1 < 2 * nblk) cluster_arrive();
     if (!turn_round) {
@@ -333,10 +362,22 @@ size_t cluster_smem(int nr, int mo) {
 // the factorisation).  One CTA per block and triangle: four threads per
 // column of the identity, 8 rows each, the row groups solved in order and
 // broadcast by shuffles.
+//
+// Behind them a flag per block: whether a product with the inverse wants a
+// correction.  The product's residual is up to || |T| |T^-1| || (for the conjugate
+// transpose, the one-norm of |T^-1| |T|) times a substitution's.  Residuals for
+// random right-hand sides, rms in units of 1e-17 of |T| |x| + |y|, substitution /
+// product, by that norm: 8 to 16 5.5 / 6.9, 16 to 32 4.5 / 6.6, 32 to 64 4.5 / 6.9, 64 to
+// 96 4.2 / 7.0 (the blocks of all merges of the elliptic and Helmholtz operators), 512
+// to 4096 6.9 / 217, above 4.0 / 46 (dense impedance leaves).  Solutions of the former
+// have the same errors with and without the correction; the line lies between.
+constexpr double CORRECT_FROM = 256.0;
 template <typename T>
 __global__ void __launch_bounds__(128) k_block_inverses(BOp<T> LU, int n, T* out) {
   __shared__ T Ls[32 * 32];
   __shared__ T dv[32];
+  __shared__ double mv[32 * 33];   // magnitudes of the inverse
+  __shared__ int wants[2];
   const int j = blockIdx.x, nblk = gridDim.x, b = blockIdx.z;
   const bool upper = blockIdx.y == 1;
   const int pb = min(32, n - j * 32);
@@ -384,9 +425,30 @@ __global__ void __launch_bounds__(128) k_block_inverses(BOp<T> LU, int n, T* out
         for (int q = 0; q < 8; ++q) x[i] = fmsc(x[i], Ls[(8 * g + i) + (8 * blk + q) * 32], xb[q]);
     }
   }
-  T* o = out + (((int64_t)b * 2 + blockIdx.y) * nblk + j) * 1024 + 32 * col + 8 * g;
+  const int64_t at = ((int64_t)b * 2 + blockIdx.y) * nblk + j;
+  T* o = out + at * 1024 + 32 * col + 8 * g;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) o[i] = x[i];
+  for (int i = 0; i < 8; ++i) {
+    o[i] = x[i];
+    mv[(8 * g + i) * 33 + col] = mag1(x[i]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    // |T| (|V| 1), a row per lane (warp 0), or (1 |V|) |T|, a column per lane (warp 1)
+    const int lane = threadIdx.x & 31;
+    const bool rows = threadIdx.x < 32;
+    double sum = 0.0, norm = 0.0;
+    for (int k = 0; k < 32; ++k) sum += rows ? mv[lane * 33 + k] : mv[k * 33 + lane];
+    for (int k = 0; k < 32; ++k) {
+      const int r = rows ? lane : k, c = rows ? k : lane;
+      const double t = r == c && !upper ? 1.0 : (upper ? r <= c : r >= c) ? mag1(Ls[r + c * 32]) : 0.0;
+      norm = fma(t, __shfl_sync(0xffffffffu, sum, k), norm);
+    }
+    const bool over = __any_sync(0xffffffffu, !(norm <= CORRECT_FROM));
+    if (lane == 0) wants[rows ? 0 : 1] = over;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) out[(int64_t)gridDim.z * 2 * nblk * 1024 + at] = T(wants[0] || wants[1] ? 1.0 : 0.0);
 }
 
 // Cluster shape: a power of two of CTAs, at most 16, the SMs' share of a

@@ -309,13 +309,16 @@ __global__ void __launch_bounds__(256) k_gemm_skinny_kg(GemmArgs<T> g) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[c] = T(0.0);
     if (act) {
-      // eight entries (and their gathered indices) in flight
+      // U entries of A and U NC of B (and their gathered indices) in flight: more
+      // than 16 doubles of B cost warps (64 items of 300 x 300 with five columns, whole
+      // call: 8 / 4 / 2 entries real 331 / 289 / 286 us, complex 760 / 646 / 579)
+      constexpr int U0 = 16 / (NC * (int)(sizeof(T) / sizeof(double))), U = U0 > 8 ? 8 : U0 < 2 ? 2 : U0;
       const int* ac = g.acol.idx ? g.acol.idx + (b % g.acol.period) * g.acol.len : nullptr;
       const int* bi = g.brow.idx ? g.brow.idx + (b % g.brow.period) * g.brow.len : nullptr;
-      for (int l0 = w; l0 < g.K; l0 += 64) {
-        T a[8], x[8][NC];
+      for (int l0 = w; l0 < g.K; l0 += 8 * U) {
+        T a[U], x[U][NC];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < U; ++k) {
           const int l = l0 + 8 * k;
           const bool in = l < g.K;
           a[k] = in ? A[ar + (int64_t)(ac ? ac[l] : l) * g.A.ld] : T(0.0);
@@ -324,7 +327,7 @@ __global__ void __launch_bounds__(256) k_gemm_skinny_kg(GemmArgs<T> g) {
           for (int c = 0; c < NC; ++c) x[k][c] = in && c < g.N ? B[br + (int64_t)c * g.B.ld] : T(0.0);
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
+        for (int k = 0; k < U; ++k)
 #pragma unroll
           for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], a[k], x[k][c]);
       }

@@ -99,8 +99,8 @@ inline int epi_mode(const GemmArgs<T>& g) {
 
 // Products on the FP64 pipe, N > 8: BM x 256 / BM tiles (BM = 32, 16 or 8 rows,
 // whichever pads the shape least), four warps, a thread per row and
-// pair of columns, 32 steps of K staged at once with the next 32 in flight in
-// registers.
+// pair of columns, 32 steps of K (complex: 16) staged at once with the next in
+// flight in registers.
 //
 // The pipe does two multiply-adds per clock and SM, so that even these small
 // tiles need only 2.5 of the 30 bytes per clock that L2 delivers to an SM; what
@@ -114,7 +114,10 @@ inline int epi_mode(const GemmArgs<T>& g) {
 // the real products P1 = Ar Br, P2 = Ai Bi and P3 = (Ar + Ai)(Br + Bi) give
 // C = (P1 - P2) + i (P3 - P1 - P2).  Each complex multiply-add costs three
 // real FMAs instead of four on the FP64 pipe; the sums Ar + Ai and Br + Bi
-// are formed once per element when the tile is staged in shared memory.
+// are formed once per element when the tile is staged in shared memory.  The
+// three planes of 32 steps would leave room for seven CTAs per SM and load past
+// short K: 4096 items of 28 x 28 x 16 and 64 x 114 x 4 take 584 and 1288 us (whole
+// call) with 32 steps, 550 and 1132 with 16, longer K the same.
 // With MODE == EPI_SUB the accumulators start from C so that the update
 // needs three additions per element: p1 = 0, p2 = Re C, p3 = Re C - Im C give
 // Re(C - AB) = p2 - p1 and Im(C - AB) = p1 + p2 - p3 after the products.
@@ -126,12 +129,13 @@ __device__ __forceinline__ double gemm_plane(cplx v, int p) { return p == 0 ? v.
 
 template <typename T, int MODE, int BM>
 __global__ void __launch_bounds__(128) k_gemm(GemmArgs<T> g) {
-  constexpr int P = GemmPlanes<T>::N, BN = 256 / BM, BK = 32, LA = BM / 4, LB = BN / 4;
+  constexpr int P = GemmPlanes<T>::N, BN = 256 / BM, BK = P == 1 ? 32 : 16, LA = BM * BK / 128, LB = BN * BK / 128;
   __shared__ double As[P][BK][BM];
   __shared__ __align__(16) double Bs[P][BK][BN + 2];   // + 2: the staging writes go down a column
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int tid = threadIdx.x;
   const int r = tid % BM, c0 = 2 * (tid / BM);   // this thread's row and columns c0, c0 + 1 of the tile
   const int ra = tid % BM, la = tid / BM;        // what it stages of A: row ra, steps la, la + 128 / BM, ...
+  const int lb = tid % BK, cb = tid / BK;        // and of B: step lb, columns cb, cb + 128 / BK, ...
   const int tiles_m = (g.M + BM - 1) / BM;
   const int i = blockIdx.x % tiles_m * BM + r, j0 = blockIdx.x / tiles_m * BN;
   const bool beta = MODE == EPI_SUB || (MODE == EPI_GENERAL && !is_zero(g.beta));
@@ -149,11 +153,11 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs<T> g) {
         const int l = k0 + la + 128 / BM * u;
         a[u] = row && l < g.K ? A[ai + (int64_t)g.acol.at(b, l) * g.A.ld] : T(0.0);
       }
-      const int l = k0 + lane;
+      const int l = k0 + lb;
       const int64_t bi = l < g.K ? g.brow.at(b, l) : 0;
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        const int j = j0 + w + 4 * u;
+        const int j = j0 + cb + 128 / BK * u;
         bb[u] = l < g.K && j < g.N ? B[bi + (int64_t)j * g.B.ld] : T(0.0);
       }
     };
@@ -181,7 +185,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs<T> g) {
         for (int u = 0; u < LA; ++u)
           if (la + 128 / BM * u < kc) As[p][la + 128 / BM * u][ra] = gemm_plane(a[u], p);
 #pragma unroll
-        for (int u = 0; u < LB; ++u) Bs[p][lane][w + 4 * u] = gemm_plane(bb[u], p);
+        for (int u = 0; u < LB; ++u) Bs[p][lb][cb + 128 / BK * u] = gemm_plane(bb[u], p);
       }
       __syncthreads();
       if (k0 + BK < g.K) load(k0 + BK);

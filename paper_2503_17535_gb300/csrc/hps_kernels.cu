@@ -463,6 +463,7 @@ cudaError_t merge_gather_h(const T* hc, int nmerge, int nch, int nbc, int n_ext,
 // very long rows, the ranges cost locality: 432 real tiles 94 -> 137, 216 of
 // 13824 columns 246 -> 265).  With one warp per 32 rows up to 255 columns, as
 // before, 64 real merges of 176 columns took 80 us, now 12.
+constexpr int64_t kDownL2 = 64 << 20;
 constexpr int kGridY = 65535;   // groups of right-hand sides in one launch (grid limit)
 template <typename T, int CG, int NC, bool CL>
 __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X, const T* xp, const T* gpar,
@@ -582,7 +583,12 @@ cudaError_t launch_down_gint(const T* X, const T* xp, const T* gpar, int nmerge,
   // groups of four, 105 one by one; 224 tiles: 96 in groups of four, 115 of three)
   int most = 4;
   while (most > 1 && 2 * tiles * ((nrhs + most - 1) / most) < 5 * device_sms()) --most;
-  const int nc = rhs_group(nrhs, most);
+  int nc = rhs_group(nrhs, most);
+  // While L2 keeps X (up to half of it) groups save no memory traffic.  Complex
+  // rows are then bound by the pipe anyway and finish sooner one by one (128 tiles
+  // of 256 columns, eight right-hand sides: 68 us, in groups of three 90), real ones when
+  // the last group would be short (192 tiles of 192, five: 18 us, in groups of three 29).
+  if (rows * n_ext * (int64_t)sizeof(T) < kDownL2 && (sizeof(T) == 16 || nrhs % nc != 0)) nc = 1;
   const int64_t warps = tiles * ((nrhs + nc - 1) / nc);
   const bool cluster = warps < 2 * device_sms() && n_ext < 8192;
   const int cg = down_groups(warps, n_ext, cluster ? 32 : 16);

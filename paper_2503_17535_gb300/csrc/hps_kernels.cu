@@ -683,16 +683,15 @@ struct LeafRow {
   }
 };
 
-// u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides, so
-// that an entry of Y serves NC multiply-adds.  Bound by the FP64 pipe (385 us
+// u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides (a
+// divisor of nrhs), so that an entry of Y serves NC multiply-adds.  Bound by the FP64 pipe (385 us
 // for 4096 complex leaves of 256 x 56, of which the pipe needs 392 at its nominal
-// rate); one right-hand side per thread read every entry from L2 again for
-// each and walked a warp's boundary and interior nodes one after the other: 1533
-// us for eight real ones, now 784.
+// rate; eight real right-hand sides 784, and 1533 while a warp walked its boundary
+// and interior nodes one after the other).
 template <typename T, int NC>
 __global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, int nrhs, const T* X, const T* xp,
                                                      const T* g, T* u, bool iti) {
-  const int64_t total = (int64_t)((nrhs + NC - 1) / NC) * nl * k.npts;
+  const int64_t total = (int64_t)(nrhs / NC) * nl * k.npts;
   const int xrows = iti ? k.npts : k.ni;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -702,29 +701,25 @@ __global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, i
     const int c0 = (int)(lc / nl) * NC;
     const T* gl = g + (leaf * nrhs + c0) * (int64_t)k.nb;
     const T* Xl = X + leaf * (int64_t)xrows * (k.nb + 1);
-    int go[NC];   // columns beyond the last repeat it
     T acc[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) go[c] = min(c, nrhs - 1 - c0) * k.nb;
     const LeafRow<T> row(k, iti, node, Xl, xrows);
 #pragma unroll
     for (int c = 0; c < NC; ++c)
       acc[c] = row.edge ? T(0.0)
-               : xp     ? xp[(leaf * nrhs + min(c0 + c, nrhs - 1)) * (int64_t)xrows + row.r]
+               : xp     ? xp[(leaf * nrhs + c0 + c) * (int64_t)xrows + row.r]
                         : Xl[row.r + (int64_t)k.nb * xrows];
 #pragma unroll 4
     for (int j = 0; j < k.nb; ++j) {
       const T x = row.at(j);
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], x, gl[go[c] + j]);
+      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], x, gl[c * k.nb + j]);
     }
     if (row.negate) {
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[c] = -acc[c];
     }
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (c0 + c < nrhs) u[((c0 + c) * nl + leaf) * k.npts + node] = acc[c];
+    for (int c = 0; c < NC; ++c) u[((c0 + c) * nl + leaf) * k.npts + node] = acc[c];
   }
 }
 
@@ -733,13 +728,19 @@ cudaError_t leaf_output(const LeafConsts& k, int64_t nl, int nrhs, const T* X, c
                         T* u, bool iti, cudaStream_t st, Prof* pf) {
   const double F = sizeof(T) == sizeof(cplx) ? 8.0 : 2.0;
   if (pf) pf->begin(st);
-  const int nc = rhs_group(nrhs, 4);
-  const int grid = grid_for((int64_t)((nrhs + nc - 1) / nc) * nl * k.npts);
-  switch (nc) {
-    case 1: k_leaf_output<T, 1><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
-    case 2: k_leaf_output<T, 2><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
-    case 3: k_leaf_output<T, 3><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
-    default: k_leaf_output<T, 4><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti); break;
+  // Whole groups of four or three real right-hand sides when seven CTAs per SM
+  // are left to hide the loads; else, and for complex data, one by one (us, nodes x
+  // right-hand sides, one by one / in fours or threes: real 1048576 x 8 834 / 782 and x 3
+  // 324 / 301, 262144 x 16 406 / 397, 32768 x 24 295 / 332, 1728 x 8 16 / 33; x 5, in
+  // threes, 1048576 524 / 590; complex 262144 x 8 772 / 803, 65536 x 8 205 / 238)
+  int nc = 1;
+  if constexpr (sizeof(T) == sizeof(double)) nc = nrhs % 4 == 0 ? 4 : nrhs % 3 == 0 ? 3 : 1;
+  if (nl * k.npts * (nrhs / nc) < 262144) nc = 1;
+  const int grid = grid_for((int64_t)(nrhs / nc) * nl * k.npts);
+  if (nc == 1) k_leaf_output<T, 1><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (nc == 3) k_leaf_output<T, 3><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti);
+    if (nc == 4) k_leaf_output<T, 4><<<grid, 256, 0, st>>>(k, nl, nrhs, X, xp, g, u, iti);
   }
   if (pf) pf->end(K_DOWN, F * (double)nrhs * nl * k.npts * k.nb, st);
   return cudaGetLastError();

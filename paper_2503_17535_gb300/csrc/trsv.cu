@@ -39,6 +39,10 @@ constexpr int NT = 128, NW = 4;   // threads and warps of a CTA
 constexpr int MAXN = 8;           // right-hand sides per launch column group
 constexpr size_t BLOCK_SMEM = 200 * 1024;   // most that k_trsv_block takes
 
+// Columns that a CTA of a launch for nrhs right-hand sides takes at a time; its
+// shared memory, and so the rule that takes the launch, go with them.
+int few_cols(int nrhs) { return nrhs <= 2 ? nrhs : nrhs <= 4 ? 4 : MAXN; }
+
 // ------------------------------------------------------------ many matrices
 
 // Entry (r, c) of the 32 x 32 block whose rows start at i0 and columns at j0 of
@@ -491,12 +495,22 @@ cudaError_t dispatch_cluster(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, co
   const int cs = cluster_of(n, batch), mo = own_blocks(n, cs);
   // the partial sums of all own blocks stay in registers: at most 64 of them,
   // more columns go to further clusters
-  constexpr int W = (int)(sizeof(T) / 4);
-  constexpr int N2 = NR * 2 * W <= 64 ? NR : NR / 2, N4 = NR * 4 * W <= 64 ? NR : 64 / (4 * W),
-                N8 = NR * 8 * W <= 64 ? NR : 64 / (8 * W);
-  if (mo <= 2) return launch_cluster<T, N2, HERM, 2>(LU, n, X, nrhs, batch, cs, dinv, st);
-  if (mo <= 4) return launch_cluster<T, N4, HERM, 4>(LU, n, X, nrhs, batch, cs, dinv, st);
+  constexpr int N8 = NR < 4 ? NR : 4;
+  if (mo <= 2) return launch_cluster<T, NR, HERM, 2>(LU, n, X, nrhs, batch, cs, dinv, st);
+  if (mo <= 4) return launch_cluster<T, NR, HERM, 4>(LU, n, X, nrhs, batch, cs, dinv, st);
   return launch_cluster<T, N8, HERM, 8>(LU, n, X, nrhs, batch, cs, dinv, st);
+}
+
+// Columns that a cluster takes at a time.  A column of its own: a step's chain is
+// mostly the multiply-adds of its own CTA, and clusters beside one another fill
+// the SMs (us, one / two / four / eight columns a cluster: eight complex columns of one
+// matrix of 512 217 / 244 / 472 / 1024, of 16 of 448 375 / 514 / 547 / 993; eight real
+// columns of eight of 1728 726 / 982 / 1385 / 1441).  Real columns of many matrices,
+// whose short clusters fill the SMs alone, share the matrix's entries (64 of 432, four
+// columns 291 / 217 / 255 / 254, eight 457 / 434 / 330 / 326).
+template <typename T>
+int cluster_cols(int nrhs, int batch) {
+  return sizeof(T) == 16 || batch <= 16 || nrhs < 4 ? 1 : few_cols(nrhs);
 }
 
 template <typename T, int NR, bool HERM>
@@ -508,10 +522,6 @@ cudaError_t launch_block(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, cudaSt
   return cudaGetLastError();
 }
 
-// Columns that a launch for nrhs right-hand sides takes at a time; its shared
-// memory, and so the rule that takes the launch, go with them.
-int few_cols(int nrhs) { return nrhs <= 2 ? nrhs : nrhs <= 4 ? 4 : MAXN; }
-
 template <typename T, bool HERM>
 cudaError_t solve_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, const T* dinv, cudaStream_t st) {
   if (!dinv) {
@@ -522,12 +532,12 @@ cudaError_t solve_few(BOp<T> LU, int n, BOp<T> X, int nrhs, int batch, const T* 
       default: return launch_block<T, 8, HERM>(LU, n, X, nrhs, batch, st);
     }
   }
-  switch (few_cols(nrhs)) {
-    case 1: return dispatch_cluster<T, 1, HERM>(LU, n, X, nrhs, batch, dinv, st);
-    case 2: return dispatch_cluster<T, 2, HERM>(LU, n, X, nrhs, batch, dinv, st);
-    case 4: return dispatch_cluster<T, 4, HERM>(LU, n, X, nrhs, batch, dinv, st);
-    default: return dispatch_cluster<T, 8, HERM>(LU, n, X, nrhs, batch, dinv, st);
+  const int nc = cluster_cols<T>(nrhs, batch);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (nc == 4) return dispatch_cluster<T, 4, HERM>(LU, n, X, nrhs, batch, dinv, st);
+    if (nc == 8) return dispatch_cluster<T, 8, HERM>(LU, n, X, nrhs, batch, dinv, st);
   }
+  return dispatch_cluster<T, 1, HERM>(LU, n, X, nrhs, batch, dinv, st);
 }
 
 }  // namespace

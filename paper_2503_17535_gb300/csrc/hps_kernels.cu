@@ -463,7 +463,7 @@ cudaError_t merge_gather_h(const T* hc, int nmerge, int nch, int nbc, int n_ext,
 // very long rows, the ranges cost locality: 432 real tiles 94 -> 137, 216 of
 // 13824 columns 246 -> 265).  With one warp per 32 rows up to 255 columns, as
 // before, 64 real merges of 176 columns took 80 us, now 12.
-constexpr int64_t kDownL2 = 64 << 20;
+constexpr int64_t kDownL2 = 64 << 20;   // bytes of X that stay in L2 between groups
 constexpr int kGridY = 65535;   // groups of right-hand sides in one launch (grid limit)
 template <typename T, int CG, int NC, bool CL>
 __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X, const T* xp, const T* gpar,
@@ -683,15 +683,15 @@ struct LeafRow {
   }
 };
 
-// u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides (a
-// divisor of nrhs), so that an entry of Y serves NC multiply-adds.  Bound by the FP64 pipe (385 us
+// u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides, so
+// that an entry of Y serves NC multiply-adds.  Bound by the FP64 pipe (385 us
 // for 4096 complex leaves of 256 x 56, of which the pipe needs 392 at its nominal
 // rate; eight real right-hand sides 784, and 1533 while a warp walked its boundary
 // and interior nodes one after the other).
 template <typename T, int NC>
 __global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, int nrhs, const T* X, const T* xp,
                                                      const T* g, T* u, bool iti) {
-  const int64_t total = (int64_t)(nrhs / NC) * nl * k.npts;
+  const int64_t total = (int64_t)((nrhs + NC - 1) / NC) * nl * k.npts;
   const int xrows = iti ? k.npts : k.ni;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -701,25 +701,29 @@ __global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, i
     const int c0 = (int)(lc / nl) * NC;
     const T* gl = g + (leaf * nrhs + c0) * (int64_t)k.nb;
     const T* Xl = X + leaf * (int64_t)xrows * (k.nb + 1);
+    int go[NC];   // columns beyond the last repeat it
     T acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) go[c] = min(c, nrhs - 1 - c0) * k.nb;
     const LeafRow<T> row(k, iti, node, Xl, xrows);
 #pragma unroll
     for (int c = 0; c < NC; ++c)
       acc[c] = row.edge ? T(0.0)
-               : xp     ? xp[(leaf * nrhs + c0 + c) * (int64_t)xrows + row.r]
+               : xp     ? xp[(leaf * nrhs + min(c0 + c, nrhs - 1)) * (int64_t)xrows + row.r]
                         : Xl[row.r + (int64_t)k.nb * xrows];
 #pragma unroll 4
     for (int j = 0; j < k.nb; ++j) {
       const T x = row.at(j);
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], x, gl[c * k.nb + j]);
+      for (int c = 0; c < NC; ++c) acc[c] = fmac(acc[c], x, gl[go[c] + j]);
     }
     if (row.negate) {
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[c] = -acc[c];
     }
 #pragma unroll
-    for (int c = 0; c < NC; ++c) u[((c0 + c) * nl + leaf) * k.npts + node] = acc[c];
+    for (int c = 0; c < NC; ++c)
+      if (c0 + c < nrhs) u[((c0 + c) * nl + leaf) * k.npts + node] = acc[c];
   }
 }
 

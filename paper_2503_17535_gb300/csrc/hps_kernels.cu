@@ -539,9 +539,10 @@ inline int rhs_group(int nrhs, int most) {
   return (nrhs + groups - 1) / groups;
 }
 
+// the right-hand sides [cfirst, cend) of nrhs
 template <typename T, int CG, int NC, bool CL>
 cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t rows, int n_ext, int n_int, int nrhs,
-                                int cs, T* gint, cudaStream_t st) {
+                                int cfirst, int cend, int cs, T* gint, cudaStream_t st) {
   constexpr int NW = CG < 4 ? 4 : CG;
   const int per = 32 * (NW / CG);
   cudaLaunchConfig_t cfg = {};
@@ -556,8 +557,8 @@ cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t 
   cfg.attrs = at;
   cfg.numAttrs = CL ? 1 : 0;
   cudaError_t e = cudaSuccess;
-  for (int c = 0; c < nrhs && e == cudaSuccess; c += kGridY * NC) {
-    cfg.gridDim.y = std::min(kGridY, (nrhs - c + NC - 1) / NC);
+  for (int c = cfirst; c < cend && e == cudaSuccess; c += kGridY * NC) {
+    cfg.gridDim.y = std::min(kGridY, (cend - c + NC - 1) / NC);
     e = cudaLaunchKernelEx(&cfg, k_down_gint<T, CG, NC, CL>, X, xp, gpar, rows, n_ext, n_int, nrhs, cs, c, gint);
   }
   return e;
@@ -565,39 +566,54 @@ cudaError_t launch_down_gint_nc(const T* X, const T* xp, const T* gpar, int64_t 
 
 template <typename T, int CG, bool CL>
 cudaError_t launch_down_gint_cg(const T* X, const T* xp, const T* gpar, int64_t rows, int n_ext, int n_int, int nrhs,
-                                int cs, T* gint, int nc, cudaStream_t st) {
+                                int cfirst, int cend, int cs, T* gint, int nc, cudaStream_t st) {
   switch (nc) {
-    case 1: return launch_down_gint_nc<T, CG, 1, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
-    case 2: return launch_down_gint_nc<T, CG, 2, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
-    case 3: return launch_down_gint_nc<T, CG, 3, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
-    default: return launch_down_gint_nc<T, CG, 4, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cs, gint, st);
+    case 1: return launch_down_gint_nc<T, CG, 1, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cfirst, cend, cs, gint, st);
+    case 2: return launch_down_gint_nc<T, CG, 2, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cfirst, cend, cs, gint, st);
+    case 3: return launch_down_gint_nc<T, CG, 3, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cfirst, cend, cs, gint, st);
+    default: return launch_down_gint_nc<T, CG, 4, CL>(X, xp, gpar, rows, n_ext, n_int, nrhs, cfirst, cend, cs, gint, st);
   }
+}
+
+// right-hand sides per thread for `cols` of them
+inline int down_cols(int64_t tiles, int cols) {
+  // fewer where the row tiles would not go round the SMs two and a half times (112
+  // tiles, eight right-hand sides, real: 182 us in groups of four, 105 one by one; 224
+  // tiles: 96 in groups of four, 115 of three)
+  int most = 4;
+  while (most > 1 && 2 * tiles * ((cols + most - 1) / most) < 5 * device_sms()) --most;
+  return rhs_group(cols, most);
 }
 
 template <typename T>
 cudaError_t launch_down_gint(const T* X, const T* xp, const T* gpar, int nmerge, int n_ext, int n_int, int nrhs,
                              T* gint, cudaStream_t st) {
   const int64_t rows = (int64_t)nmerge * n_int, tiles = (rows + 31) / 32;
-  // fewer right-hand sides per thread where the row tiles would not go round the
-  // SMs two and a half times (112 tiles, eight right-hand sides, real: 182 us in
-  // groups of four, 105 one by one; 224 tiles: 96 in groups of four, 115 of three)
-  int most = 4;
-  while (most > 1 && 2 * tiles * ((nrhs + most - 1) / most) < 5 * device_sms()) --most;
-  int nc = rhs_group(nrhs, most);
+  auto range = [&](int c0, int c1, int nc) {
+    const int64_t warps = tiles * ((c1 - c0 + nc - 1) / nc);
+    const bool cluster = warps < 2 * device_sms() && n_ext < 8192;
+    const int cg = down_groups(warps, n_ext, cluster ? 32 : 16);
+    if (cg == 1) return launch_down_gint_cg<T, 1, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, 1, gint, nc, st);
+    if (cg == 2) return launch_down_gint_cg<T, 2, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, 1, gint, nc, st);
+    if (cg == 4) return launch_down_gint_cg<T, 4, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, 1, gint, nc, st);
+    if (cluster) return launch_down_gint_cg<T, 4, true>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, cg / 4, gint, nc, st);
+    if (cg == 8) return launch_down_gint_cg<T, 8, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, 1, gint, nc, st);
+    return launch_down_gint_cg<T, 16, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, c0, c1, 1, gint, nc, st);
+  };
+  const int nc = down_cols(tiles, nrhs);
+  const bool cplx_rows = sizeof(T) == 16, even = nrhs % nc == 0;
   // While L2 keeps X (up to half of it) groups save no memory traffic.  Complex
   // rows are then bound by the pipe anyway and finish sooner one by one (128 tiles
   // of 256 columns, eight right-hand sides: 68 us, in groups of three 90), real ones when
   // the last group would be short (192 tiles of 192, five: 18 us, in groups of three 29).
-  if (rows * n_ext * (int64_t)sizeof(T) < kDownL2 && (sizeof(T) == 16 || nrhs % nc != 0)) nc = 1;
-  const int64_t warps = tiles * ((nrhs + nc - 1) / nc);
-  const bool cluster = warps < 2 * device_sms() && n_ext < 8192;
-  const int cg = down_groups(warps, n_ext, cluster ? 32 : 16);
-  if (cg == 1) return launch_down_gint_cg<T, 1, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
-  if (cg == 2) return launch_down_gint_cg<T, 2, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
-  if (cg == 4) return launch_down_gint_cg<T, 4, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
-  if (cluster) return launch_down_gint_cg<T, 4, true>(X, xp, gpar, rows, n_ext, n_int, nrhs, cg / 4, gint, nc, st);
-  if (cg == 8) return launch_down_gint_cg<T, 8, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
-  return launch_down_gint_cg<T, 16, false>(X, xp, gpar, rows, n_ext, n_int, nrhs, 1, gint, nc, st);
+  if (rows * n_ext * (int64_t)sizeof(T) < kDownL2) return range(0, nrhs, cplx_rows || !even ? 1 : nc);
+  // Beyond, a short last group of complex rows costs a full one's work: the
+  // columns left over by fours go in a launch of their own (205 MB, five right-hand
+  // sides, all six levels of 4096 leaves: 3.13 ms in groups of three, 2.71 as four and one).
+  if (!cplx_rows || even || nrhs <= 4) return range(0, nrhs, nc);
+  const int whole = nrhs / 4 * 4, wide = down_cols(tiles, whole);
+  const cudaError_t e = range(0, whole, wide == 3 ? 2 : wide);
+  return e != cudaSuccess || whole == nrhs ? e : range(whole, nrhs, down_cols(tiles, nrhs - whole));
 }
 
 template <typename T>

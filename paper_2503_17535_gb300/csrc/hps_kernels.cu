@@ -463,7 +463,7 @@ cudaError_t merge_gather_h(const T* hc, int nmerge, int nch, int nbc, int n_ext,
 // very long rows, the ranges cost locality: 432 real tiles 94 -> 137, 216 of
 // 13824 columns 246 -> 265).  With one warp per 32 rows up to 255 columns, as
 // before, 64 real merges of 176 columns took 80 us, now 12.
-constexpr int64_t kDownL2 = 64 << 20;   // bytes of X that stay in L2 between groups
+constexpr int64_t kDownL2 = 116 << 20;   // bytes of X that stay in L2 (129 MB) between groups
 constexpr int kGridY = 65535;   // groups of right-hand sides in one launch (grid limit)
 template <typename T, int CG, int NC, bool CL>
 __global__ void __launch_bounds__(32 * (CG < 4 ? 4 : CG)) k_down_gint(const T* X, const T* xp, const T* gpar,
@@ -602,7 +602,7 @@ cudaError_t launch_down_gint(const T* X, const T* xp, const T* gpar, int nmerge,
   };
   const int nc = down_cols(tiles, nrhs);
   const bool cplx_rows = sizeof(T) == 16, even = nrhs % nc == 0;
-  // While L2 keeps X (up to half of it) groups save no memory traffic.  Complex
+  // While L2 keeps X groups save no memory traffic.  Complex
   // rows are then bound by the pipe anyway and finish sooner one by one (128 tiles
   // of 256 columns, eight right-hand sides: 68 us, in groups of three 90), real ones when
   // the last group would be short (192 tiles of 192, five: 18 us, in groups of three 29).
@@ -672,31 +672,32 @@ cudaError_t down_children(const T* gpar, const T* gint, int nmerge, int nch, int
   return cudaGetLastError();
 }
 
-// The row of the leaf's solution map that a node takes: of Y for ItI, of -Y at
-// interior and of P at boundary nodes for DtN.  For real data the two are one
-// pointer and stride, so that a warp with nodes of both kinds (every warp of a 2D
-// leaf) walks one loop.
+// The row of the leaf's solution map that a node takes: of Y for ItI (complex
+// data), of -Y at interior and of P at boundary nodes for DtN (real data), whose
+// two are one pointer and stride, so that a warp with nodes of both kinds (every
+// warp of a 2D leaf) walks one loop.
 template <typename T>
 struct LeafRow {
-  const double* p;   // real rows: entry j at p[j ld]
-  const T* x;        // complex rows
+  const T* p;   // entry j at p[j ld]
   int64_t ld;
-  int r;             // row of Y
+  int r;        // row of Y
   bool edge, negate;
-  __device__ LeafRow(const LeafConsts& k, bool iti, int node, const T* Xl, int xrows) {
-    const int pr = iti ? -1 : k.prow[node];
-    edge = pr >= 0;
-    negate = !iti && !edge;
-    r = iti ? node : edge ? 0 : k.iidx[node];
-    ld = edge ? k.ne : xrows;
-    x = Xl + r;
-    if constexpr (sizeof(T) == sizeof(double)) p = edge ? k.P + pr : Xl + r;
-    else p = k.P + pr;
+  __device__ LeafRow(const LeafConsts& k, int node, const T* Xl, int xrows) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+      const int pr = k.prow[node];
+      edge = pr >= 0;
+      negate = !edge;
+      r = edge ? 0 : k.iidx[node];
+      ld = edge ? k.ne : xrows;
+      p = edge ? k.P + pr : Xl + r;
+    } else {
+      edge = negate = false;
+      r = node;
+      ld = xrows;
+      p = Xl + r;
+    }
   }
-  __device__ T at(int j) const {
-    if constexpr (sizeof(T) == sizeof(double)) return p[j * ld];
-    else return edge ? T(p[j * ld]) : x[j * ld];
-  }
+  __device__ T at(int j) const { return p[j * ld]; }
 };
 
 // u = Y g + v at a leaf's nodes, a thread per node and NC right-hand sides, so
@@ -721,7 +722,7 @@ __global__ void __launch_bounds__(256) k_leaf_output(LeafConsts k, int64_t nl, i
     T acc[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) go[c] = min(c, nrhs - 1 - c0) * k.nb;
-    const LeafRow<T> row(k, iti, node, Xl, xrows);
+    const LeafRow<T> row(k, node, Xl, xrows);
 #pragma unroll
     for (int c = 0; c < NC; ++c)
       acc[c] = row.edge ? T(0.0)
@@ -889,7 +890,7 @@ __global__ void k_leaf_output_group(LeafGroup<T> grp) {
     const int xrows = grp.iti ? k.npts : k.ni;
     const T* gl = tk.g + (leaf * tk.nrhs + c) * (int64_t)k.nb;
     const T* Xl = tk.X + leaf * (int64_t)xrows * (k.nb + 1);
-    const LeafRow<T> row(k, grp.iti, node, Xl, xrows);
+    const LeafRow<T> row(k, node, Xl, xrows);
     T acc = row.edge ? T(0.0) : Xl[row.r + (int64_t)k.nb * xrows];
 #pragma unroll 4
     for (int j = 0; j < k.nb; ++j) acc = fmac(acc, row.at(j), gl[j]);

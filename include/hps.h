@@ -406,8 +406,9 @@ int64_t hps_debug_alloc_count(void);
 /* Bounded-wait check for tests (no counterpart in the paper).  Every wait
  * inside the library's kernels -- the inter-CTA barrier of the cooperative
  * panel LU (which = 0), the flag wait of the flag-ordered triangular solves
- * of a lazy root (which = 1) and the mbarrier wait of the tensor-core product
- * pipeline (which = 2) -- gives up after a bounded number of polls, records
+ * of a lazy root (which = 1) and the mbarrier waits of the tensor-core product
+ * pipeline and of the panel LU's cluster exchange (which = 2, one after the
+ * other; HPS_ERR_CUDA if they end differently) -- gives up after a bounded number of polls, records
  * a timeout in a device status word and lets its kernel end, so that a wait
  * that can never be satisfied costs an error status, not a hung GPU.  This
  * call runs the chosen wait in a one-CTA kernel on a word that nothing else

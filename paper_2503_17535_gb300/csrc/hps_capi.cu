@@ -1371,21 +1371,23 @@ hps_status hps_solve_adjoint(hps_handle* h, int nrhs, const void* ubar, void* gb
 hps_status hps_debug_wait_timeout(int which, int satisfied, int64_t limit_polls, struct CUstream_st* stream) {
   if (which < 0 || which > 2 || limit_polls < 1 || limit_polls > ((int64_t)1 << 24)) return HPS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned* d = nullptr;  // words[0..2] waited on, words[3] the status word
+  unsigned* d = nullptr;  // words[0..2] waited on (which 2: words[2] the panel wait's status), words[3] the status word
   HPS_CUDA(cudaMalloc(&d, 4 * sizeof(unsigned)));
   cudaError_t e = cudaMemsetAsync(d, 0, 4 * sizeof(unsigned), st);
   if (e == cudaSuccess)
     e = which == 2 ? hps::debug_mbar_wait(satisfied ? 1 : 0, (long)limit_polls, d + 3, st)
                    : hps::debug_wait(which, satisfied ? 1 : 0, d, (unsigned long long)limit_polls, d + 3, st);
-  unsigned herr = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, d + 3, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && which == 2) e = hps::debug_panel_wait(satisfied ? 1 : 0, (long)limit_polls, d + 2, st);
+  unsigned herr[2] = {0, 0};   // words[2], words[3]
+  if (e == cudaSuccess) e = cudaMemcpyAsync(herr, d + 2, sizeof(herr), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(d);
-  if (e != cudaSuccess) {
+  // of two waits both have to come to the same end
+  if (e != cudaSuccess || (which == 2 && herr[0] != herr[1])) {
     cudaGetLastError();
     return HPS_ERR_CUDA;
   }
-  return (herr & hps::DEV_ERR_TIMEOUT) ? HPS_ERR_TIMEOUT : HPS_OK;
+  return (herr[1] & hps::DEV_ERR_TIMEOUT) ? HPS_ERR_TIMEOUT : HPS_OK;
 }
 
 hps_status hps_tune_set(int param, int value) {

@@ -1050,8 +1050,8 @@ __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 // bounded wait for a phase whose bytes come from the cluster's CTAs
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, int parity) {
-  for (int it = 0; it < (1 << 22); ++it) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, int parity, long limit = 1L << 22) {
+  for (long it = 0; it < limit; ++it) {
     uint32_t ok;
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                  : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
@@ -2474,6 +2474,27 @@ __global__ void k_debug_wait(int which, int satisfied, unsigned* words, unsigned
 cudaError_t debug_wait(int which, int satisfied, unsigned* words, unsigned long long limit, unsigned* err,
                        cudaStream_t st) {
   k_debug_wait<<<1, 128, 0, st>>>(which, satisfied, words, limit, err);
+  return cudaGetLastError();
+}
+
+
+// The panel LU's wait on an mbarrier (hps_debug_wait_timeout, which 2), as
+// debug_mbar_wait does with the product pipeline's.
+__global__ void k_debug_panel_wait(int satisfied, long limit, unsigned* err) {
+  __shared__ __align__(8) uint64_t bar;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (satisfied) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&bar)) : "memory");
+    if (!mbar_wait_cluster(&bar, 0, limit)) atomicOr(err, DEV_ERR_TIMEOUT);
+  }
+}
+
+cudaError_t debug_panel_wait(int satisfied, long limit, unsigned* err, cudaStream_t st) {
+  k_debug_panel_wait<<<1, 32, 0, st>>>(satisfied, limit, err);
   return cudaGetLastError();
 }
 

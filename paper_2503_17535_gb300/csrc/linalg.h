@@ -105,10 +105,12 @@ cudaError_t gemm(const GemmArgs<T>& g, cudaStream_t st, Prof* pf);
 // Bounded-wait checks (hps_debug_wait_timeout): one CTA runs one of the
 // library's bounded waits on a word nothing else writes (linalg.cu: the group
 // barrier, which 0, and the triangular solves' flag wait, which 1, on the
-// zeroed words[0..2]; gemm_tc.cu: the tensor-core pipeline's mbarrier wait).
+// zeroed words[0..2]; gemm_tc.cu: the tensor-core pipeline's mbarrier wait;
+// linalg.cu: that of the panel LU's cluster exchange).
 cudaError_t debug_wait(int which, int satisfied, unsigned* words, unsigned long long limit, unsigned* err,
                        cudaStream_t st);
 cudaError_t debug_mbar_wait(int satisfied, long limit, unsigned* err, cudaStream_t st);
+cudaError_t debug_panel_wait(int satisfied, long limit, unsigned* err, cudaStream_t st);
 
 // Tensor-core FP64 products (gemm_tc.cu): workspace for the operands' fp16
 // digit slices.  gemm() routes a product to the tensor cores when the calling

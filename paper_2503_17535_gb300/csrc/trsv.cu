@@ -375,13 +375,14 @@ size_t cluster_smem(int nr, int mo) {
 // 96 4.2 / 7.0 (the blocks of all merges of the elliptic and Helmholtz operators), 512
 // to 4096 6.9 / 217, above 4.0 / 46 (dense impedance leaves).  Solutions of the former
 // have the same errors with and without the correction; the line lies between.
-constexpr double CORRECT_FROM = 256.0;
+constexpr float CORRECT_FROM = 256.0f;
+__device__ __forceinline__ float magf(double v) { return fabsf((float)v); }
+__device__ __forceinline__ float magf(cplx v) { return fabsf((float)v.re) + fabsf((float)v.im); }
 template <typename T>
 __global__ void __launch_bounds__(128) k_block_inverses(BOp<T> LU, int n, T* out) {
   __shared__ T Ls[32 * 32];
   __shared__ T dv[32];
-  __shared__ double mv[32 * 33];   // magnitudes of the inverse
-  __shared__ int wants[2];
+  __shared__ float mv[32 * 33], rsum[32], csum[32];   // magnitudes of the inverse, their row and column sums
   const int j = blockIdx.x, nblk = gridDim.x, b = blockIdx.z;
   const bool upper = blockIdx.y == 1;
   const int pb = min(32, n - j * 32);
@@ -431,28 +432,40 @@ __global__ void __launch_bounds__(128) k_block_inverses(BOp<T> LU, int n, T* out
   }
   const int64_t at = ((int64_t)b * 2 + blockIdx.y) * nblk + j;
   T* o = out + at * 1024 + 32 * col + 8 * g;
+  // |T| (|V| 1) and (1 |V|) |T|, four threads per row or column; in single
+  // precision, off the FP64 pipe: what overflows or is no number is marked
+  auto quad = [](float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+  };
+  float sum = 0.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     o[i] = x[i];
-    mv[(8 * g + i) * 33 + col] = mag1(x[i]);
+    const float m = magf(x[i]);
+    mv[(8 * g + i) * 33 + col] = m;
+    sum += m;
   }
+  csum[col] = quad(sum);
   __syncthreads();
-  if (threadIdx.x < 64) {
-    // |T| (|V| 1), a row per lane (warp 0), or (1 |V|) |T|, a column per lane (warp 1)
-    const int lane = threadIdx.x & 31;
-    const bool rows = threadIdx.x < 32;
-    double sum = 0.0, norm = 0.0;
-    for (int k = 0; k < 32; ++k) sum += rows ? mv[lane * 33 + k] : mv[k * 33 + lane];
-    for (int k = 0; k < 32; ++k) {
-      const int r = rows ? lane : k, c = rows ? k : lane;
-      const double t = r == c && !upper ? 1.0 : (upper ? r <= c : r >= c) ? mag1(Ls[r + c * 32]) : 0.0;
-      norm = fma(t, __shfl_sync(0xffffffffu, sum, k), norm);
-    }
-    const bool over = __any_sync(0xffffffffu, !(norm <= CORRECT_FROM));
-    if (lane == 0) wants[rows ? 0 : 1] = over;
+  const int r = col, k0 = 8 * g;   // this thread's row or column of T, and the entries it takes
+  sum = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) sum += mv[r * 33 + k0 + k];
+  rsum[r] = quad(sum);
+  __syncthreads();
+  float rn = 0.0f, cn = 0.0f;
+#pragma unroll
+  for (int k = k0; k < k0 + 8; ++k) {
+    const float tr = upper ? (k >= r ? magf(Ls[r + k * 32]) : 0.0f) : k < r ? magf(Ls[r + k * 32]) : k == r ? 1.0f : 0.0f;
+    const float tc = upper ? (k <= r ? magf(Ls[k + r * 32]) : 0.0f) : k > r ? magf(Ls[k + r * 32]) : k == r ? 1.0f : 0.0f;
+    rn = fmaf(tr, rsum[k], rn);
+    cn = fmaf(tc, csum[k], cn);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) out[(int64_t)gridDim.z * 2 * nblk * 1024 + at] = T(wants[0] || wants[1] ? 1.0 : 0.0);
+  rn = quad(rn);
+  cn = quad(cn);
+  const int wants = __syncthreads_or(!(rn <= CORRECT_FROM) || !(cn <= CORRECT_FROM));
+  if (threadIdx.x == 0) out[(int64_t)gridDim.z * 2 * nblk * 1024 + at] = T(wants ? 1.0 : 0.0);
 }
 
 // Cluster shape: a power of two of CTAs, at most 16, the SMs' share of a

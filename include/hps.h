@@ -42,14 +42,17 @@
  * streams are ordered on the device: each call's stream first waits for the
  * handle's previous work (an event the handle records), so they never
  * overlap on the handle's buffers (not while the caller captures the stream
- * into a graph, where the caller's graph orders the work).  A handle must
- * not be used from two host threads at the same time.
+ * into a graph, where the caller's graph orders the work; a solve recorded
+ * there needs device buffers and the workspace of an earlier solve with at
+ * least as many right-hand sides, on an adaptive tree as many).  A handle
+ * must not be used from two host threads at the same time.
  *
  * Device memory of handles and their workspaces comes from a stream-ordered
  * pool per device (cudaMallocFromPoolAsync / cudaFreeAsync): building,
  * growing a workspace or freeing a handle never waits for other streams.
  * The pool keeps up to a sixteenth of the device's memory after frees for the
- * next builds; hps_trim gives it back.
+ * next builds (other allocations of the process get it when memory runs short,
+ * other processes do not); hps_trim gives it back.
  *
  * Errors: every call returns an hps_status; nothing is thrown across the ABI.
  * On failure *out handles are set to NULL and no memory is leaked.
